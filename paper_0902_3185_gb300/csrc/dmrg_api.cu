@@ -539,7 +539,7 @@ void lz_alloc(dmrg_sb* sb, int cap) {
   sb->lz_ab = dalloc<double>((size_t)(2 * B * cap));
   sb->lz_s = dalloc<double>((size_t)(B * cap));
   sb->lz_out = dalloc<double>((size_t)(4 * B + 1));
-  sb->lz_ctl = dalloc<int32_t>((size_t)(LZ_CTL_MEMBER + 2 * B));
+  sb->lz_ctl = dalloc<int32_t>((size_t)lz_ctl_words(B));
   void* hp = nullptr;
   CK(cudaMallocHost(&hp, sizeof(int32_t) * (LZ_CTL_MEMBER + 2 * B)));
   sb->h_ctl = static_cast<int32_t*>(hp);
@@ -589,10 +589,9 @@ void lz_enqueue_iteration(dmrg_sb* sb, int prec, cudaStream_t st) {
   lz_launch_multidot(sb->lz_V, sb->lz_w, sb->lz_partial, ctl, D, B, cap, 0, sb->lz_gate, st, nullptr, nullptr, pair);
   lz_launch_reduce_rows(sb->lz_partial, hC, ctl, lz_dot_nparts(D), cap, B, 0, sb->lz_gate, st);
   lz_launch_multiaxpy(sb->lz_V, sb->lz_w, hC, nC, ctl, D, B, cap, nch, 0, sb->lz_gate, st, pair);
-  lz_launch_finalize_ab(sb->lz_h, nB, nC, sb->lz_gate, sb->lz_ab, ctl, B, cap, nch, st);
-  lz_launch_tridiag(sb->lz_ab, sb->lz_s, sb->lz_out, ctl, sb->lz_out + 4 * B, B, cap, D, st);  // tol at out[4B]
+  lz_launch_tridiag(sb->lz_h, nB, nC, sb->lz_gate, nch, sb->lz_ab, sb->lz_s, sb->lz_out, ctl, sb->lz_out + 4 * B, B,
+                    cap, D, st);  // tol at out[4B]
   lz_launch_next_vector(sb->lz_w, sb->lz_ab, sb->lz_V, sb->lz_vcur, ctl, D, B, cap, st, pair);
-  lz_launch_advance(ctl, B, st);
   CK(cudaGetLastError());
 }
 
@@ -640,7 +639,7 @@ int matvec_launches(const dmrg_sb* sb, int prec) {
     return (sb->f64_fwd1.n_tiles > 0) + (sb->f64_fwd2.n_tiles > 0) + (sb->f64_fwd3.n_tiles > 0);
   return tc_launches(sb, prec);
 }
-constexpr int LZ_KERNELS_PER_ITER = 13;  // everything in lz_enqueue_iteration besides the product
+constexpr int LZ_KERNELS_PER_ITER = 11;  // everything in lz_enqueue_iteration besides the product
 
 // One Lanczos run from psi0 (device [batch][D]) to psi_out for the members
 // whose initial control code is LZ_RUNNING (the others are LZ_HOLD: skipped,
@@ -657,7 +656,7 @@ LzRun lz_run(dmrg_sb* sb, const double* psi0, double* psi_out, int prec, double 
   lz_launch_sumsq(psi0, part, D, B, nch, st);
   lz_launch_sum_chunks(part, nrm2, nch, B, st);
   lz_launch_scale_unit(psi0, nrm2, sb->lz_V, sb->lz_vcur, D, B, st, lz_pair(prec));
-  std::vector<int32_t> hc(LZ_CTL_MEMBER + 2 * B, 0);
+  std::vector<int32_t> hc(lz_ctl_words(B), 0);
   hc[LZ_CTL_MAXIT] = max_iter;
   hc[LZ_CTL_CHECK] = std::max(1, check_every);
   hc[LZ_CTL_FORCE] = force;
@@ -677,7 +676,8 @@ LzRun lz_run(dmrg_sb* sb, const double* psi0, double* psi_out, int prec, double 
     if (launched > max_iter + K) throw Invalid{"Lanczos control did not terminate"};
   }
   // float64 eigenpairs of the members that stopped on the float32 test, side by side
-  lz_launch_tridiag(sb->lz_ab, sb->lz_s, sb->lz_out, sb->lz_ctl, sb->lz_out + 4 * B, B, cap, D, st, 1);
+  lz_launch_tridiag(nullptr, nullptr, nullptr, nullptr, 0, sb->lz_ab, sb->lz_s, sb->lz_out, sb->lz_ctl,
+                    sb->lz_out + 4 * B, B, cap, D, st, 1);
   CK(cudaMemcpyAsync(sb->h_ctl, sb->lz_ctl, sizeof(int32_t) * (LZ_CTL_MEMBER + 2 * B), cudaMemcpyDeviceToHost, st));
   lz_launch_ritz(sb->lz_V, sb->lz_s, sb->lz_ctl, psi_out, D, B, cap, st, lz_pair(prec));
   lz_launch_sumsq(psi_out, part, D, B, nch, st);
@@ -1438,7 +1438,7 @@ dmrg_status dmrg_time_reorth(dmrg_sb* sb, int32_t prec, int32_t j, int32_t reps,
     const bool pair = lz_pair(prec);
     // every member running at Krylov index j; the basis rows and w hold whatever
     // the last solve left (the timing does not depend on the values)
-    std::vector<int32_t> hc(LZ_CTL_MEMBER + 2 * B, 0);
+    std::vector<int32_t> hc(lz_ctl_words(B), 0);
     hc[LZ_CTL_J] = j;
     hc[LZ_CTL_MAXIT] = cap;
     hc[LZ_CTL_CHECK] = 1;

@@ -30,7 +30,8 @@
 // 5 pending: stopped on the float32 test, float64 check after the loop;
 // 6 resume: that check failed with iterations left, the host restarts the
 // member from its Ritz vector; 7 hold: done in an earlier run, skipped)
-// and [5 + batch + b] number of Lanczos vectors in its tridiagonal matrix.
+// and [5 + batch + b] number of Lanczos vectors in its tridiagonal matrix;
+// last, [5 + 2 batch] counts the blocks of k_tridiag that have finished.
 
 #include <cfloat>
 
@@ -415,25 +416,6 @@ __global__ void k_dgks(const double* __restrict__ npart_a, const double* __restr
   if (threadIdx.x == 0) gate[b] = (nb >= 0.5 * na) ? 0 : 1;  // NaN: run pass C, then the NaN check stops it
 }
 
-// alpha_j = sum of the v_j coefficients of the passes that ran, beta_j = |w|
-// after the last pass.  One warp per member (deterministic).
-__global__ void k_finalize_ab(const double* __restrict__ h, const double* __restrict__ npart_b,
-                              const double* __restrict__ npart_c, const int32_t* __restrict__ gate,
-                              double* __restrict__ ab, const int32_t* __restrict__ ctl, int batch, int cap,
-                              int nchunk) {
-  const int b = blockIdx.x;
-  if (member_done(ctl, b)) return;
-  const int j = ctl[LZ_CTL_J];
-  const bool c = gate[b] != 0;
-  const double t = warp_sum_chunks((c ? npart_c : npart_b) + (int64_t)b * nchunk, nchunk);
-  if (threadIdx.x == 0) {
-    double a = h[(int64_t)b * cap + j] + h[((int64_t)batch + b) * cap + j];
-    if (c) a += h[(2 * (int64_t)batch + b) * cap + j];
-    ab[(int64_t)b * cap + j] = a;
-    ab[((int64_t)batch + b) * cap + j] = sqrt(t);
-  }
-}
-
 // Sign and zero test of a float / double from its bit pattern (integer
 // instructions: GB300's float64 pipe is narrow), and its biased exponent.
 __device__ __forceinline__ bool is_neg(float v) { return __float_as_int(v) < 0; }
@@ -467,18 +449,20 @@ __device__ __forceinline__ double sturm_scale(double scale) {
 // of a_i - x or e2_{i-1}, as in the pivot form.  When the larger of the last
 // two minors leaves the exponent window both are scaled by the same power of
 // two (exact); a zero minor takes its predecessor's sign, which puts the
-// sign change on the next minor.
+// sign change on the next minor.  as, es: the scaled entries s a_i and
+// s^2 e2_i (s a power of two: exact, and three float64 instructions a step
+// instead of five); x is scaled here.
 template <class T>
-__device__ int sturm_count(const T* a, const T* e2, int n, T x, T s) {
+__device__ int sturm_count(const T* as, const T* es, int n, T x, T s) {
   constexpr int bias = SturmWindow<T>::bias, W = SturmWindow<T>::W;
-  const T s2 = s * s;
+  x *= s;
   T pm = T(1);
-  T p = (a[0] - x) * s;
+  T p = as[0] - x;
   bool neg = is_neg(p) && !is_zero(p);
   int cnt = neg ? 1 : 0;
   for (int i = 1; i < n; ++i) {
-    const T t = (a[i] - x) * s;
-    const T q = (e2[i - 1] * s2) * pm;
+    const T t = as[i] - x;
+    const T q = es[i - 1] * pm;
     const T pn = fma(t, p, -q);
     const bool nn = is_zero(pn) ? neg : is_neg(pn);
     cnt += nn != neg;
@@ -499,14 +483,14 @@ __device__ int sturm_count(const T* a, const T* e2, int n, T x, T s) {
 // spaced points of [lo, hi] (count(lo) = 0 <= 1 <= count(hi) ... holds for
 // the lowest eigenvalue) and keep the sub-interval that holds it.
 template <class T>
-__device__ void multisection(const T* a, const T* e2, int n, T& lo, T& hi, T rel, int max_rounds, T s) {
+__device__ void multisection(const T* as, const T* es, int n, T& lo, T& hi, T rel, int max_rounds, T s) {
   const int lane = threadIdx.x & 31;
   for (int round = 0; round < max_rounds; ++round) {
     const T w = hi - lo;
     if (!(w > rel * fmax(fabs(lo), fabs(hi))) || !(w > T(0))) break;
     const T step = w / T(33);
     const T x = lo + step * T(lane + 1);
-    const int cnt = sturm_count<T>(a, e2, n, x, s);
+    const int cnt = sturm_count<T>(as, es, n, x, s);
     const unsigned ball = __ballot_sync(0xffffffffu, cnt >= 1);
     const int f = ball ? __ffs(ball) - 1 : 32;  // first point with an eigenvalue below it
     const T nlo = lo + step * T(f);
@@ -556,31 +540,138 @@ __device__ void inverse_iteration(const T* a, const T* e, int n, T sigma, T* z, 
   }
 }
 
-// Lowest eigenpair of the (j+1) x (j+1) tridiagonal matrix of each member and
-// the convergence test.  One warp per member.
-//  - every check: float32 multisection and float32 inverse iteration give
-//    theta and the last Ritz-vector component to a few digits, enough for the
-//    test beta_j |s_j| <= tol max(1, |theta|);
-//  - when the float32 test passes with a factor 2 to spare, the member stops
-//    as LZ_PENDING; after the iteration loop one launch (final_pass) redoes
-//    the float32 step for every pending member at its own length, computes
-//    the eigenpair in float64 (multisection from the float32 bracket, widened
-//    by its rounding bound, then inverse iteration), repeats the test with
-//    the float64 values (a member that then misses the tolerance ends as
-//    LZ_RESUME, or LZ_CAP at max_iter; the host restarts a resumed member from
-//    its Ritz vector) and stores s for the Ritz vector: the members' float64 solves
-//    run side by side in one launch instead of each in the launch where its
-//    member converged;
-//  - at breakdown or the cap the float64 eigenpair is computed at once;
-//  - tolerances below 1e-5 are beyond the float32 estimate's resolution:
-//    near convergence (estimate <= 1e-2 |T|) those members take the float64
-//    eigenpair and test at every check instead of stopping as pending.
-// GB300 issues float64 at 1/64 of the float32 rate, which is why the per-
-// iteration test runs in float32.
-__global__ void __launch_bounds__(32)
-k_tridiag(const double* __restrict__ ab, double* __restrict__ s_out, double* __restrict__ out,
-          int32_t* __restrict__ ctl, const double* __restrict__ tolp, int batch, int cap, int64_t D,
-          int final_pass) {
+// Whether any eigenvalue lies below x / s, in float32 (the smallest eigenvalue
+// needs no count beyond the first sign change): the same minors, te[i] =
+// (s a_i, s^2 e2_{i-1}), rescaled every four steps only: a step grows a minor
+// by less than 4, and from a larger minor near 1 four steps stay far above
+// the smallest float as long as no s^2 e2 is below 2^-30 twice running
+// (breakdown stops a member at beta < 1e-14 |T| before that).  It steers the
+// estimate only; the deciding test counts as above.
+__device__ __forceinline__ bool sturm_below(const float2* te, int n, float x) {
+  float pm = 1.0f;
+  float p = te[0].x - x;
+  int neg = __float_as_int(p) & (p != 0.0f ? -1 : 0);  // the sign bit collects the signs of all minors
+  int i = 1;
+  for (; i + 3 < n; i += 4) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const float2 v = te[i + u];
+      const float pn = fmaf(v.x - x, p, -(v.y * pm));
+      pm = p;
+      p = pn;
+      neg |= __float_as_int(p) & (p != 0.0f ? -1 : 0);
+    }
+    const float f = pow2_to_one(min(max(bexp(p), bexp(pm)), 253), 0.0f);
+    p *= f;
+    pm *= f;
+  }
+  for (; i < n; ++i) {
+    const float2 v = te[i];
+    const float pn = fmaf(v.x - x, p, -(v.y * pm));
+    pm = p;
+    p = pn;
+    neg |= __float_as_int(p) & (p != 0.0f ? -1 : 0);
+  }
+  return neg < 0;
+}
+
+// float sum and maximum over the block, the same in every thread
+__device__ __forceinline__ float tri_block_sum(float v, float* red) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  float t = 0.0f;
+#pragma unroll
+  for (int w = 0; w < LZ_TRI / 32; ++w) t += red[w];
+  return t;
+}
+template <bool MIN>
+__device__ __forceinline__ float tri_block_ext(float v, float* red) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float u = __shfl_xor_sync(0xffffffffu, v, o);
+    v = MIN ? fminf(v, u) : fmaxf(v, u);
+  }
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  float t = red[0];
+#pragma unroll
+  for (int w = 1; w < LZ_TRI / 32; ++w) t = MIN ? fminf(t, red[w]) : fmaxf(t, red[w]);
+  return t;
+}
+
+// Inclusive product scan of r[0..n-1] in place by one warp (forward: from
+// r[0] up; backward: from r[n-1] down): lane-contiguous chunks, their
+// products scanned by shuffles, then multiplied through.
+__device__ __forceinline__ void warp_product_scan(float* r, int n, bool backward) {
+  const int lane = threadIdx.x & 31;
+  const int m = (n + 31) / 32;
+  const int b = min(n, lane * m), e = min(n, b + m);
+  auto at = [&](int i) -> float& { return r[backward ? n - 1 - i : i]; };
+  float t = 1.0f;
+  for (int i = b; i < e; ++i) {
+    t *= at(i);
+    at(i) = t;
+  }
+  float pre = t;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const float u = __shfl_up_sync(0xffffffffu, pre, o);
+    if (lane >= o) pre *= u;
+  }
+  const float before = __shfl_up_sync(0xffffffffu, pre, 1);
+  if (lane > 0)
+    for (int i = b; i < e; ++i) at(i) *= before;
+}
+
+// The end of a Lanczos step, one block per member:
+//  - alpha_j = the sum of the v_j coefficients of the passes that ran, beta_j
+//    = |w| after the last pass (not in the final pass);
+//  - the lowest eigenpair of the (j+1) x (j+1) tridiagonal matrix and the
+//    convergence test;
+//  - the last block to finish advances the iteration (not in the final pass).
+// The test has two stages.
+//  Estimate, every check, float32: multisection by the whole block (LZ_TRI + 1
+//  sub-intervals a round: three rounds from the Gershgorin interval to float32
+//  resolution) gives theta; the eigenvector comes from the twisted
+//  factorisation of T - sigma I, sigma just below theta: pivots from the top
+//  and from the bottom (two warps, a chain of reciprocals each), joined at the
+//  index of the smallest twist pivot, where the eigenvector is largest; its
+//  entries are products of ratios e / pivot on either side.  All pivots are
+//  positive, so every ratio, and with them the last component, keeps its
+//  relative accuracy however small it is, and beta_j |s_j| resolves every
+//  tolerance.  (An inverse iteration's last component is good to eps |T| / gap
+//  in absolute terms only: tolerances below 1e-5 had needed the float64
+//  eigenpair at every check from 1e-2 |T| on.)
+//  Decision, by one warp:
+//  - tol >= 1e-5, once the estimate is within a factor 2 of the value that
+//    stops the member (half the tolerance): float32 multisection and inverse
+//    iteration; when they pass, the member stops as LZ_PENDING; after the
+//    iteration loop one launch (final_pass) computes the eigenpair of every
+//    pending member at its own length in float64 (multisection from the
+//    float32 bracket, widened by its rounding bound, then one solve from the
+//    float32 vector), repeats the test with the float64 values (a member that
+//    then misses the tolerance ends as LZ_RESUME, or LZ_CAP at max_iter; the
+//    host restarts a resumed member from its Ritz vector) and stores s for the
+//    Ritz vector: the members' float64 solves run side by side in one launch
+//    instead of each in the launch where its member converged;
+//  - tol < 1e-5: that float64 eigenpair and test as soon as the estimate is
+//    within a factor 8 of the tolerance;
+//  - a pivot that was not positive leaves no estimate: the warp decides;
+//  - at breakdown or the cap the float64 eigenpair is computed at once.
+// GB300 issues float64 at 1/64 of the float32 rate: a warp's instruction holds
+// its scheduler's pipe for 64 cycles, so one float64 eigenpair of n = 80 costs
+// about 200 us.  Float64 solve of the m = 200 Hubbard chain (80 steps, tol
+// 1e-12): 23.1 -> 15.1 ms (this kernel had been 123 us a step, plus 3.8 us for
+// two kernels it absorbed); Hubbard chain m = 160 DMRG run: 218 -> 22 us a step.
+__global__ void __launch_bounds__(LZ_TRI)
+k_tridiag(const double* __restrict__ h, const double* __restrict__ npart_b, const double* __restrict__ npart_c,
+          const int32_t* __restrict__ gate, int nchunk, double* __restrict__ ab, double* __restrict__ s_out,
+          double* __restrict__ out, int32_t* __restrict__ ctl, const double* __restrict__ tolp, int batch, int cap,
+          int64_t D, int final_pass) {
   extern __shared__ double sm[];
   double* a = sm;
   double* e = sm + cap;
@@ -592,24 +683,201 @@ k_tridiag(const double* __restrict__ ab, double* __restrict__ s_out, double* __r
   float* e232 = e32 + cap;
   float* z32 = e232 + cap;
   float* rp32 = z32 + cap;
+  // the estimate's arrays, in the decision's places
+  float2* te = reinterpret_cast<float2*>(z);
+  float* dpl = e232;
+  float* dmi = rp32;
+  __shared__ float red[LZ_TRI / 32];
+  __shared__ int first_pt, bad_piv;
+  __shared__ unsigned long long best;
   const int b = blockIdx.x;
-  const int lane = threadIdx.x;
-  if (final_pass ? ctl[LZ_CTL_MEMBER + b] != LZ_PENDING : member_done(ctl, b)) return;
-  const int n = final_pass ? ctl[LZ_CTL_MEMBER + batch + b] : ctl[LZ_CTL_J] + 1;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int j = ctl[LZ_CTL_J];
+  // every path of the test ends here: the last block advances the iteration
+  auto leave = [&]() {
+    if (final_pass || tid != 0) return;
+    __threadfence();
+    int32_t* ticket = ctl + LZ_CTL_MEMBER + 2 * batch;
+    if (atomicAdd(ticket, 1) != batch - 1) return;
+    *ticket = 0;
+    __threadfence();
+    volatile int32_t* vc = ctl;
+    if (vc[LZ_CTL_ALLDONE]) return;
+    int all = 1;
+    for (int q = 0; q < batch; ++q) all &= vc[LZ_CTL_MEMBER + q] != 0;
+    if (all) vc[LZ_CTL_ALLDONE] = 1;
+    else vc[LZ_CTL_J] = j + 1;
+  };
+  if (final_pass ? ctl[LZ_CTL_MEMBER + b] != LZ_PENDING : member_done(ctl, b)) {
+    leave();
+    return;
+  }
+  const int n = final_pass ? ctl[LZ_CTL_MEMBER + batch + b] : j + 1;
   const int max_iter = ctl[LZ_CTL_MAXIT];
   const int check_every = ctl[LZ_CTL_CHECK];
   const double tol = *tolp;
+  if (!final_pass && wid == 0) {  // alpha_j, beta_j
+    const bool c = gate[b] != 0;
+    const double t = warp_sum_chunks((c ? npart_c : npart_b) + (int64_t)b * nchunk, nchunk);
+    if (lane == 0) {
+      double aj = h[(int64_t)b * cap + j] + h[((int64_t)batch + b) * cap + j];
+      if (c) aj += h[(2 * (int64_t)batch + b) * cap + j];
+      const double bj = sqrt(t);
+      ab[(int64_t)b * cap + j] = aj;
+      ab[((int64_t)batch + b) * cap + j] = bj;
+      a[j] = aj;
+      e[j] = bj;
+    }
+  }
+  for (int i = tid; i < (final_pass ? n : j); i += LZ_TRI) {
+    a[i] = ab[(int64_t)b * cap + i];
+    e[i] = ab[((int64_t)batch + b) * cap + i];  // e[n-1] = beta_j, the residual factor
+  }
+  if (tid == 0) {
+    bad_piv = 0;
+    best = ~0ull;
+  }
+  __syncthreads();
+  const double beta = e[n - 1];
+  if (!isfinite(a[n - 1]) || !isfinite(beta)) {
+    if (tid == 0) {
+      ctl[LZ_CTL_MEMBER + b] = LZ_NAN;
+      ctl[LZ_CTL_MEMBER + batch + b] = n;
+    }
+    leave();
+    return;
+  }
+  const bool last = n >= max_iter || (int64_t)n >= D;
+  const bool force = ctl[LZ_CTL_FORCE] != 0;
+  if (!final_pass) {
+    // ---- estimate: Gershgorin bounds and the scale in float32
+    float glo = 3e38f, ghi = 3e38f, amax = 0.0f;
+    for (int i = tid; i < n; i += LZ_TRI) {
+      const float ai = tc::d2f_rn32(a[i]), el = i > 0 ? tc::d2f_rn32(e[i - 1]) : 0.0f;
+      const float rad = fabsf(el) + (i < n - 1 ? fabsf(tc::d2f_rn32(e[i])) : 0.0f);
+      a32[i] = ai;
+      e32[i] = el;  // the off-diagonal above row i
+      glo = fminf(glo, ai - rad);
+      ghi = fminf(ghi, ai);
+      amax = fmaxf(amax, fabsf(ai) + rad);
+    }
+    glo = tri_block_ext<true>(glo, red);
+    ghi = tri_block_ext<true>(ghi, red);
+    amax = tri_block_ext<false>(amax, red);
+    const float scale32 = fmaxf(1.0f, amax);
+    // near breakdown (twice the decision's bound, float32 rounding apart) the warp decides
+    const bool tiny_beta = beta < 2e-14 * (double)scale32;
+    if (!((n % check_every == 0) || last || tiny_beta)) {
+      leave();
+      return;
+    }
+    if (!last && !tiny_beta) {
+      const float eps32 = 1.2e-7f;
+      const float s32 = (float)sturm_scale((double)scale32);
+      const float slack = 16.0f * eps32 * scale32;  // rounding of T to float32, Sturm backward error
+      for (int i = tid; i < n; i += LZ_TRI) {
+        const float es = e32[i] * s32;
+        te[i] = make_float2(a32[i] * s32, es * es);
+      }
+      float lo = glo - slack, hi = ghi + slack;
+      for (int round = 0; round < 8; ++round) {
+        const float w = hi - lo;
+        if (!(w > 4.0f * eps32 * fmaxf(fabsf(lo), fabsf(hi))) || !(w > 0.0f)) break;
+        if (tid == 0) first_pt = LZ_TRI;
+        __syncthreads();
+        const float step = w / (float)(LZ_TRI + 1);
+        const bool below = sturm_below(te, n, (lo + step * (float)(tid + 1)) * s32);
+        const unsigned ball = __ballot_sync(0xffffffffu, below);
+        if (ball && lane == 0) atomicMin(&first_pt, (wid << 5) + __ffs(ball) - 1);
+        __syncthreads();
+        const int f = first_pt;  // first point with an eigenvalue below it
+        const float nlo = lo + step * (float)f;
+        hi = f < LZ_TRI ? lo + step * (float)(f + 1) : hi;
+        lo = nlo;
+        __syncthreads();
+      }
+      const float th32 = 0.5f * (lo + hi);
+      const float sg = (lo - slack) * s32;
+      // pivots of s (T - sigma I) from the top (warp 0) and from the bottom (warp 1)
+      __syncthreads();
+      if (lane == 0 && wid < 2) {
+        bool pos = true;
+        if (wid == 0) {
+          float d = te[0].x - sg;
+          dpl[0] = d;
+          pos = d > 0.0f;
+#pragma unroll 4
+          for (int i = 1; i < n; ++i) {
+            d = (te[i].x - sg) - __fdividef(te[i].y, d);
+            dpl[i] = d;
+            pos = pos && d > 0.0f;
+          }
+        } else {
+          float d = te[n - 1].x - sg;
+          dmi[n - 1] = d;
+          pos = d > 0.0f;
+#pragma unroll 4
+          for (int i = n - 2; i >= 0; --i) {
+            d = (te[i].x - sg) - __fdividef(te[i + 1].y, d);
+            dmi[i] = d;
+            pos = pos && d > 0.0f;
+          }
+        }
+        if (!pos) bad_piv = 1;
+      }
+      __syncthreads();
+      for (int i = tid; i < n; i += LZ_TRI) {
+        const float g = fabsf(dpl[i] + dmi[i] - (te[i].x - sg));
+        atomicMin(&best, ((unsigned long long)__float_as_uint(g) << 32) | (unsigned)i);
+      }
+      __syncthreads();
+      const int kt = (int)(best & 0xffffffffu);
+      const bool unsure = bad_piv != 0;
+      // z_i / z_{i-1} below the twist index, z_i / z_{i+1} above it, then the products
+      for (int i = tid; i < n; i += LZ_TRI) {
+        const float dn = i > kt ? -__fdividef(e32[i] * s32, dmi[i]) : 1.0f;
+        const float up = i < kt ? -__fdividef(e32[i + 1] * s32, dpl[i]) : 1.0f;
+        dmi[i] = dn;
+        dpl[i] = up;
+      }
+      __syncthreads();
+      if (wid == 0) warp_product_scan(dmi, n, false);
+      if (wid == 1) warp_product_scan(dpl, n, true);
+      __syncthreads();
+      float nz = 0.0f;
+      for (int i = tid; i < n; i += LZ_TRI) {
+        const float zi = i >= kt ? dmi[i] : dpl[i];
+        nz = fmaf(zi, zi, nz);
+      }
+      nz = tri_block_sum(nz, red);
+      const double est = beta * (double)(fabsf(n - 1 >= kt ? dmi[n - 1] : dpl[n - 1]) * rsqrtf(nz));
+      const double bound = tol * fmax(1.0, fabs((double)th32));
+      // a decision is due when the estimate is within a factor 2 of the value
+      // that stops the member, or says nothing
+      const bool far = !unsure && isfinite(est) && est > (tol < 1e-5 ? 2.0 : 1.0) * bound;
+      if (far && !force) {
+        if (tid == 0) {
+          out[b * 4 + 0] = th32;
+          out[b * 4 + 1] = est;
+          out[b * 4 + 2] = beta;
+        }
+        leave();
+        return;
+      }
+    }
+    __syncthreads();  // the estimate's arrays are read; warp 0 overwrites them
+  }
+
+  // ---- decision, by warp 0: float32 bracket and start vector, then the float64 eigenpair
+  if (wid != 0) return;
   for (int i = lane; i < n; i += 32) {
-    const double ai = ab[(int64_t)b * cap + i], ei = ab[((int64_t)batch + b) * cap + i];
-    a[i] = ai;
-    e[i] = ei;  // e[n-1] = beta_j, the residual factor
+    const double ai = a[i], ei = e[i];
     e2[i] = ei * ei;
     a32[i] = (float)ai;
     e32[i] = (float)ei;
     e232[i] = (float)(ei * ei);
   }
   __syncwarp();
-  const double beta = e[n - 1];
   // Gershgorin bounds (float64, lane-parallel), amax for the scales
   double glo = 1e300, ghi = 1e300, amax = 0.0;
   for (int i = lane; i < n; i += 32) {
@@ -625,36 +893,32 @@ k_tridiag(const double* __restrict__ ab, double* __restrict__ s_out, double* __r
     amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, o));
   }
   const double scale_t = fmax(1.0, amax);
-  const bool bad = !isfinite(a[n - 1]) || !isfinite(beta);
   const bool small_beta = beta < 1e-14 * scale_t;
-  const bool last = n >= max_iter || (int64_t)n >= D;
-  if (bad) {
-    if (lane == 0) {
-      ctl[LZ_CTL_MEMBER + b] = LZ_NAN;
-      ctl[LZ_CTL_MEMBER + batch + b] = n;
-    }
+  if (!final_pass && !((n % check_every == 0) || last || small_beta)) {
+    leave();
     return;
   }
-  if (!final_pass && !((n % check_every == 0) || last || small_beta)) return;
-
-  // ---- float32 estimate
   const float eps32 = 1.2e-7f;
   const float slack = (float)(8.0 * n * 6e-8 * scale_t);  // rounding of T to float32, Sturm backward error
   float lo = (float)glo - slack, hi = (float)ghi + slack;
   const double ssc = sturm_scale(scale_t);
-  multisection<float>(a32, e232, n, lo, hi, 4.0f * eps32, 12, (float)ssc);
-  const float th32 = 0.5f * (lo + hi);
+  // the scaled entries of the Sturm counts, in the places of e2 and the pivots
+  for (int i = lane; i < n; i += 32) {
+    rp[i] = a[i] * ssc;
+    e2[i] *= ssc * ssc;
+    rp32[i] = a32[i] * (float)ssc;
+    e232[i] *= (float)(ssc * ssc);
+  }
+  __syncwarp();
+  multisection<float>(rp32, e232, n, lo, hi, 4.0f * eps32, 12, (float)ssc);
+  __syncwarp();
   // the multipliers overwrite e2 (the Sturm counts are done)
   inverse_iteration<float>(a32, e32, n, lo - 2.0f * slack - 1e-6f * (float)scale_t, z32, rp32, e232, 3, 1e-30f,
                            false);
   __syncwarp();
   const double est = beta * fabs((double)z32[n - 1]);
-  const bool force = ctl[LZ_CTL_FORCE] != 0;
+  const float th32 = 0.5f * (lo + hi);
   const bool pass32 = est <= 0.5 * tol * fmax(1.0, fabs((double)th32)) || force;
-  // The float32 last component is accurate only to about eps32 |T| / gap
-  // (absolute), so the float32 estimate cannot resolve tolerances much below
-  // 1e-5: such solves take the float64 eigenpair at every check once the
-  // estimate has come within 1e-2 |T|, and stop on the float64 test.
   const bool check64 = !final_pass && tol < 1e-5 && !force && est <= 1e-2 * scale_t;
   if (!final_pass && !(small_beta || last) && !check64) {
     if (lane == 0) {
@@ -666,6 +930,7 @@ k_tridiag(const double* __restrict__ ab, double* __restrict__ s_out, double* __r
         ctl[LZ_CTL_MEMBER + batch + b] = n;
       }
     }
+    leave();
     return;
   }
 
@@ -673,12 +938,13 @@ k_tridiag(const double* __restrict__ ab, double* __restrict__ s_out, double* __r
   double lo64 = (double)lo - 2.0 * slack, hi64 = (double)hi + 2.0 * slack;
   lo64 = fmax(lo64, glo - 1e-300);
   {  // the bracket must hold lambda_min: lane 0 counts at lo64, lane 1 at hi64
-    const int c = sturm_count<double>(a, e2, n, lane == 0 ? lo64 : hi64, ssc);
+    const int c = sturm_count<double>(rp, e2, n, lane == 0 ? lo64 : hi64, ssc);
     const int c_lo = __shfl_sync(0xffffffffu, c, 0), c_hi = __shfl_sync(0xffffffffu, c, 1);
     if (c_lo != 0) lo64 = glo - 1e-300;
     if (c_hi == 0) hi64 = ghi + 1e-12 * scale_t;
   }
-  multisection<double>(a, e2, n, lo64, hi64, 4.0 * 2.2e-16, 64, ssc);
+  multisection<double>(rp, e2, n, lo64, hi64, 4.0 * 2.2e-16, 64, ssc);
+  __syncwarp();
   const double theta = 0.5 * (lo64 + hi64);
   // one solve from the float32 eigenvector: the shift is within a few ulps of
   // lambda_min, so a solve reduces the error by (lambda_1 - sigma) / gap
@@ -686,6 +952,7 @@ k_tridiag(const double* __restrict__ ab, double* __restrict__ s_out, double* __r
   __syncwarp();
   inverse_iteration<double>(a, e, n, lo64 - 4.0 * 2.2e-16 * scale_t, z, rp, e2, 1, 1e-300, true);
   __syncwarp();
+  for (int i = lane; i < n; i += 32) s_out[(int64_t)b * cap + i] = z[i];
   if (lane == 0) {
     const double resid = beta * fabs(z[n - 1]);
     const double scale = fmax(1.0, fabs(theta));
@@ -698,15 +965,16 @@ k_tridiag(const double* __restrict__ ab, double* __restrict__ s_out, double* __r
     out[b * 4 + 0] = theta;
     out[b * 4 + 1] = resid;
     out[b * 4 + 2] = beta;
-    for (int i = 0; i < n; ++i) s_out[(int64_t)b * cap + i] = z[i];
     if (code) {
       ctl[LZ_CTL_MEMBER + b] = code;
       ctl[LZ_CTL_MEMBER + batch + b] = n;
     }
   }
+  leave();
 }
 
-// v_{j+1} = w / beta_j for running members (into the basis and the current vector)
+// v_{j+1} = w / beta_j for running members (into the basis and the current
+// vector); it follows k_tridiag, which has advanced the iteration: j + 1 = ctl[LZ_CTL_J]
 template <bool PAIR>
 __global__ void k_next_vector(const double* __restrict__ w, const double* __restrict__ ab,
                               double* __restrict__ V, double* __restrict__ vcur,
@@ -714,7 +982,7 @@ __global__ void k_next_vector(const double* __restrict__ w, const double* __rest
   __shared__ double s_inv;
   const int b = blockIdx.y;
   if (member_done(ctl, b)) return;
-  const int j = ctl[LZ_CTL_J];
+  const int j = ctl[LZ_CTL_J] - 1;
   // one float64 division per block, not per element (GB300's float64 pipe is narrow)
   if (threadIdx.x == 0) s_inv = 1.0 / ab[((int64_t)batch + b) * cap + j];
   __syncthreads();
@@ -726,15 +994,6 @@ __global__ void k_next_vector(const double* __restrict__ w, const double* __rest
     else vn[d] = v;
     vcur[(int64_t)b * D + d] = v;
   }
-}
-
-__global__ void k_advance(int32_t* ctl, int batch) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  if (ctl[LZ_CTL_ALLDONE]) return;
-  int all = 1;
-  for (int b = 0; b < batch; ++b) all &= (ctl[LZ_CTL_MEMBER + b] != 0);
-  if (all) ctl[LZ_CTL_ALLDONE] = 1;
-  else ctl[LZ_CTL_J] += 1;
 }
 
 // ----------------------------------------------------------- vector helpers
@@ -916,14 +1175,11 @@ void lz_launch_dgks(const double* npart_a, const double* npart_b, int32_t* gate,
                     int nchunk_a, int nchunk, cudaStream_t st) {
   k_dgks<<<batch, 32, 0, st>>>(npart_a, npart_b, gate, ctl, nchunk_a, nchunk);
 }
-void lz_launch_finalize_ab(const double* h, const double* npart_b, const double* npart_c, const int32_t* gate,
-                           double* ab, const int32_t* ctl, int batch, int cap, int nchunk, cudaStream_t st) {
-  k_finalize_ab<<<batch, 32, 0, st>>>(h, npart_b, npart_c, gate, ab, ctl, batch, cap, nchunk);
-}
-void lz_launch_tridiag(const double* ab, double* s, double* out, int32_t* ctl, const double* tol, int batch,
+void lz_launch_tridiag(const double* h, const double* npart_b, const double* npart_c, const int32_t* gate,
+                       int nchunk, double* ab, double* s, double* out, int32_t* ctl, const double* tol, int batch,
                        int cap, int64_t D, cudaStream_t st, int final_pass) {
-  k_tridiag<<<batch, 32, (5 * cap * sizeof(double) + 5 * cap * sizeof(float)), st>>>(ab, s, out, ctl, tol, batch,
-                                                                                   cap, D, final_pass);
+  k_tridiag<<<batch, LZ_TRI, 5 * cap * sizeof(double) + 5 * cap * sizeof(float), st>>>(
+      h, npart_b, npart_c, gate, nchunk, ab, s, out, ctl, tol, batch, cap, D, final_pass);
 }
 static int vec_blocks(int64_t D) {
   int64_t nb = (D + 255) / 256;
@@ -934,7 +1190,6 @@ void lz_launch_next_vector(const double* w, const double* ab, double* V, double*
   if (pair) k_next_vector<true><<<dim3(vec_blocks(D), batch), 256, 0, st>>>(w, ab, V, vcur, ctl, D, batch, cap);
   else k_next_vector<false><<<dim3(vec_blocks(D), batch), 256, 0, st>>>(w, ab, V, vcur, ctl, D, batch, cap);
 }
-void lz_launch_advance(int32_t* ctl, int batch, cudaStream_t st) { k_advance<<<1, 32, 0, st>>>(ctl, batch); }
 void lz_launch_sumsq(const double* x, double* part, int64_t D, int batch, int nchunk, cudaStream_t st) {
   k_sumsq<<<dim3(nchunk, batch), LZ_THREADS, 0, st>>>(x, part, D, nchunk);
 }

@@ -11,7 +11,7 @@ constexpr int LZ_THREADS = 256;   // threads of the vector kernels
 constexpr int LZ_EPT = 4;         // elements per thread
 constexpr int LZ_CHUNK = LZ_THREADS * LZ_EPT;
 constexpr int LZ_ROWS = 4;        // Krylov rows reduced together in k_multidot
-constexpr int LZ_TRI = 32;        // threads of the tridiagonal multisection (one warp)
+constexpr int LZ_TRI = 256;       // threads of the tridiagonal eigenproblem
 constexpr int LZ_DOT_EPT = 16;    // elements per thread in the reorthogonalisation dots
 constexpr int LZ_DOT_CHUNK = LZ_THREADS * LZ_DOT_EPT;
 constexpr int LZ_DOT_WARPS = LZ_THREADS / 32;  // dot partials per chunk (one per warp)
@@ -28,6 +28,9 @@ enum LzCode : int {
   LZ_RUNNING = 0, LZ_CONVERGED = 1, LZ_BREAKDOWN = 2, LZ_NAN = 3, LZ_CAP = 4, LZ_PENDING = 5, LZ_RESUME = 6,
   LZ_HOLD = 7
 };
+
+// control words of a superblock: the header, two per member, k_tridiag's block count
+inline int lz_ctl_words(int batch) { return LZ_CTL_MEMBER + 2 * batch + 1; }
 
 inline int lz_nchunk(int64_t D) { return (int)((D + LZ_CHUNK - 1) / LZ_CHUNK); }
 inline int lz_dot_nchunk(int64_t D) { return (int)((D + LZ_DOT_CHUNK - 1) / LZ_DOT_CHUNK); }
@@ -53,17 +56,18 @@ void lz_launch_multiaxpy(const double* V, double* w, const double* h, double* no
                          const int32_t* gate, cudaStream_t st, bool pair);
 void lz_launch_dgks(const double* npart_a, const double* npart_b, int32_t* gate, const int32_t* ctl, int batch,
                     int nchunk_a, int nchunk, cudaStream_t st);
-void lz_launch_finalize_ab(const double* h, const double* npart_b, const double* npart_c, const int32_t* gate,
-                           double* ab, const int32_t* ctl, int batch, int cap, int nchunk, cudaStream_t st);
 // continued fractions of Lanczos coefficients at complex points (per member)
 void lz_launch_cfrac(const double* norm2, const double* alpha, const double* beta, const int32_t* n, int ld,
                      const double* zr, const double* zi, int n_z, double* gr, double* gi, int batch,
                      cudaStream_t st);
-void lz_launch_tridiag(const double* ab, double* s, double* out, int32_t* ctl, const double* tol, int batch,
+// the end of a Lanczos step: alpha_j and beta_j from the passes' coefficients
+// (h) and norm partials, the tridiagonal test, the iteration's advance;
+// final_pass: the float64 eigenpairs of the pending members only
+void lz_launch_tridiag(const double* h, const double* npart_b, const double* npart_c, const int32_t* gate,
+                       int nchunk, double* ab, double* s, double* out, int32_t* ctl, const double* tol, int batch,
                        int cap, int64_t D, cudaStream_t st, int final_pass = 0);
 void lz_launch_next_vector(const double* w, const double* ab, double* V, double* vcur, const int32_t* ctl,
                            int64_t D, int batch, int cap, cudaStream_t st, bool pair);
-void lz_launch_advance(int32_t* ctl, int batch, cudaStream_t st);
 void lz_launch_sumsq(const double* x, double* part, int64_t D, int batch, int nchunk, cudaStream_t st);
 void lz_launch_dot(const double* x, const double* y, double* part, int64_t D, int batch, int nchunk,
                    cudaStream_t st);
