@@ -109,13 +109,9 @@ struct GPair {
   OpAcc A, B;
 };
 
-SegF64 seg_base() {
-  SegF64 g{};
-  g.coef = -1;
-  return g;
-}
+SegF64 seg_base() { return SegF64{}; }
 
-// L = a block operand (no members)
+// L = a block operand (shared by the members)
 void set_L_op(SegF64& g, const OpAcc& o) {
   g.l_buf = BUF_OPS;
   g.l_off = o.off;
@@ -129,52 +125,26 @@ void set_R_opT(SegF64& g, const OpAcc& o) {
   g.ldr = o.ld;
   g.r_trans = o.trans ? 0 : 1;
 }
-
-// Tile shape of an M x N output: the 16*ni x 16*nj tiling (ni, nj in 1..4)
-// with the least padded area; among equals the largest tile (fewer operand
-// reloads).  Returns ni | nj << 8.
-int32_t f64_shape(int32_t M, int32_t N) {
-  int64_t best = -1;
-  int32_t shape = 4 | (4 << 8);
-  for (int32_t ni = 1; ni <= 4; ++ni)
-    for (int32_t nj = 1; nj <= 4; ++nj) {
-      const int64_t bm = 16 * ni, bn = 16 * nj;
-      const int64_t area = ((M + bm - 1) / bm * bm) * ((N + bn - 1) / bn * bn);
-      const int64_t bs = (int64_t)(shape & 0xff) * (shape >> 8);
-      if (best < 0 || area < best || (area == best && ni * nj > bs)) {
-        best = area;
-        shape = ni | (nj << 8);
-      }
-    }
-  return shape;
+// a member's matrix (row-major, leading dimension ld) as the left or right operand
+void set_L_mat(SegF64& g, int32_t buf, int64_t off, int32_t ld, int64_t bs) {
+  g.l_buf = buf; g.l_off = off; g.ldl = ld; g.l_bs = bs;
+}
+void set_R_mat(SegF64& g, int32_t buf, int64_t off, int32_t ld, int64_t bs) {
+  g.r_buf = buf; g.r_off = off; g.ldr = ld; g.r_bs = bs;
 }
 
-// Append the tiles of one M x N output and its segment list; returns the
-// positions (before sorting) of the new tiles in *ids.
-void add_output(TaskListF64& tl, const TileF64& proto, const std::vector<SegF64>& segs, std::vector<int64_t>* ids) {
-  if (proto.M <= 0 || proto.N <= 0) return;
-  const int32_t sb = (int32_t)tl.h_segs.size();
-  tl.h_segs.insert(tl.h_segs.end(), segs.begin(), segs.end());
-  const int32_t se = (int32_t)tl.h_segs.size();
-  const int32_t shape = f64_shape(proto.M, proto.N);
-  const int32_t bm = 16 * (shape & 0xff), bn = 16 * (shape >> 8);
-  for (int32_t m0 = 0; m0 < proto.M; m0 += bm)
-    for (int32_t n0 = 0; n0 < proto.N; n0 += bn) {
-      TileF64 t = proto;
-      t.m0 = m0;
-      t.n0 = n0;
-      t.seg_begin = sb;
-      t.seg_end = se;
-      t.shape = shape;
-      if (ids) ids->push_back((int64_t)tl.h_tiles.size());
-      tl.h_tiles.push_back(t);
-    }
-}
+// One output matrix and its segments: the first nM form the first group.
+struct OutF64 {
+  TileF64 proto;
+  std::vector<SegF64> segs;
+  int32_t nM = 0;
+};
 
-TileF64 out_tile(int32_t buf, int64_t off, int32_t ldc, int32_t M, int32_t N, int32_t mode) {
+TileF64 out_tile(int32_t buf, int64_t off, int64_t bs, int32_t ldc, int32_t M, int32_t N, int32_t mode) {
   TileF64 t{};
   t.c_buf = buf;
   t.c_off = off;
+  t.c_bs = bs;
   t.ldc = ldc;
   t.M = M;
   t.N = N;
@@ -182,24 +152,100 @@ TileF64 out_tile(int32_t buf, int64_t off, int32_t ldc, int32_t M, int32_t N, in
   return t;
 }
 
-// Heaviest tiles first (one CTA per tile); returns new position of each old tile.
-std::vector<int64_t> sort_tiles(TaskListF64& tl) {
-  const size_t n = tl.h_tiles.size();
-  std::vector<int64_t> w(n), perm(n), where(n);
-  for (size_t i = 0; i < n; ++i) {
-    int64_t k = 0;
-    for (int32_t s = tl.h_tiles[i].seg_begin; s < tl.h_tiles[i].seg_end; ++s) k += tl.h_segs[s].K;
-    w[i] = k * (tl.h_tiles[i].shape & 0xff) * (tl.h_tiles[i].shape >> 8);  // FMAs per thread
+// Below this many 16 x 16 tiles (all members) a list is cut into 8 x 8 tiles:
+// with fewer than about six blocks per SM the longest tile and the SMs left
+// idle cost more than the padding and the copies of small tiles.  Both ways,
+// float64: 69 tiles 37 (16) / 19 us (8), 142 62 / 29, 380 136 / 78, 433 177 /
+// 118, 677 371 / 282 us; from here on the same within 3 % (805 tiles in the
+// output list, more in the intermediates': 279 / 285 us; 355 wide ones 413 /
+// 423 us), double-float 5 to 9 % in favour of 16.
+constexpr int64_t SEG_FEW_TILES = 152 * 6;
+
+// Tile shape of an M x N output with `chunks` K chunks of sumK in all:
+// 8*ni x 8*nj of the least estimated cost.  A tile pays its area, padding
+// included, for every k, and for every chunk a fixed cost (barrier, loop) and
+// its edges (copies).  In cycles of an SM: 0.5 per element and k in float64
+// (2 multiply-adds per clock), 0.1 in double-float (13 instructions, 128
+// lanes), 30 + 0.6 per edge element for a chunk (two warps' instructions on
+// four schedulers).  8 x 8 when the list has few tiles.
+int32_t seg_shape(int32_t M, int32_t N, int64_t sumK, int64_t chunks, bool few, bool df) {
+  if (few) return 1 | (1 << 8);
+  double best = -1.0;
+  int32_t shape = 1 | (1 << 8);
+  for (int32_t ni = 2; ni >= 1; --ni)
+    for (int32_t nj = 2; nj >= 1; --nj) {
+      const int32_t bm = 8 * ni, bn = 8 * nj;
+      const double tiles = (double)((M + bm - 1) / bm) * ((N + bn - 1) / bn);
+      const double cost = tiles * ((df ? 0.1 : 0.5) * sumK * bm * bn + chunks * (30.0 + 0.6 * (bm + bn)));
+      if (best < 0 || cost < best) {
+        best = cost;
+        shape = ni | (nj << 8);
+      }
+    }
+  return shape;
+}
+
+// Cut outputs (their descriptors with the segment range set, their segments in
+// tl.h_segs) into tiles, the heaviest first (one block per tile and member);
+// which[i] (optional) gets the output of tile i.
+std::vector<TileF64> cut_tiles(const TaskListF64& tl, const std::vector<TileF64>& outs, int batch, bool df,
+                               std::vector<int32_t>* which = nullptr) {
+  int64_t t16 = 0;
+  for (const TileF64& o : outs) t16 += (int64_t)((o.M + 15) / 16) * ((o.N + 15) / 16);
+  const bool few = t16 * batch < SEG_FEW_TILES;
+  std::vector<TileF64> tiles;
+  std::vector<int32_t> from;
+  std::vector<int64_t> w;
+  for (size_t i = 0; i < outs.size(); ++i) {
+    TileF64 t = outs[i];
+    if (t.M <= 0 || t.N <= 0) continue;
+    int64_t k = 0, chunks = 0;
+    for (int32_t q = t.seg_begin; q < t.seg_end; ++q) {
+      k += tl.h_segs[q].K;
+      chunks += (tl.h_segs[q].K + 15) / 16;
+    }
+    t.shape = seg_shape(t.M, t.N, k, chunks, few, df);
+    const int32_t bm = 8 * (t.shape & 0xff), bn = 8 * (t.shape >> 8);
+    for (t.m0 = 0; t.m0 < t.M; t.m0 += bm)
+      for (t.n0 = 0; t.n0 < t.N; t.n0 += bn) {
+        tiles.push_back(t);
+        from.push_back((int32_t)i);
+        w.push_back(k * bm * bn);
+      }
   }
+  std::vector<int64_t> perm(tiles.size());
   std::iota(perm.begin(), perm.end(), 0);
   std::stable_sort(perm.begin(), perm.end(), [&](int64_t a, int64_t b) { return w[a] > w[b]; });
-  std::vector<TileF64> nt(n);
-  for (size_t i = 0; i < n; ++i) {
-    nt[i] = tl.h_tiles[perm[i]];
-    where[perm[i]] = (int64_t)i;
+  std::vector<TileF64> out;
+  out.reserve(tiles.size());
+  if (which) which->clear();
+  for (int64_t p : perm) {
+    out.push_back(tiles[p]);
+    if (which) which->push_back(from[p]);
   }
-  tl.h_tiles.swap(nt);
-  return where;
+  if ((int64_t)out.size() * batch > INT32_MAX) throw Invalid{"too many product tiles"};
+  return out;
+}
+
+void make_tiles(TaskListF64& tl, const std::vector<OutF64>& outs, int batch, std::vector<int32_t>* which = nullptr) {
+  std::vector<TileF64> protos;
+  for (const OutF64& o : outs) {
+    TileF64 t = o.proto;
+    t.seg_begin = (int32_t)tl.h_segs.size();
+    t.seg_mid = t.seg_begin + o.nM;
+    tl.h_segs.insert(tl.h_segs.end(), o.segs.begin(), o.segs.end());
+    t.seg_end = (int32_t)tl.h_segs.size();
+    protos.push_back(t);
+  }
+  tl.h_tiles = cut_tiles(tl, protos, batch, false, which);
+}
+
+// the outputs of a list: its tiles at the origin
+std::vector<TileF64> list_outputs(const TaskListF64& tl) {
+  std::vector<TileF64> outs;
+  for (const TileF64& t : tl.h_tiles)
+    if (t.m0 == 0 && t.n0 == 0) outs.push_back(t);
+  return outs;
 }
 
 void finish(TaskListF64& tl) {
@@ -211,100 +257,100 @@ void finish(TaskListF64& tl) {
 void free_tl(TaskListF64& tl) {
   if (tl.d_tiles) cudaFree(tl.d_tiles);
   if (tl.d_segs) cudaFree(tl.d_segs);
+  if (tl.d_tiles_df) cudaFree(tl.d_tiles_df);
+  tl.d_tiles_df = nullptr;
   tl.d_tiles = nullptr;
   tl.d_segs = nullptr;
 }
 
 bool is_gemm_pair(int flags) { return (flags & (DMRG_ID_A | DMRG_ID_B)) == 0; }
 
-// One product over a pair set with the batch members stacked:
-//   phase 1 (two-GEMM pairs): order 1  X_b = c Psi_b B^T  (members along M)
-//                              order 0  T_b = c A Psi_b    (members along N)
-//   group M (members along M): Y_b += c Psi_b B^T (A = 1), Y_b += T_b B^T
-//   group N (members along N): Y_b += c A Psi_b (B = 1),   Y_b += A X_b
-// Intermediates: member b, pair i at T + b*Tm + toff[i], row-major (order 1:
-// r_in x c_out, order 0: r_out x c_in).  scaled = false drops every
+// The intermediates of the two-GEMM pairs: order 1  X_b = c Psi_b B^T,
+// order 0  T_b = c A Psi_b; member b, pair i at T + b*Tm + toff[i], row-major
+// (order 1: r_in x c_out, order 0: r_out x c_in).  scaled = false drops every
 // coefficient (for the per-term dot products).
-// dots = true (with scaled = false): the output tiles are TM_STORE_DOTS and
-// each segment carries its term (coef) for the tile to apply per member.
-void build_stacked(const dmrg_sb* sb, const std::vector<GPair>& P, const std::vector<int64_t>& toff, int64_t Tm,
-                   bool scaled, TaskListF64& ph1, TaskListF64* gM, TaskListF64* gN, bool dots = false) {
-  const int nb = sb->batch;
-  const int64_t D = sb->D;
-  const auto& r = sb->r;
-  const auto& c = sb->c;
+std::vector<OutF64> phase1_outs(const dmrg_sb* sb, const std::vector<GPair>& P, const std::vector<int64_t>& toff,
+                                int64_t Tm, bool scaled) {
+  std::vector<OutF64> outs;
   for (size_t i = 0; i < P.size(); ++i) {
     const GPair& p = P[i];
     if (!is_gemm_pair(p.flags)) continue;
-    const int32_t ro = r[p.s_out], ri = r[p.s_in], co = c[p.s_out], ci = c[p.s_in];
+    const int32_t ro = sb->r[p.s_out], ri = sb->r[p.s_in], co = sb->c[p.s_out], ci = sb->c[p.s_in];
     SegF64 g = seg_base();
     g.K = p.order == 1 ? ci : ri;
-    if (scaled) { g.coef = p.term; g.coef_mode = p.order == 1 ? 1 : 2; }
-    if (p.order == 1) {  // X_b = Psi_b B^T : M = (b, a'), N = beta, K = c_in
-      g.l_buf = BUF_X; g.l_off = sb->off[p.s_in]; g.ldl = ci; g.l_rm = ri; g.l_bs = D;
+    if (scaled) { g.term = p.term; g.scale = p.order == 1 ? 1 : 2; }
+    OutF64 o;
+    if (p.order == 1) {  // X_b = Psi_b B^T
+      set_L_mat(g, BUF_X, sb->off[p.s_in], ci, sb->D);
       set_R_opT(g, p.B);
-      TileF64 t = out_tile(BUF_T, toff[i], co, nb * ri, co, TM_STORE);
-      t.c_rm = ri; t.c_axis = 0; t.c_bs = Tm;
-      add_output(ph1, t, {g}, nullptr);
-    } else {  // T_b = A Psi_b : M = alpha, N = (b, beta'), K = r_in
+      o.proto = out_tile(BUF_T, toff[i], Tm, co, ri, co, TM_STORE);
+    } else {  // T_b = A Psi_b
       set_L_op(g, p.A);
-      g.r_buf = BUF_X; g.r_off = sb->off[p.s_in]; g.ldr = ci; g.r_trans = 0; g.r_rm = ci; g.r_bs = D;
-      TileF64 t = out_tile(BUF_T, toff[i], ci, ro, nb * ci, TM_STORE);
-      t.c_rm = ci; t.c_axis = 1; t.c_bs = Tm;
-      add_output(ph1, t, {g}, nullptr);
+      set_R_mat(g, BUF_X, sb->off[p.s_in], ci, sb->D);
+      o.proto = out_tile(BUF_T, toff[i], Tm, ci, ro, ci, TM_STORE);
     }
+    o.segs.push_back(g);
+    o.nM = 1;
+    outs.push_back(std::move(o));
   }
-  if (!gM) return;
+  return outs;
+}
+
+// The last GEMM of pair i, unscaled unless an identity pair and `scaled`
+// (the two-GEMM pairs carry their coefficient in the intermediate):
+// Psi_b B^T (A = 1), T_b B^T (order 0), A Psi_b (B = 1) or A X_b (order 1).
+SegF64 phase2_seg(const dmrg_sb* sb, const GPair& p, int64_t toff, int64_t Tm, bool scaled) {
+  const int32_t ri = sb->r[p.s_in], ci = sb->c[p.s_in], co = sb->c[p.s_out];
+  SegF64 g = seg_base();
+  g.term = p.term;
+  if (p.flags & DMRG_ID_A) {
+    g.K = ci;
+    set_L_mat(g, BUF_X, sb->off[p.s_in], ci, sb->D);
+    set_R_opT(g, p.B);
+    g.scale = scaled ? 1 : 0;
+  } else if (p.flags & DMRG_ID_B) {
+    g.K = ri;
+    set_L_op(g, p.A);
+    set_R_mat(g, BUF_X, sb->off[p.s_in], ci, sb->D);
+    g.scale = scaled ? 2 : 0;
+  } else if (p.order == 0) {
+    g.K = ci;
+    set_L_mat(g, BUF_T, toff, ci, Tm);
+    set_R_opT(g, p.B);
+  } else {
+    g.K = ri;
+    set_L_op(g, p.A);
+    set_R_mat(g, BUF_T, toff, co, Tm);
+  }
+  return g;
+}
+// whether that GEMM's right operand is an operator (the first group of an output's segments)
+bool in_group_M(const GPair& p) {
+  if (p.flags & DMRG_ID_A) return true;
+  if (p.flags & DMRG_ID_B) return false;
+  return p.order == 0;
+}
+
+// The outputs of the product: Y_b[s] = the segments that end with an operator
+// on the right, then those with one on the left.  dots: the tiles are
+// TM_STORE_DOTS (unscaled segments, each carries its term for the tile).
+std::vector<OutF64> phase2_outs(const dmrg_sb* sb, const std::vector<GPair>& P, const std::vector<int64_t>& toff,
+                                int64_t Tm, bool scaled, bool dots = false) {
   std::vector<std::vector<size_t>> by_out(sb->S);
   for (size_t i = 0; i < P.size(); ++i) by_out[P[i].s_out].push_back(i);
+  std::vector<OutF64> outs;
   for (int s = 0; s < sb->S; ++s) {
-    if ((int64_t)r[s] * c[s] == 0) continue;
-    std::vector<SegF64> sM, sN;
-    for (size_t i : by_out[s]) {
-      const GPair& p = P[i];
-      const int32_t ri = r[p.s_in], ci = c[p.s_in], co = c[p.s_out];
-      SegF64 g = seg_base();
-      if (dots) {
-        g.coef = p.term;
-        g.coef_mode = -1;  // no scaling while loading: the tile scales the segment's sum
-      }
-      if (p.flags & DMRG_ID_A) {  // Y_b += c Psi_b B^T
-        g.K = ci;
-        g.l_buf = BUF_X; g.l_off = sb->off[p.s_in]; g.ldl = ci; g.l_rm = ri; g.l_bs = D;
-        set_R_opT(g, p.B);
-        if (scaled) { g.coef = p.term; g.coef_mode = 1; }
-        sM.push_back(g);
-      } else if (p.flags & DMRG_ID_B) {  // Y_b += c A Psi_b
-        g.K = ri;
-        set_L_op(g, p.A);
-        g.r_buf = BUF_X; g.r_off = sb->off[p.s_in]; g.ldr = ci; g.r_trans = 0; g.r_rm = ci; g.r_bs = D;
-        if (scaled) { g.coef = p.term; g.coef_mode = 2; }
-        sN.push_back(g);
-      } else if (p.order == 0) {  // Y_b += T_b B^T
-        g.K = ci;
-        g.l_buf = BUF_T; g.l_off = toff[i]; g.ldl = ci; g.l_rm = r[p.s_out]; g.l_bs = Tm;
-        set_R_opT(g, p.B);
-        sM.push_back(g);
-      } else {  // Y_b += A X_b
-        g.K = ri;
-        set_L_op(g, p.A);
-        g.r_buf = BUF_T; g.r_off = toff[i]; g.ldr = co; g.r_trans = 0; g.r_rm = co; g.r_bs = Tm;
-        sN.push_back(g);
-      }
+    if ((int64_t)sb->r[s] * sb->c[s] == 0) continue;
+    OutF64 o;
+    o.proto = out_tile(BUF_Y, sb->off[s], sb->D, sb->c[s], sb->r[s], sb->c[s], dots ? TM_STORE_DOTS : TM_STORE);
+    for (int grp = 0; grp < 2; ++grp) {
+      for (size_t i : by_out[s])
+        if (in_group_M(P[i]) == (grp == 0)) o.segs.push_back(phase2_seg(sb, P[i], toff[i], Tm, scaled));
+      if (grp == 0) o.nM = (int32_t)o.segs.size();
     }
-    const bool hasM = !sM.empty(), hasN = !sN.empty();
-    const int32_t mode = dots ? TM_STORE_DOTS : TM_STORE;
-    if (hasM || !hasN) {
-      TileF64 t = out_tile(BUF_Y, sb->off[s], c[s], nb * r[s], c[s], mode);
-      t.c_rm = r[s]; t.c_axis = 0; t.c_bs = D;
-      add_output(*gM, t, sM, nullptr);
-    }
-    if (hasN) {
-      TileF64 t = out_tile(BUF_Y, sb->off[s], c[s], r[s], nb * c[s], mode);
-      t.c_rm = c[s]; t.c_axis = 1; t.c_bs = D; t.add = hasM ? 1 : 0;
-      add_output(*gN, t, sN, nullptr);
-    }
+    outs.push_back(std::move(o));
   }
+  return outs;
 }
 
 // intermediate layout of a pair set: offsets per pair inside one member's T
@@ -321,8 +367,38 @@ int64_t layout_T(const dmrg_sb* sb, const std::vector<GPair>& P, std::vector<int
   return T;
 }
 
+// The partials of a dot list per (member, term), in list order: item i, of
+// term terms[i], has SEG_DOT_PARTS for every member.
+void upload_dot_lists(const dmrg_sb* sb, const std::vector<int32_t>& terms, int32_t*& d_ptr, int32_t*& d_idx,
+                      double*& d_part) {
+  const int64_t per = (int64_t)sb->batch * SEG_DOT_PARTS;
+  if ((int64_t)terms.size() * per > INT32_MAX) throw Invalid{"too many product segments for the per-term dots"};
+  std::vector<std::vector<int32_t>> items((size_t)sb->n_terms);
+  for (size_t i = 0; i < terms.size(); ++i) items[terms[i]].push_back((int32_t)i);
+  std::vector<int32_t> ptr(1, 0), idx;
+  for (int b = 0; b < sb->batch; ++b)
+    for (const std::vector<int32_t>& l : items) {
+      for (int32_t i : l)
+        for (int w = 0; w < SEG_DOT_PARTS; ++w) idx.push_back((int32_t)((i * (int64_t)sb->batch + b) * SEG_DOT_PARTS + w));
+      ptr.push_back((int32_t)idx.size());
+    }
+  upload(d_ptr, ptr);
+  upload(d_idx, idx);
+  if (d_part) cudaFree(d_part);
+  d_part = dalloc<double>((size_t)std::max<int64_t>(1, (int64_t)terms.size() * per));
+}
+
+// number the (tile, segment) items of TM_STORE_DOTS tiles; returns their terms
+std::vector<int32_t> number_segments(const TaskListF64& tl, std::vector<TileF64>& tiles) {
+  std::vector<int32_t> terms;
+  for (TileF64& t : tiles) {
+    t.dot_base = (int32_t)terms.size();
+    for (int32_t q = t.seg_begin; q < t.seg_end; ++q) terms.push_back(tl.h_segs[q].term);
+  }
+  return terms;
+}
+
 void build_f64_tasks(dmrg_sb* sb) {
-  const int nt = sb->n_terms;
   const auto& r = sb->r;
   const auto& c = sb->c;
   std::vector<GPair> fw, bw;
@@ -347,105 +423,59 @@ void build_f64_tasks(dmrg_sb* sb) {
   if (sb->d_T) cudaFree(sb->d_T);
   sb->d_T = dalloc<double>((size_t)sb->T_elems);
 
-  build_stacked(sb, fw, toff_f, Tm, true, sb->f64_fwd1, &sb->f64_fwd2, &sb->f64_fwd3);
-  build_stacked(sb, bw, toff_b, Tm, true, sb->f64_bwd1, &sb->f64_bwd2, &sb->f64_bwd3);
-  build_stacked(sb, fw, toff_f, Tm, false, sb->f64_dot1, nullptr, nullptr);
+  make_tiles(sb->f64_fwd1, phase1_outs(sb, fw, toff_f, Tm, true), sb->batch);
+  make_tiles(sb->f64_fwd2, phase2_outs(sb, fw, toff_f, Tm, true), sb->batch);
+  make_tiles(sb->f64_bwd1, phase1_outs(sb, bw, toff_b, Tm, true), sb->batch);
+  make_tiles(sb->f64_bwd2, phase2_outs(sb, bw, toff_b, Tm, true), sb->batch);
+  make_tiles(sb->f64_dot1, phase1_outs(sb, fw, toff_f, Tm, false), sb->batch);
 
-  // per-term dots: one unstacked output per (member, pair), dotted with G
-  std::vector<std::vector<int64_t>> dot_list((size_t)sb->batch * nt);
-  for (int b = 0; b < sb->batch; ++b) {
-    const int64_t xb = (int64_t)b * sb->D, tb = (int64_t)b * Tm;
+  {  // per-term dots: one output per pair, dotted with G
+    std::vector<OutF64> outs;
     for (size_t i = 0; i < fw.size(); ++i) {
       const GPair& p = fw[i];
-      const int32_t ri = r[p.s_in], ci = c[p.s_in], co = c[p.s_out];
-      SegF64 g = seg_base();
-      if (p.flags & DMRG_ID_B) {
-        g.K = ri; set_L_op(g, p.A);
-        g.r_buf = BUF_X; g.r_off = xb + sb->off[p.s_in]; g.ldr = ci; g.r_trans = 0;
-      } else if (p.flags & DMRG_ID_A) {
-        g.K = ci; g.l_buf = BUF_X; g.l_off = xb + sb->off[p.s_in]; g.ldl = ci; set_R_opT(g, p.B);
-      } else if (p.order == 0) {
-        g.K = ci; g.l_buf = BUF_T; g.l_off = tb + toff_f[i]; g.ldl = ci; set_R_opT(g, p.B);
-      } else {
-        g.K = ri; set_L_op(g, p.A);
-        g.r_buf = BUF_T; g.r_off = tb + toff_f[i]; g.ldr = co; g.r_trans = 0;
-      }
-      std::vector<int64_t> ids;
-      add_output(sb->f64_dot2, out_tile(BUF_G, xb + sb->off[p.s_out], c[p.s_out], r[p.s_out], c[p.s_out], TM_DOT),
-                 {g}, &ids);
-      for (int64_t id : ids) dot_list[(size_t)b * nt + p.term].push_back(id);
+      OutF64 o;
+      o.proto = out_tile(BUF_G, sb->off[p.s_out], sb->D, c[p.s_out], r[p.s_out], c[p.s_out], TM_DOT);
+      o.segs.push_back(phase2_seg(sb, p, toff_f[i], Tm, false));
+      o.nM = 1;
+      outs.push_back(std::move(o));
     }
+    std::vector<int32_t> which;
+    make_tiles(sb->f64_dot2, outs, sb->batch, &which);
+    std::vector<int32_t> terms;
+    for (int32_t i : which) terms.push_back(fw[i].term);
+    upload_dot_lists(sb, terms, sb->d_dot_red_ptr, sb->d_dot_red_idx, sb->d_dot_partial);
   }
-  // H psi with the per-term dots <psi, (A_k x B_k) psi> in one pass: the
-  // output launches of the product with unscaled segments (after f64_dot1's
-  // unscaled intermediates); the tiles apply c(member, term) themselves
-  {
-    TaskListF64 unused;
-    build_stacked(sb, fw, toff_f, Tm, false, unused, &sb->f64_pdot2, &sb->f64_pdot3, true);
+  {  // H psi with the per-term dots <psi, (A_k x B_k) psi> in one pass: the
+     // output launch of the product with unscaled segments (after f64_dot1's
+     // unscaled intermediates); the tiles apply c(member, term) themselves
+    make_tiles(sb->f64_pdot2, phase2_outs(sb, fw, toff_f, Tm, false, true), sb->batch);
+    upload_dot_lists(sb, number_segments(sb->f64_pdot2, sb->f64_pdot2.h_tiles), sb->d_pdot_ptr, sb->d_pdot_idx,
+                     sb->d_pdot_partial);
   }
-  for (TaskListF64* tl : {&sb->f64_fwd1, &sb->f64_fwd2, &sb->f64_fwd3, &sb->f64_bwd1, &sb->f64_bwd2, &sb->f64_bwd3,
-                          &sb->f64_dot1, &sb->f64_pdot2, &sb->f64_pdot3})
-    sort_tiles(*tl);
-  {  // partials of f64_pdot2/3: 64 per (tile, segment) in tile order, then the (member, term) lists
-    std::vector<std::vector<int32_t>> lists((size_t)sb->batch * nt);
-    int32_t base = 0;
-    for (TaskListF64* tl : {&sb->f64_pdot2, &sb->f64_pdot3})
-      for (TileF64& t : tl->h_tiles) {
-        t.dot_base = base;
-        const bool by_col = t.c_rm && t.c_axis == 1;
-        const int32_t bm = 16 * (t.shape & 0xff), bn = 16 * (t.shape >> 8);
-        for (int32_t q = t.seg_begin; q < t.seg_end; ++q) {
-          const int32_t term = tl->h_segs[q].coef;
-          const int64_t slot = (int64_t)(base + (q - t.seg_begin)) * 64;
-          for (int32_t e = 0; e < (by_col ? bn : bm); ++e) {
-            const int32_t g = (by_col ? t.n0 : t.m0) + e;
-            if (g >= (by_col ? t.N : t.M)) break;
-            const int32_t member = t.c_rm ? g / t.c_rm : t.member;
-            lists[(size_t)member * nt + term].push_back((int32_t)(slot + e));
-          }
-        }
-        base += t.seg_end - t.seg_begin;
-      }
-    if ((int64_t)base * 64 > INT32_MAX) throw Invalid{"too many product segments for the per-term dots"};
-    std::vector<int32_t> ptr(1, 0), idx;
-    for (auto& l : lists) {
-      idx.insert(idx.end(), l.begin(), l.end());
-      ptr.push_back((int32_t)idx.size());
-    }
-    upload(sb->d_pdot_ptr, ptr);
-    upload(sb->d_pdot_idx, idx);
-    if (sb->d_pdot_partial) cudaFree(sb->d_pdot_partial);
-    sb->d_pdot_partial = dalloc<double>((size_t)std::max<int64_t>(1, (int64_t)base * 64));
-  }
-  const std::vector<int64_t> where = sort_tiles(sb->f64_dot2);
-  std::vector<int32_t> ptr(1, 0), idx;
-  for (auto& lst : dot_list) {
-    for (int64_t id : lst) idx.push_back((int32_t)where[id]);
-    ptr.push_back((int32_t)idx.size());
-  }
-  upload(sb->d_dot_red_ptr, ptr);
-  upload(sb->d_dot_red_idx, idx);
-  if (sb->d_dot_partial) cudaFree(sb->d_dot_partial);
-  sb->d_dot_partial = dalloc<double>((size_t)std::max<int64_t>(1, (int64_t)sb->f64_dot2.h_tiles.size()));
-  for (TaskListF64* tl : {&sb->f64_fwd1, &sb->f64_fwd2, &sb->f64_fwd3, &sb->f64_dot1, &sb->f64_dot2, &sb->f64_bwd1,
-                          &sb->f64_bwd2, &sb->f64_bwd3, &sb->f64_pdot2, &sb->f64_pdot3})
+  for (TaskListF64* tl : {&sb->f64_fwd1, &sb->f64_fwd2, &sb->f64_dot1, &sb->f64_dot2, &sb->f64_bwd1, &sb->f64_bwd2,
+                          &sb->f64_pdot2})
     finish(*tl);
 }
 
 // ------------------------------------------------------------- products
 // Double-float products read pre-split pairs: the operator arena (split at
 // the first such product) and the input, split into a buffer of its own each
-// time; the intermediates are written and read as pairs.  Returns the
-// buffers and their pair mask.
-uint32_t df_bufs(dmrg_sb* sb, const double* x, double* y, Bufs& bufs, cudaStream_t st) {
+// time; the intermediates are written and read as pairs.
+Bufs df_bufs(dmrg_sb* sb, const double* x, double* y, cudaStream_t st) {
   if (!sb->d_ops_df) {
+    for (TaskListF64* tl : {&sb->f64_fwd1, &sb->f64_fwd2, &sb->f64_dot1, &sb->f64_pdot2}) {
+      std::vector<TileF64> tiles = cut_tiles(*tl, list_outputs(*tl), sb->batch, true);
+      if (tl == &sb->f64_pdot2)
+        upload_dot_lists(sb, number_segments(*tl, tiles), sb->d_pdot_ptr_df, sb->d_pdot_idx_df, sb->d_pdot_partial_df);
+      upload(tl->d_tiles_df, tiles);
+      tl->n_tiles_df = (int64_t)tiles.size();
+    }
     sb->d_ops_df = dalloc<double>((size_t)std::max<int64_t>(sb->ops_elems, 1));
     launch_split_pairs(sb->d_ops, sb->d_ops_df, sb->ops_elems, st);
   }
   if (!sb->d_x_df) sb->d_x_df = dalloc<double>((size_t)(sb->batch * sb->D));
   launch_split_pairs(x, sb->d_x_df, sb->batch * sb->D, st);
-  bufs = Bufs{{sb->d_x_df, y, sb->d_T, sb->d_ops_df, nullptr}};
-  return (1u << BUF_X) | (1u << BUF_T) | (1u << BUF_OPS);
+  return Bufs{{sb->d_x_df, y, sb->d_T, sb->d_ops_df, nullptr}};
 }
 
 // member_done (tensor-core precisions only, may be null): device [batch]
@@ -455,15 +485,12 @@ void matvec(dmrg_sb* sb, int prec, const double* x, double* y, int accumulate, c
             cudaStream_t st, const int32_t* member_done = nullptr) {
   if (prec == DMRG_FP64) {
     Bufs bufs{{const_cast<double*>(x), y, sb->d_T, sb->d_ops, nullptr}};
-    launch_seg_gemm_f64(sb->f64_fwd1, bufs, sb->d_coeffs, sb->n_terms, 0, nullptr, skip, st);
-    launch_seg_gemm_f64(sb->f64_fwd2, bufs, sb->d_coeffs, sb->n_terms, accumulate, nullptr, skip, st);
-    launch_seg_gemm_f64(sb->f64_fwd3, bufs, sb->d_coeffs, sb->n_terms, accumulate, nullptr, skip, st);
+    launch_seg_gemm_f64(sb->f64_fwd1, bufs, sb->d_coeffs, sb->n_terms, sb->batch, 0, nullptr, skip, st);
+    launch_seg_gemm_f64(sb->f64_fwd2, bufs, sb->d_coeffs, sb->n_terms, sb->batch, accumulate, nullptr, skip, st);
   } else if (prec == DMRG_DF64) {  // the same task lists in double-float arithmetic
-    Bufs bufs;
-    const uint32_t pm = df_bufs(sb, x, y, bufs, st);
-    launch_seg_gemm_df(sb->f64_fwd1, bufs, sb->d_coeffs, sb->n_terms, 0, nullptr, skip, st, pm);
-    launch_seg_gemm_df(sb->f64_fwd2, bufs, sb->d_coeffs, sb->n_terms, accumulate, nullptr, skip, st, pm);
-    launch_seg_gemm_df(sb->f64_fwd3, bufs, sb->d_coeffs, sb->n_terms, accumulate, nullptr, skip, st, pm);
+    const Bufs bufs = df_bufs(sb, x, y, st);
+    launch_seg_gemm_df(sb->f64_fwd1, bufs, sb->d_coeffs, sb->n_terms, sb->batch, 0, st);
+    launch_seg_gemm_df(sb->f64_fwd2, bufs, sb->d_coeffs, sb->n_terms, sb->batch, accumulate, st);
   } else {
     tc_matvec(sb, prec, x, y, accumulate, skip, st, member_done);
   }
@@ -473,25 +500,26 @@ void matvec(dmrg_sb* sb, int prec, const double* x, double* y, int accumulate, c
 // y = H psi and dc[b][k] = <psi_b, (A_k x B_k) psi_b> in one pass, in float64
 // or (df) double-float arithmetic
 void matvec_f64_dots(dmrg_sb* sb, const double* psi, double* y, double* dc, cudaStream_t st, bool df = false) {
-  Bufs bufs{{const_cast<double*>(psi), y, sb->d_T, sb->d_ops, nullptr}};
   if (df) {
-    const uint32_t pm = df_bufs(sb, psi, y, bufs, st);
-    launch_seg_gemm_df(sb->f64_dot1, bufs, sb->d_coeffs, sb->n_terms, 0, nullptr, nullptr, st, pm);
-    launch_seg_gemm_df_dots(sb->f64_pdot2, bufs, sb->d_coeffs, sb->n_terms, 0, sb->d_pdot_partial, nullptr, st, pm);
-    launch_seg_gemm_df_dots(sb->f64_pdot3, bufs, sb->d_coeffs, sb->n_terms, 0, sb->d_pdot_partial, nullptr, st, pm);
+    const Bufs bufs = df_bufs(sb, psi, y, st);
+    launch_seg_gemm_df(sb->f64_dot1, bufs, sb->d_coeffs, sb->n_terms, sb->batch, 0, st);
+    launch_seg_gemm_df_dots(sb->f64_pdot2, bufs, sb->d_coeffs, sb->n_terms, sb->batch, 0, sb->d_pdot_partial_df,
+                            st);
   } else {
-    launch_seg_gemm_f64(sb->f64_dot1, bufs, sb->d_coeffs, sb->n_terms, 0, nullptr, nullptr, st);
-    launch_seg_gemm_f64_dots(sb->f64_pdot2, bufs, sb->d_coeffs, sb->n_terms, 0, sb->d_pdot_partial, nullptr, st);
-    launch_seg_gemm_f64_dots(sb->f64_pdot3, bufs, sb->d_coeffs, sb->n_terms, 0, sb->d_pdot_partial, nullptr, st);
+    Bufs bufs{{const_cast<double*>(psi), y, sb->d_T, sb->d_ops, nullptr}};
+    launch_seg_gemm_f64(sb->f64_dot1, bufs, sb->d_coeffs, sb->n_terms, sb->batch, 0, nullptr, nullptr, st);
+    launch_seg_gemm_f64_dots(sb->f64_pdot2, bufs, sb->d_coeffs, sb->n_terms, sb->batch, 0, sb->d_pdot_partial,
+                             nullptr, st);
   }
-  lz_launch_reduce_terms(sb->d_pdot_partial, sb->d_pdot_ptr, sb->d_pdot_idx, dc, sb->batch * sb->n_terms, st);
+  lz_launch_reduce_terms(df ? sb->d_pdot_partial_df : sb->d_pdot_partial, df ? sb->d_pdot_ptr_df : sb->d_pdot_ptr,
+                         df ? sb->d_pdot_idx_df : sb->d_pdot_idx, dc, sb->batch * sb->n_terms, st);
   CK(cudaGetLastError());
 }
 
 void term_dots(dmrg_sb* sb, const double* psi, const double* g, double* dc, cudaStream_t st) {
   Bufs bufs{{const_cast<double*>(psi), nullptr, sb->d_T, sb->d_ops, const_cast<double*>(g)}};
-  launch_seg_gemm_f64(sb->f64_dot1, bufs, sb->d_coeffs, sb->n_terms, 0, nullptr, nullptr, st);
-  launch_seg_gemm_f64(sb->f64_dot2, bufs, sb->d_coeffs, sb->n_terms, 0, sb->d_dot_partial, nullptr, st);
+  launch_seg_gemm_f64(sb->f64_dot1, bufs, sb->d_coeffs, sb->n_terms, sb->batch, 0, nullptr, nullptr, st);
+  launch_seg_gemm_f64(sb->f64_dot2, bufs, sb->d_coeffs, sb->n_terms, sb->batch, 0, sb->d_dot_partial, nullptr, st);
   lz_launch_reduce_terms(sb->d_dot_partial, sb->d_dot_red_ptr, sb->d_dot_red_idx, dc, sb->batch * sb->n_terms, st);
   CK(cudaGetLastError());
 }
@@ -636,7 +664,7 @@ struct LzRun {
 
 int matvec_launches(const dmrg_sb* sb, int prec) {
   if (prec == DMRG_FP64 || prec == DMRG_DF64)
-    return (sb->f64_fwd1.n_tiles > 0) + (sb->f64_fwd2.n_tiles > 0) + (sb->f64_fwd3.n_tiles > 0);
+    return (sb->f64_fwd1.n_tiles > 0) + (sb->f64_fwd2.n_tiles > 0);
   return tc_launches(sb, prec);
 }
 constexpr int LZ_KERNELS_PER_ITER = 11;  // everything in lz_enqueue_iteration besides the product
@@ -858,7 +886,7 @@ RfRun rf_solve(dmrg_sb* sb, double* psi, int prec, int rprec, double tol, int ma
     rf_launch_dir(sb->rf_p, sb->rf_res, sb->rf_psi32, sb->rf_minv, sb->rf_sc, nullptr, D, B, 1, nullptr, st);
     CK(cudaMemcpyAsync(hsc.data(), sb->rf_sc, sizeof(double) * RF_NSC * B, cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
-    r.launches += 9 + (with_dots ? 4 : matvec_launches(sb, rprec));
+    r.launches += 9 + (with_dots ? 3 : matvec_launches(sb, rprec));
     ++r.outer;
     bool all = true;
     for (int b = 0; b < B; ++b) {
@@ -1075,13 +1103,13 @@ void destroy(dmrg_sb* sb) {
   if (!sb) return;
   lz_free(sb);
   tc_free(sb);
-  for (TaskListF64* tl : {&sb->f64_fwd1, &sb->f64_fwd2, &sb->f64_fwd3, &sb->f64_dot1, &sb->f64_dot2, &sb->f64_bwd1,
-                          &sb->f64_bwd2, &sb->f64_bwd3, &sb->f64_pdot2, &sb->f64_pdot3})
+  for (TaskListF64* tl : {&sb->f64_fwd1, &sb->f64_fwd2, &sb->f64_dot1, &sb->f64_dot2, &sb->f64_bwd1, &sb->f64_bwd2,
+                          &sb->f64_pdot2})
     free_tl(*tl);
   for (double* p : {sb->d_coeffs, sb->d_ops, sb->d_T, sb->d_dot_partial, sb->d_scratch, sb->d_red, sb->d_dg,
-                    sb->d_pdot_partial, sb->d_ops_df, sb->d_x_df})
+                    sb->d_pdot_partial, sb->d_pdot_partial_df, sb->d_ops_df, sb->d_x_df})
     if (p) cudaFree(p);
-  for (int32_t* p : {sb->d_pdot_ptr, sb->d_pdot_idx})
+  for (int32_t* p : {sb->d_pdot_ptr, sb->d_pdot_idx, sb->d_pdot_ptr_df, sb->d_pdot_idx_df})
     if (p) cudaFree(p);
   if (sb->d_dg_terms) cudaFree(sb->d_dg_terms);
   if (sb->d_tc_err) cudaFree(sb->d_tc_err);
@@ -1200,9 +1228,8 @@ dmrg_status dmrg_apply_H_backward(dmrg_sb* sb, const double* psi, const double* 
     if (dpsi) {
       if (prec == DMRG_FP64 || !tc_available(sb)) {
         Bufs bufs{{const_cast<double*>(g), dpsi, sb->d_T, sb->d_ops, nullptr}};
-        launch_seg_gemm_f64(sb->f64_bwd1, bufs, sb->d_coeffs, sb->n_terms, 0, nullptr, nullptr, st);
-        launch_seg_gemm_f64(sb->f64_bwd2, bufs, sb->d_coeffs, sb->n_terms, 0, nullptr, nullptr, st);
-        launch_seg_gemm_f64(sb->f64_bwd3, bufs, sb->d_coeffs, sb->n_terms, 0, nullptr, nullptr, st);
+        launch_seg_gemm_f64(sb->f64_bwd1, bufs, sb->d_coeffs, sb->n_terms, sb->batch, 0, nullptr, nullptr, st);
+        launch_seg_gemm_f64(sb->f64_bwd2, bufs, sb->d_coeffs, sb->n_terms, sb->batch, 0, nullptr, nullptr, st);
       } else {
         tc_matvec_T(sb, prec, g, dpsi, st);
       }

@@ -20,12 +20,10 @@ struct Bufs {
   double* p[NBUF];
 };
 
-// One product L (M x K) * R (K x N) added into the tile.  Either operand may
-// stack the batch members along its outer dimension (rows of L, columns of
-// R): element index -> (member, index within the member) with `*_rm` rows
-// per member and `*_bs` elements between members.  The coefficient is a
-// table index (coef_mode 0, -1 = none) or a term whose member is taken from
-// the stacked side (coef_mode 1: rows of L, 2: columns of R).
+// One product L (M x K) * R (K x N) added into the tile, for batch member b:
+// the operands start at l_off + b l_bs and r_off + b r_bs (stride 0: the
+// operator blocks, shared by all members).  scale: the coefficient of the
+// member's `term` multiplies L (1), R (2) or nothing (0).
 struct SegF64 {
   int64_t l_off, r_off;
   int64_t l_bs, r_bs;
@@ -34,30 +32,24 @@ struct SegF64 {
   int32_t K;
   int32_t l_trans;  // 0: L(m,k) = X[m*ldl + k]; 1: L(m,k) = X[k*ldl + m]
   int32_t r_trans;  // 0: R(k,n) = X[k*ldr + n]; 1: R(k,n) = X[n*ldr + k]
-  int32_t l_rm, r_rm;
-  int32_t coef;
-  int32_t coef_mode;
+  int32_t term, scale;
   int32_t pad;
 };
 
-// One output tile C[m0:m0+16*ni, n0:n0+16*nj] of an M x N matrix (ni, nj in
-// 1..4, chosen per output to fit its shape); the members may be stacked along
-// M (c_axis 0) or N (c_axis 1), c_rm rows per member.
+// One output tile C[m0:m0+8*ni, n0:n0+8*nj] of an M x N matrix (ni, nj in 1..2,
+// chosen per output), for every batch member b at c_off + b c_bs.  Its
+// segments form two groups, each summed by itself, then added.
 enum TileMode : int32_t { TM_STORE = 0, TM_DOT = 2, TM_STORE_DOTS = 3 };
 struct TileF64 {
   int64_t c_off, c_bs;
   int32_t c_buf, ldc;
   int32_t M, N, m0, n0;
-  int32_t seg_begin, seg_end;
-  int32_t mode;     // TM_STORE: C = acc (C += acc when the launch accumulates or `add`); TM_DOT: sum(acc .* C);
-                    // TM_STORE_DOTS: C = sum over segments of c(member, seg) * seg_acc, and per segment
-                    // sum(seg_acc .* X) at the same offset of BUF_X (one member per tile)
-  int32_t c_rm, c_axis;
-  int32_t c_trans;  // 0: C(mm, nn) at [mm*ldc + nn]; 1: at [nn*ldc + mm]
-  int32_t add;      // second writer of an output block: always accumulate
+  int32_t seg_begin, seg_mid, seg_end;
+  int32_t mode;     // TM_STORE: C = acc (C += acc when the launch accumulates); TM_DOT: sum(acc .* C);
+                    // TM_STORE_DOTS: C = sum over segments of c(member, term) * seg_acc, and per segment
+                    // sum(seg_acc .* X) at the same offset of BUF_X
   int32_t shape;    // ni | nj << 8
-  int32_t member;   // TM_STORE_DOTS: the batch member of the tile
-  int32_t dot_base; // TM_STORE_DOTS: partials of segment s at dot_out[(dot_base + s - seg_begin) * 64 + row/col]
+  int32_t dot_base; // TM_STORE_DOTS: index of the tile's first segment among all (tile, segment) of the list
 };
 
 struct TaskListF64 {
@@ -65,23 +57,28 @@ struct TaskListF64 {
   std::vector<SegF64> h_segs;
   TileF64* d_tiles = nullptr;
   SegF64* d_segs = nullptr;
-  int64_t n_tiles = 0;
+  int64_t n_tiles = 0;  // per member: a launch has n_tiles * batch blocks, block tile * batch + member
+  // the same outputs cut for double-float arithmetic (at the first such product)
+  TileF64* d_tiles_df = nullptr;
+  int64_t n_tiles_df = 0;
 };
 
+// dot partials per (tile, member), or per (tile, segment, member): one per warp of a block
+constexpr int SEG_DOT_PARTS = 2;
+
 // skip: optional device flag; when *skip != 0 the launch does nothing
-void launch_seg_gemm_f64(const TaskListF64& tl, const Bufs& bufs, const double* coef, int n_terms,
+void launch_seg_gemm_f64(const TaskListF64& tl, const Bufs& bufs, const double* coef, int n_terms, int batch,
                          int accumulate, double* dot_out, const int32_t* skip, cudaStream_t st);
 // tiles of mode TM_STORE_DOTS (product and per-segment dots in one pass)
-void launch_seg_gemm_f64_dots(const TaskListF64& tl, const Bufs& bufs, const double* coef, int n_terms,
+void launch_seg_gemm_f64_dots(const TaskListF64& tl, const Bufs& bufs, const double* coef, int n_terms, int batch,
                               int accumulate, double* dot_out, const int32_t* skip, cudaStream_t st);
-// the same task lists in double-float arithmetic (matvec_df.cu); buffers whose
-// bit is set in pair_mask (1 << BufId) hold float32 pairs (hi, lo) in their
-// 8-byte slots: read without splitting, written (TM_STORE) as pairs
-void launch_seg_gemm_df(const TaskListF64& tl, const Bufs& bufs, const double* coef, int n_terms, int accumulate,
-                        double* dot_out, const int32_t* skip, cudaStream_t st, uint32_t pair_mask = 0);
-void launch_seg_gemm_df_dots(const TaskListF64& tl, const Bufs& bufs, const double* coef, int n_terms,
-                             int accumulate, double* dot_out, const int32_t* skip, cudaStream_t st,
-                             uint32_t pair_mask = 0);
+// the same task lists in double-float arithmetic (matvec_df.cu): the input,
+// the operators and the intermediates hold float32 pairs (hi, lo) in their
+// 8-byte slots, the output is float64
+void launch_seg_gemm_df(const TaskListF64& tl, const Bufs& bufs, const double* coef, int n_terms, int batch,
+                        int accumulate, cudaStream_t st);
+void launch_seg_gemm_df_dots(const TaskListF64& tl, const Bufs& bufs, const double* coef, int n_terms, int batch,
+                             int accumulate, double* dot_out, cudaStream_t st);
 // dst[i] = the double-float pair of src[i] (n elements)
 void launch_split_pairs(const double* src, double* dst, int64_t n, cudaStream_t st);
 
@@ -111,13 +108,16 @@ struct dmrg_sb {
   double flops = 0;            // algorithmic flops of one product, one member
 
   // FP64 task lists
-  dmrg::TaskListF64 f64_fwd1, f64_fwd2, f64_fwd3;  // forward: intermediates, outputs (members along M, along N)
-  dmrg::TaskListF64 f64_bwd1, f64_bwd2, f64_bwd3;  // H^T g
+  dmrg::TaskListF64 f64_fwd1, f64_fwd2;   // forward: intermediates, outputs
+  dmrg::TaskListF64 f64_bwd1, f64_bwd2;   // H^T g
   dmrg::TaskListF64 f64_dot1, f64_dot2;   // per-pair <g, A psi B^T>
-  dmrg::TaskListF64 f64_pdot2, f64_pdot3; // H psi and per-term <psi, (A_k x B_k) psi> in one pass (after f64_dot1)
+  dmrg::TaskListF64 f64_pdot2;            // H psi and per-term <psi, (A_k x B_k) psi> in one pass (after f64_dot1)
   int32_t* d_pdot_ptr = nullptr;          // term reduction of its segment partials, as d_dot_red_*
   int32_t* d_pdot_idx = nullptr;
   double* d_pdot_partial = nullptr;
+  int32_t* d_pdot_ptr_df = nullptr;       // the same for the double-float tiles
+  int32_t* d_pdot_idx_df = nullptr;
+  double* d_pdot_partial_df = nullptr;
   double* d_T = nullptr;                  // FP64 intermediate workspace
   int64_t T_elems = 0;
   int64_t T_fwd_elems = 0;               // the part of it the forward product uses
