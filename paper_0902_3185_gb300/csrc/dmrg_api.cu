@@ -563,7 +563,8 @@ void lz_alloc(dmrg_sb* sb, int cap) {
   sb->lz_partial = dalloc<double>((size_t)B * std::max(sb->lz_nchunk, lz_dot_nparts(sb->D)) * cap);
   sb->lz_h = dalloc<double>((size_t)(3 * B * cap));
   sb->lz_npart = dalloc<double>((size_t)(3 * B * sb->lz_nchunk));
-  sb->lz_gate = dalloc<int32_t>((size_t)B);
+  sb->lz_gate = dalloc<int32_t>((size_t)(2 * B));  // the gates, then the block counts of k_norm_gate
+  CK(cudaMemset(sb->lz_gate, 0, sizeof(int32_t) * 2 * B));
   sb->lz_ab = dalloc<double>((size_t)(2 * B * cap));
   sb->lz_s = dalloc<double>((size_t)(B * cap));
   sb->lz_out = dalloc<double>((size_t)(4 * B + 1));
@@ -608,12 +609,20 @@ void lz_enqueue_iteration(dmrg_sb* sb, int prec, cudaStream_t st) {
   const int ndot = lz_dot_nchunk(D);
   const bool pair = lz_pair(prec);  // the Krylov basis as double-float pairs (mixed-precision solves)
   lz_launch_dots_local(sb->lz_V, sb->lz_w, sb->lz_partial, ctl, D, B, cap, st, pair);
-  lz_launch_reduce_rows(sb->lz_partial, hA, ctl, lz_dot_nparts(D), cap, B, 2, nullptr, st);
-  // pass A's update runs inside pass B's dot sweep (norm partials per dot chunk)
-  lz_launch_multidot(sb->lz_V, sb->lz_w, sb->lz_partial, ctl, D, B, cap, 0, nullptr, st, hA, nA, pair);
-  lz_launch_reduce_rows(sb->lz_partial, hB, ctl, lz_dot_nparts(D), cap, B, 0, nullptr, st);
-  lz_launch_multiaxpy(sb->lz_V, sb->lz_w, hB, nB, ctl, D, B, cap, nch, 0, nullptr, st, pair);
-  lz_launch_dgks(nA, nB, sb->lz_gate, ctl, B, ndot, nch, st);
+  if (lz_short(D, B)) {
+    lz_launch_update_local(sb->lz_V, sb->lz_w, sb->lz_partial, hA, nA, ctl, D, B, cap, st, pair);
+    lz_launch_multidot(sb->lz_V, sb->lz_w, sb->lz_partial, ctl, D, B, cap, 0, nullptr, st, nullptr, nullptr, pair);
+    lz_launch_reduce_rows(sb->lz_partial, hB, ctl, lz_dot_nparts(D), cap, B, 0, nullptr, st);
+    lz_launch_multiaxpy(sb->lz_V, sb->lz_w, hB, nullptr, ctl, D, B, cap, nch, 0, nullptr, st, pair);
+    lz_launch_norm_gate(sb->lz_w, nB, nA, sb->lz_gate, sb->lz_gate + B, ctl, D, B, st);
+  } else {
+    lz_launch_reduce_rows(sb->lz_partial, hA, ctl, lz_dot_nparts(D), cap, B, 2, nullptr, st);
+    // pass A's update runs inside pass B's dot sweep (norm partials per dot chunk)
+    lz_launch_multidot(sb->lz_V, sb->lz_w, sb->lz_partial, ctl, D, B, cap, 0, nullptr, st, hA, nA, pair);
+    lz_launch_reduce_rows(sb->lz_partial, hB, ctl, lz_dot_nparts(D), cap, B, 0, nullptr, st);
+    lz_launch_multiaxpy(sb->lz_V, sb->lz_w, hB, nB, ctl, D, B, cap, nch, 0, nullptr, st, pair);
+    lz_launch_dgks(nA, nB, sb->lz_gate, ctl, B, ndot, nch, st);
+  }
   lz_launch_multidot(sb->lz_V, sb->lz_w, sb->lz_partial, ctl, D, B, cap, 0, sb->lz_gate, st, nullptr, nullptr, pair);
   lz_launch_reduce_rows(sb->lz_partial, hC, ctl, lz_dot_nparts(D), cap, B, 0, sb->lz_gate, st);
   lz_launch_multiaxpy(sb->lz_V, sb->lz_w, hC, nC, ctl, D, B, cap, nch, 0, sb->lz_gate, st, pair);
@@ -1477,7 +1486,8 @@ dmrg_status dmrg_time_reorth(dmrg_sb* sb, int32_t prec, int32_t j, int32_t reps,
       lz_launch_multidot(sb->lz_V, sb->lz_w, sb->lz_partial, sb->lz_ctl, D, B, cap, 0, nullptr, st, nullptr, nullptr,
                          pair);
       lz_launch_reduce_rows(sb->lz_partial, hB, sb->lz_ctl, lz_dot_nparts(D), cap, B, 0, nullptr, st);
-      lz_launch_multiaxpy(sb->lz_V, sb->lz_w, hB, nB, sb->lz_ctl, D, B, cap, nch, 0, nullptr, st, pair);
+      lz_launch_multiaxpy(sb->lz_V, sb->lz_w, hB, lz_short(D, B) ? nullptr : nB, sb->lz_ctl, D, B, cap, nch, 0, nullptr,
+                          st, pair);
     };
     pass();
     cudaEvent_t a, b;

@@ -33,6 +33,7 @@
 // and [5 + batch + b] number of Lanczos vectors in its tridiagonal matrix;
 // last, [5 + 2 batch] counts the blocks of k_tridiag that have finished.
 
+#include <algorithm>
 #include <cfloat>
 
 #include "df.cuh"
@@ -95,20 +96,31 @@ __device__ __forceinline__ int first_row(int j, int win) { return win ? max(0, j
 // With h_pre != NULL the previous pass's update (the three-term step,
 // w -= h_pre[j-1] v_{j-1} + h_pre[j] v_j, in that order) is applied first,
 // written back to w, and its per-chunk sum of squares stored in npart_pre:
-// one sweep instead of an update sweep followed by a dot sweep.
+// one sweep instead of an update sweep followed by a dot sweep (blocks of
+// LZ_THREADS, one row of blocks).
+// The warps of a chunk are independent: a short vector, which would leave most
+// SMs without a block, takes blocks of one warp and splits the groups of 8
+// rows over blockIdx.z (the update then has a kernel of its own,
+// k_update_local); each partial is the same sum either way.  Float64 pass B of
+// the 32-site chain at m = 200 (D = 13 596, 4 chunks, j = 40 on average): 50 us
+// with the update inside, now 3.9 + 9 us.
 template <bool PAIR>
 __global__ void __launch_bounds__(LZ_THREADS, PAIR ? 2 : 3)
 k_multidot(const double* __restrict__ V, double* __restrict__ w, double* __restrict__ partial,
            const int32_t* __restrict__ ctl, int64_t D, int batch, int cap, int nchunk, int win,
            const int32_t* __restrict__ gate, const double* __restrict__ h_pre, double* __restrict__ npart_pre) {
   __shared__ double red[LZ_THREADS / 32][8];
-  const int b = blockIdx.y, chunk = blockIdx.x;
+  const int b = blockIdx.y;
   if (member_skip(ctl, gate, b)) return;
   const int j = ctl[LZ_CTL_J];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
+  const int vw = blockIdx.x * (int)(blockDim.x >> 5) + (int)(threadIdx.x >> 5);  // warp of the member
+  const int chunk = vw / LZ_DOT_WARPS, wid = vw % LZ_DOT_WARPS;
+  const int row0 = first_row(j, win) + 8 * (int)blockIdx.z;
+  if (row0 > j) return;
   double wv[LZ_DOT_EPT];  // w (float64 basis)
   float2 wf[LZ_DOT_EPT];  // w split into double-float pairs (pair basis)
-  const int64_t base = (int64_t)chunk * LZ_DOT_CHUNK + threadIdx.x;
+  const int64_t base = (int64_t)chunk * LZ_DOT_CHUNK + wid * 32 + lane;
   // the pre-update's rows (j - 1 when it exists, then j) and coefficients
   const bool two = j >= 1;
   const double* v0 = V + ((int64_t)(two ? j - 1 : j) * batch + b) * D;
@@ -144,7 +156,7 @@ k_multidot(const double* __restrict__ V, double* __restrict__ w, double* __restr
     }
   }
   const bool full = base + (LZ_DOT_EPT - 1) * LZ_THREADS < D;
-  for (int i0 = first_row(j, win); i0 <= j; i0 += 8) {
+  for (int i0 = row0; i0 <= j; i0 += 8 * (int)gridDim.z) {
     // per-thread sums of 8 rows: float64, or double-float pairs (pair basis)
     double p[8];
     float2 p2[8];
@@ -246,11 +258,13 @@ template <bool PAIR>
 __global__ void __launch_bounds__(LZ_THREADS, 2)
 k_dots_local(const double* __restrict__ V, const double* __restrict__ w, double* __restrict__ partial,
              const int32_t* __restrict__ ctl, int64_t D, int batch, int cap, int nchunk) {
-  const int b = blockIdx.y, chunk = blockIdx.x;
+  const int b = blockIdx.y;
   if (member_done(ctl, b)) return;
   const int j = ctl[LZ_CTL_J];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int64_t base = (int64_t)chunk * LZ_DOT_CHUNK + threadIdx.x;
+  const int lane = threadIdx.x & 31;
+  const int vw = blockIdx.x * (int)(blockDim.x >> 5) + (int)(threadIdx.x >> 5);  // as in k_multidot
+  const int chunk = vw / LZ_DOT_WARPS, wid = vw % LZ_DOT_WARPS;
+  const int64_t base = (int64_t)chunk * LZ_DOT_CHUNK + wid * 32 + lane;
   const bool two = j >= 1;
   const double* wb = w + (int64_t)b * D + base;
   const double* r0 = V + ((int64_t)(two ? j - 1 : j) * batch + b) * D + base;
@@ -304,22 +318,13 @@ k_dots_local(const double* __restrict__ V, const double* __restrict__ w, double*
   }
 }
 
-// h[b*cap + i] = sum of row i's nparts partials, first_row(j, win) <= i <= j:
-// one warp per row (8 rows per block), lane l summing partials l, l + 32, ...
-// in four interleaved accumulators (loads in flight), then a fixed shuffle
-// tree: the same order on every call (deterministic).
-__global__ void __launch_bounds__(256)
-k_reduce_rows(const double* __restrict__ partial, double* __restrict__ h, const int32_t* __restrict__ ctl,
-              int nparts, int cap, int win, const int32_t* __restrict__ gate) {
-  const int b = blockIdx.x;
-  if (member_skip(ctl, gate, b)) return;
-  const int j = ctl[LZ_CTL_J];
-  const int lane = threadIdx.x & 31;
-  const int i = first_row(j, win) + blockIdx.y * 8 + (int)(threadIdx.x >> 5);
-  if (i > j) return;
-  const double* row = partial + ((int64_t)b * cap + i) * nparts;
+// Sum of a row's nparts partials by one warp, the same in every lane: lane l
+// sums partials l, l + 32, ... in four interleaved accumulators (loads in
+// flight), then a fixed shuffle tree: the same order on every call
+// (deterministic).
+__device__ __forceinline__ double warp_sum_row(const double* __restrict__ row, int nparts) {
   double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-  int s = lane;
+  int s = threadIdx.x & 31;
   for (; s + 96 < nparts; s += 128) {
     a0 += row[s];
     a1 += row[s + 32];
@@ -330,13 +335,83 @@ k_reduce_rows(const double* __restrict__ partial, double* __restrict__ h, const 
   double t = (a0 + a1) + (a2 + a3);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-  if (lane == 0) h[(int64_t)b * cap + i] = t;
+  return t;
+}
+
+// h[b*cap + i] = sum of row i's nparts partials, first_row(j, win) <= i <= j:
+// one warp per row (8 rows per block).
+__global__ void __launch_bounds__(256)
+k_reduce_rows(const double* __restrict__ partial, double* __restrict__ h, const int32_t* __restrict__ ctl,
+              int nparts, int cap, int win, const int32_t* __restrict__ gate) {
+  const int b = blockIdx.x;
+  if (member_skip(ctl, gate, b)) return;
+  const int j = ctl[LZ_CTL_J];
+  const int i = first_row(j, win) + blockIdx.y * 8 + (int)(threadIdx.x >> 5);
+  if (i > j) return;
+  const double t = warp_sum_row(partial + ((int64_t)b * cap + i) * nparts, nparts);
+  if ((threadIdx.x & 31) == 0) h[(int64_t)b * cap + i] = t;
+}
+
+// Pass A's reduction and update for a short vector: every block sums the
+// partials of rows j - 1 and j itself (two warps), then applies the three-term
+// step to its LZ_CHUNK elements of w, with the norm partial of the chunk (read
+// by the DGKS test only).
+template <bool PAIR>
+__global__ void __launch_bounds__(LZ_THREADS)
+k_update_local(const double* __restrict__ V, double* __restrict__ w, const double* __restrict__ partial,
+               double* __restrict__ h, double* __restrict__ norm_partial, const int32_t* __restrict__ ctl, int64_t D,
+               int batch, int cap, int nchunk, int nparts) {
+  __shared__ double hs[2];
+  __shared__ double red[LZ_THREADS / 32];
+  const int b = blockIdx.y, chunk = blockIdx.x;
+  if (member_done(ctl, b)) return;
+  const int j = ctl[LZ_CTL_J];
+  const bool two = j >= 1;
+  const int wid = threadIdx.x >> 5;
+  if (wid < 2 && (wid == 1 || two)) {
+    const int64_t i = (int64_t)b * cap + (wid ? j : j - 1);
+    const double t = warp_sum_row(partial + i * nparts, nparts);
+    if ((threadIdx.x & 31) == 0) {
+      hs[wid] = t;
+      if (chunk == 0) h[i] = t;
+    }
+  }
+  const double* v0 = V + ((int64_t)(two ? j - 1 : j) * batch + b) * D;
+  const double* v1 = V + ((int64_t)j * batch + b) * D;
+  double* wb = w + (int64_t)b * D;
+  double x[LZ_EPT], p0[LZ_EPT], p1[LZ_EPT];
+#pragma unroll
+  for (int e = 0; e < LZ_EPT; ++e) {
+    const int64_t d = (int64_t)chunk * LZ_CHUNK + e * LZ_THREADS + threadIdx.x;
+    const bool in = d < D;
+    x[e] = in ? wb[d] : 0.0;
+    p0[e] = in && two ? v_value<PAIR>(v0 + d) : 0.0;
+    p1[e] = in ? v_value<PAIR>(v1 + d) : 0.0;
+  }
+  __syncthreads();
+  const double h0 = two ? hs[0] : 0.0, h1 = hs[1];
+  double nrm = 0.0;
+#pragma unroll
+  for (int e = 0; e < LZ_EPT; ++e) {
+    const int64_t d = (int64_t)chunk * LZ_CHUNK + e * LZ_THREADS + threadIdx.x;
+    if (d >= D) continue;
+    double y = x[e];
+    if (two) y = fma(-p0[e], h0, y);
+    y = fma(-p1[e], h1, y);
+    wb[d] = y;
+    nrm = fma(y, y, nrm);
+  }
+  const double t = block_sum(nrm, red);
+  if (threadIdx.x == 0) norm_partial[(int64_t)b * nchunk + chunk] = t;
 }
 
 // w[b] -= sum_{i0<=i<=j} V[i][b] h[b][i] (i0 = first_row(j, win)); with
-// norm_partial != NULL also the per-chunk sum of squares of the new w.
-template <bool PAIR>
-__global__ void __launch_bounds__(LZ_THREADS)
+// norm_partial != NULL also the per-chunk sum of squares of the new w (EPT =
+// LZ_EPT, blocks of LZ_THREADS).  A short vector takes one element per thread
+// and blocks of two warps, so that every SM has a share of it (its norm
+// partials come from k_norm_gate).
+template <bool PAIR, int EPT>
+__global__ void __launch_bounds__(EPT == 1 ? LZ_AXPY_SHORT : LZ_THREADS)
 k_multiaxpy(const double* __restrict__ V, double* __restrict__ w, const double* __restrict__ h,
             double* __restrict__ norm_partial, const int32_t* __restrict__ ctl, int64_t D, int batch,
             int cap, int nchunk, int win, const int32_t* __restrict__ gate) {
@@ -354,37 +429,38 @@ k_multiaxpy(const double* __restrict__ V, double* __restrict__ w, const double* 
   __syncthreads();
   // the rows in the outer loop and the thread's LZ_EPT elements inside it:
   // independent accumulators, so every row issues LZ_EPT loads at once
-  const int64_t d0 = (int64_t)chunk * LZ_CHUNK + threadIdx.x;
-  const bool full = d0 + (LZ_EPT - 1) * LZ_THREADS < D;
-  double acc[LZ_EPT], wv[LZ_EPT];
-  float ss[LZ_EPT], sc[LZ_EPT];
+  constexpr int T = EPT == 1 ? LZ_AXPY_SHORT : LZ_THREADS;
+  const int64_t d0 = (int64_t)chunk * (EPT * T) + threadIdx.x;
+  const bool full = d0 + (EPT - 1) * T < D;
+  double acc[EPT], wv[EPT];
+  float ss[EPT], sc[EPT];
 #pragma unroll
-  for (int e = 0; e < LZ_EPT; ++e) {
+  for (int e = 0; e < EPT; ++e) {
     acc[e] = 0.0;
     ss[e] = sc[e] = 0.0f;
     // w is loaded before the rows, so that its memory round trip overlaps theirs
-    const int64_t d = d0 + e * LZ_THREADS;
+    const int64_t d = d0 + e * T;
     wv[e] = d < D ? w[(int64_t)b * D + d] : 0.0;
   }
-#pragma unroll 2
+#pragma unroll (EPT == 1 ? 8 : 2)
   for (int i = i0; i <= j; ++i) {
     const double* vi = V + ((int64_t)i * batch + b) * D + d0;
     if (PAIR) {  // sum_i V[i] h[i] in double-float arithmetic
       const float2 hi = shf[i];
 #pragma unroll
-      for (int e = 0; e < LZ_EPT; ++e)
-        if (full || d0 + e * LZ_THREADS < D) df_fma(ld_pair(vi + e * LZ_THREADS), hi, ss[e], sc[e]);
+      for (int e = 0; e < EPT; ++e)
+        if (full || d0 + e * T < D) df_fma(ld_pair(vi + e * T), hi, ss[e], sc[e]);
     } else {
       const double hi = sh[i];
 #pragma unroll
-      for (int e = 0; e < LZ_EPT; ++e)
-        if (full || d0 + e * LZ_THREADS < D) acc[e] = fma(vi[e * LZ_THREADS], hi, acc[e]);
+      for (int e = 0; e < EPT; ++e)
+        if (full || d0 + e * T < D) acc[e] = fma(vi[e * T], hi, acc[e]);
     }
   }
   double nrm = 0.0;
 #pragma unroll
-  for (int e = 0; e < LZ_EPT; ++e) {
-    const int64_t d = d0 + e * LZ_THREADS;
+  for (int e = 0; e < EPT; ++e) {
+    const int64_t d = d0 + e * T;
     if (d >= D) continue;
     const double x = wv[e] - (PAIR ? df_value(ss[e], sc[e]) : acc[e]);
     w[(int64_t)b * D + d] = x;
@@ -414,6 +490,46 @@ __global__ void k_dgks(const double* __restrict__ npart_a, const double* __restr
   const double na = warp_sum_chunks(npart_a + (int64_t)b * nchunk_a, nchunk_a);
   const double nb = warp_sum_chunks(npart_b + (int64_t)b * nchunk, nchunk);
   if (threadIdx.x == 0) gate[b] = (nb >= 0.5 * na) ? 0 : 1;  // NaN: run pass C, then the NaN check stops it
+}
+
+// Pass B's end for a short vector: the norm partials of w (the sums
+// k_multiaxpy forms per chunk, in its order), and in the member's last block
+// the DGKS test on them; tickets[b] counts the member's blocks.
+__global__ void __launch_bounds__(LZ_THREADS)
+k_norm_gate(const double* __restrict__ w, double* __restrict__ npart_b, const double* __restrict__ npart_a,
+            int32_t* __restrict__ gate, int32_t* __restrict__ tickets, const int32_t* __restrict__ ctl, int64_t D,
+            int nchunk) {
+  __shared__ double red[LZ_THREADS / 32];
+  __shared__ int last;
+  const int b = blockIdx.y, chunk = blockIdx.x;
+  if (member_done(ctl, b)) return;
+  double nrm = 0.0;
+#pragma unroll
+  for (int e = 0; e < LZ_EPT; ++e) {
+    const int64_t d = (int64_t)chunk * LZ_CHUNK + e * LZ_THREADS + threadIdx.x;
+    if (d >= D) continue;
+    const double x = w[(int64_t)b * D + d];
+    nrm = fma(x, x, nrm);
+  }
+  const double t = block_sum(nrm, red);
+  if (threadIdx.x == 0) {
+    npart_b[(int64_t)b * nchunk + chunk] = t;
+    __threadfence();
+    last = atomicAdd(&tickets[b], 1) == nchunk - 1;
+  }
+  __syncthreads();
+  if (!last || threadIdx.x >= 32) return;
+  __threadfence();
+  const double na = warp_sum_chunks(npart_a + (int64_t)b * nchunk, nchunk);
+  // written by other blocks of this launch: read past L1
+  double nb = 0.0;
+  for (int ch = threadIdx.x; ch < nchunk; ch += 32) nb += __ldcg(npart_b + (int64_t)b * nchunk + ch);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) nb += __shfl_xor_sync(0xffffffffu, nb, o);
+  if (threadIdx.x == 0) {
+    gate[b] = (nb >= 0.5 * na) ? 0 : 1;  // as in k_dgks
+    tickets[b] = 0;
+  }
 }
 
 // Sign and zero test of a float / double from its bit pattern (integer
@@ -1137,24 +1253,57 @@ void lz_launch_cfrac(const double* norm2, const double* alpha, const double* bet
   if (n_z <= 0 || batch <= 0) return;
   k_cfrac<<<dim3((n_z + 127) / 128, batch), 128, 0, st>>>(norm2, alpha, beta, n, ld, zr, zi, n_z, gr, gi);
 }
+// blocks of a dot pass: LZ_DOT_WARPS warps each (one row of blocks), or for a
+// short vector single warps with the row groups over z, up to about 16 warps per SM
+static void dot_grid(int64_t D, int batch, int cap, dim3& g, int& threads) {
+  const int nch = lz_dot_nchunk(D);
+  if (!lz_short(D, batch)) {
+    g = dim3(nch, batch);
+    threads = LZ_THREADS;
+    return;
+  }
+  const int warps = nch * LZ_DOT_WARPS;
+  const int z = std::min((cap + 7) / 8, std::max(1, 152 * 16 / (warps * batch)));
+  g = dim3(warps, batch, z);
+  threads = 32;
+}
 void lz_launch_multidot(const double* V, double* w, double* partial, const int32_t* ctl, int64_t D,
                         int batch, int cap, int win, const int32_t* gate, cudaStream_t st, const double* h_pre,
                         double* npart_pre, bool pair) {
-  const dim3 g(lz_dot_nchunk(D), batch);
+  dim3 g(lz_dot_nchunk(D), batch);
+  int threads = LZ_THREADS;
+  if (!h_pre) dot_grid(D, batch, cap, g, threads);
   if (pair)
-    k_multidot<true><<<g, LZ_THREADS, 0, st>>>(V, w, partial, ctl, D, batch, cap, lz_dot_nchunk(D), win, gate, h_pre,
-                                               npart_pre);
+    k_multidot<true><<<g, threads, 0, st>>>(V, w, partial, ctl, D, batch, cap, lz_dot_nchunk(D), win, gate, h_pre,
+                                            npart_pre);
   else
-    k_multidot<false><<<g, LZ_THREADS, 0, st>>>(V, w, partial, ctl, D, batch, cap, lz_dot_nchunk(D), win, gate,
-                                                h_pre, npart_pre);
+    k_multidot<false><<<g, threads, 0, st>>>(V, w, partial, ctl, D, batch, cap, lz_dot_nchunk(D), win, gate, h_pre,
+                                             npart_pre);
 }
 void lz_launch_dots_local(const double* V, const double* w, double* partial, const int32_t* ctl, int64_t D,
                           int batch, int cap, cudaStream_t st, bool pair) {
-  const dim3 g(lz_dot_nchunk(D), batch);
+  dim3 g;
+  int threads;
+  dot_grid(D, batch, 1, g, threads);
   if (pair)
-    k_dots_local<true><<<g, LZ_THREADS, 0, st>>>(V, w, partial, ctl, D, batch, cap, lz_dot_nchunk(D));
+    k_dots_local<true><<<g, threads, 0, st>>>(V, w, partial, ctl, D, batch, cap, lz_dot_nchunk(D));
   else
-    k_dots_local<false><<<g, LZ_THREADS, 0, st>>>(V, w, partial, ctl, D, batch, cap, lz_dot_nchunk(D));
+    k_dots_local<false><<<g, threads, 0, st>>>(V, w, partial, ctl, D, batch, cap, lz_dot_nchunk(D));
+}
+void lz_launch_update_local(const double* V, double* w, const double* partial, double* h, double* norm_partial,
+                            const int32_t* ctl, int64_t D, int batch, int cap, cudaStream_t st, bool pair) {
+  const dim3 g(lz_nchunk(D), batch);
+  if (pair)
+    k_update_local<true><<<g, LZ_THREADS, 0, st>>>(V, w, partial, h, norm_partial, ctl, D, batch, cap, lz_nchunk(D),
+                                                   lz_dot_nparts(D));
+  else
+    k_update_local<false><<<g, LZ_THREADS, 0, st>>>(V, w, partial, h, norm_partial, ctl, D, batch, cap, lz_nchunk(D),
+                                                    lz_dot_nparts(D));
+}
+void lz_launch_norm_gate(const double* w, double* npart_b, const double* npart_a, int32_t* gate, int32_t* tickets,
+                         const int32_t* ctl, int64_t D, int batch, cudaStream_t st) {
+  k_norm_gate<<<dim3(lz_nchunk(D), batch), LZ_THREADS, 0, st>>>(w, npart_b, npart_a, gate, tickets, ctl, D,
+                                                               lz_nchunk(D));
 }
 void lz_launch_reduce_rows(const double* partial, double* h, const int32_t* ctl, int nchunk, int cap,
                            int batch, int win, const int32_t* gate, cudaStream_t st) {
@@ -1164,12 +1313,19 @@ void lz_launch_reduce_rows(const double* partial, double* h, const int32_t* ctl,
 void lz_launch_multiaxpy(const double* V, double* w, const double* h, double* norm_partial,
                          const int32_t* ctl, int64_t D, int batch, int cap, int nchunk, int win,
                          const int32_t* gate, cudaStream_t st, bool pair) {
-  if (pair)
-    k_multiaxpy<true><<<dim3(nchunk, batch), LZ_THREADS, cap * sizeof(double), st>>>(V, w, h, norm_partial, ctl, D,
-                                                                                   batch, cap, nchunk, win, gate);
-  else
-    k_multiaxpy<false><<<dim3(nchunk, batch), LZ_THREADS, cap * sizeof(double), st>>>(V, w, h, norm_partial, ctl,
-                                                                                    D, batch, cap, nchunk, win, gate);
+  const size_t smem = cap * sizeof(double);
+  if (!norm_partial) {  // a short vector
+    constexpr int T = LZ_AXPY_SHORT;
+    const int nb = (int)((D + T - 1) / T);
+    if (pair) k_multiaxpy<true, 1><<<dim3(nb, batch), T, smem, st>>>(V, w, h, nullptr, ctl, D, batch, cap, nb, win, gate);
+    else k_multiaxpy<false, 1><<<dim3(nb, batch), T, smem, st>>>(V, w, h, nullptr, ctl, D, batch, cap, nb, win, gate);
+  } else if (pair) {
+    k_multiaxpy<true, LZ_EPT><<<dim3(nchunk, batch), LZ_THREADS, smem, st>>>(V, w, h, norm_partial, ctl, D, batch,
+                                                                             cap, nchunk, win, gate);
+  } else {
+    k_multiaxpy<false, LZ_EPT><<<dim3(nchunk, batch), LZ_THREADS, smem, st>>>(V, w, h, norm_partial, ctl, D, batch,
+                                                                              cap, nchunk, win, gate);
+  }
 }
 void lz_launch_dgks(const double* npart_a, const double* npart_b, int32_t* gate, const int32_t* ctl, int batch,
                     int nchunk_a, int nchunk, cudaStream_t st) {

@@ -14,6 +14,7 @@ constexpr int LZ_ROWS = 4;        // Krylov rows reduced together in k_multidot
 constexpr int LZ_TRI = 256;       // threads of the tridiagonal eigenproblem
 constexpr int LZ_DOT_EPT = 16;    // elements per thread in the reorthogonalisation dots
 constexpr int LZ_DOT_CHUNK = LZ_THREADS * LZ_DOT_EPT;
+constexpr int LZ_AXPY_SHORT = 64;  // threads of the update's blocks for a short vector
 constexpr int LZ_DOT_WARPS = LZ_THREADS / 32;  // dot partials per chunk (one per warp)
 
 // LZ_CTL_FORCE (testing hook): nonzero makes the float32 test pass at its first check
@@ -37,6 +38,15 @@ inline int lz_dot_nchunk(int64_t D) { return (int)((D + LZ_DOT_CHUNK - 1) / LZ_D
 // dot partials per member and Krylov row written by one k_multidot launch
 inline int lz_dot_nparts(int64_t D) { return lz_dot_nchunk(D) * LZ_DOT_WARPS; }
 
+// A short vector (all members): too few chunks to give every SM a few warps in
+// the passes' usual blocks (two blocks of a dot pass each).  The passes then
+// use blocks of one or two warps, and pass A's update and pass B's norms
+// kernels of their own.  All of a step's passes, before -> after: 32-site
+// chain at m = 200 (4 chunks) 80 -> 31 us, ladder at m = 400 (28 chunks, 4
+// members) 134 -> 53 us, chain at m = 1000 in pairs (77 chunks) 64 -> 61 us; the
+// m = 1000 ladder (656 chunks) keeps the update inside the sweep.
+inline bool lz_short(int64_t D, int batch) { return (int64_t)lz_dot_nchunk(D) * batch < 2 * 152; }
+
 // Gram-Schmidt passes over the Krylov rows first_row(j, win)..j (win = 0: all
 // rows); members with gate != NULL and gate[b] == 0 are skipped.
 // h_pre / npart_pre: apply the three-term update with coefficients h_pre
@@ -49,8 +59,15 @@ void lz_launch_multidot(const double* V, double* w, double* partial, const int32
 // pass A's dots (w with v_{j-1} and v_j) into the partials of a win = 2 pass
 void lz_launch_dots_local(const double* V, const double* w, double* partial, const int32_t* ctl, int64_t D,
                           int batch, int cap, cudaStream_t st, bool pair);
+// short vectors: pass A's reduction and update in one launch; pass B's norm
+// partials and the DGKS test (tickets: [batch], zero between launches)
+void lz_launch_update_local(const double* V, double* w, const double* partial, double* h, double* norm_partial,
+                            const int32_t* ctl, int64_t D, int batch, int cap, cudaStream_t st, bool pair);
+void lz_launch_norm_gate(const double* w, double* npart_b, const double* npart_a, int32_t* gate, int32_t* tickets,
+                         const int32_t* ctl, int64_t D, int batch, cudaStream_t st);
 void lz_launch_reduce_rows(const double* partial, double* h, const int32_t* ctl, int nchunk, int cap,
                            int batch, int win, const int32_t* gate, cudaStream_t st);
+// norm_partial == NULL: a short vector, no norm partials
 void lz_launch_multiaxpy(const double* V, double* w, const double* h, double* norm_partial,
                          const int32_t* ctl, int64_t D, int batch, int cap, int nchunk, int win,
                          const int32_t* gate, cudaStream_t st, bool pair);
