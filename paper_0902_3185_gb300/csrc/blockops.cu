@@ -191,7 +191,7 @@ __device__ __forceinline__ double eig_block_sum(double v, double* red) {
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
   __syncthreads();
   double t = 0.0;
-  for (int w = 0; w < EIG_THREADS / 32; ++w) t += red[w];
+  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
   return t;
 }
 
@@ -303,139 +303,256 @@ __global__ void __launch_bounds__(EIG_THREADS) k_eig(const EigJob* __restrict__ 
   }
 }
 
-// The same cyclic Jacobi for a matrix too large for one block's shared
-// memory, on a cluster of EIG_CLUSTER blocks whose shared memories together
-// hold A and V (thread-block clusters with distributed shared memory).  Row i
-// of A and of V lives in block i % C (local row i / C).  A round of disjoint
-// rotations: (1) the owner of row p = min(p, q) of each pair computes (c, s)
-// from a_pp, a_pq (local) and a_qq (remote); (2) every block gathers all
-// rotations, and the owner of p rotates rows p (local) and q (remote, read
-// and written through distributed shared memory) -- no other block touches
-// them; (3) every block rotates columns p, q of its own rows of A and V.
-// Cluster barriers separate the phases.  All blocks sum the convergence test
-// in the same order, so they leave the sweep loop together.
+// The same cyclic Jacobi on a thread-block cluster, for matrices whose columns
+// fit the cluster's shared memory.
+//
+// What bounds it: one SM issues 2 float64 operations per clock, and a round
+// costs 6 n^2 of them (rows and columns of A, columns of V), so the round is
+// spread over the cluster's SMs; then the barriers between its steps count.
+// The round-robin ordering is played as a tournament: block c of the cluster
+// keeps a run of neighbouring pair slots, the columns of A and V of both
+// players of each.  Given all rotations of the round, everything is local to
+// a column pair: the row rotations act within a column, then the pair's own
+// rotation mixes its two columns (and those of V).  Between rounds the players
+// move on by one slot: inside a block that is a change of a table, and two
+// columns cross to the neighbouring blocks (distributed shared memory, into a
+// spare column there).  So a round has two cluster barriers: after A's columns
+// have moved, and after the next round's rotations are published to every
+// block; V, which no rotation depends on, is rotated between the two, beside
+// the square roots and divisions of those rotations.
+// Rotation order and arithmetic are those of k_eig (every element sees the
+// same operations in the same order).
+//
+// Measured against one block with A and V in shared memory (up to n = 110) and
+// a 16-block cluster with rows dealt to the blocks and three barriers a round
+// (above): one matrix of n = 48 2.79 -> 2.05 ms, 64 5.35 -> 2.8, 80 9.88 -> 3.6,
+// 110 24.7 -> 6.2, 300 66.7 -> 58 ms; 24 of n = 110 24.8 -> 10 ms.  At n = 300 the
+// float64 unit of the cluster's SMs is 43 % busy (a sweep is 18 million cycles
+// of it per 1000 rounds, 9 to 10 sweeps); 512 threads per block were faster
+// for one wide matrix (51 ms) but slower for many (24 of n = 110 15.5 ms).
 constexpr int EIG_CLUSTER = 16;
 
-__global__ void __launch_bounds__(EIG_THREADS) k_eig_cluster(const EigJob* __restrict__ jobs) {
+// x != 0 by its bits (a float64 compare runs on the float64 unit)
+__device__ __forceinline__ bool nonzero(double x) {
+  return ((__double2hiint(x) & 0x7fffffff) | __double2loint(x)) != 0;
+}
+
+__host__ __device__ inline int eig_active_blocks(int np, int C) { return np / 2 < 1 ? 1 : (np / 2 < C ? np / 2 : C); }
+
+constexpr int EIGC_THREADS = 256, EIGC_WARPS = EIGC_THREADS / 32;
+
+__global__ void __launch_bounds__(EIGC_THREADS) k_eig_cluster(const EigJob* __restrict__ jobs) {
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
   extern __shared__ double sm[];
-  __shared__ double red[EIG_THREADS / 32];
+  __shared__ double red[EIGC_WARPS];
   __shared__ double sums[1];
-  __shared__ int n_own;
   const int C = (int)cl.num_blocks();
   const int rank = (int)cl.block_rank();
   const EigJob jb = jobs[blockIdx.x / C];
   const int n = jb.n;
   const int n2 = (n + 1) & ~1;
   const int np = n2 / 2;
-  const int R = (n + C - 1) / C;
-  const int rows = rank < n ? (n - 1 - rank) / C + 1 : 0;  // own rows: rank, rank + C, ...
-  double* a = sm;                       // [R][n]
-  double* v = sm + (size_t)R * n;       // [R][n]
-  double* par = v + (size_t)R * n;      // [np][2] rotations of the pairs this block owns
-  double* allp = par + 2 * np;          // [np][2] all rotations of the round
-  double* dg = allp + 2 * np;           // [n] diagonal (final ordering)
-  int* own = reinterpret_cast<int*>(dg + n);  // [np] pairs this block owns
-  int* rk = own + np;                         // [n]
-  const int tid = threadIdx.x;
-  for (int e = tid; e < rows * n; e += EIG_THREADS) {
-    const int li = e / n, j = e % n, i = rank + C * li;
-    a[li * n + j] = jb.A[(int64_t)i * n + j];
-    v[li * n + j] = i == j ? 1.0 : 0.0;
-  }
-  // sum over the cluster of one value per block, in the same order in every block
-  auto cluster_sum = [&](double v) -> double {
-    v = eig_block_sum(v, red);
-    if (tid == 0) sums[0] = v;
-    cl.sync();
-    double t = 0.0;
-    for (int b = 0; b < C; ++b) t += cl.map_shared_rank(sums, b)[0];
-    cl.sync();  // read before any block writes the next one
-    return t;
-  };
-  double fro = 0.0;
-  for (int e = tid; e < rows * n; e += EIG_THREADS) {
-    const double x = a[(e / n) * n + e % n];
-    fro = fma(x, x, fro);
-  }
-  const double thr = 4.0 * 2.220446049250313e-16 * sqrt(cluster_sum(fro));
-  for (int sweep = 0; sweep < 40; ++sweep) {
-    double rot = 0.0;  // rotations this block computed in the sweep
-    for (int r = 0; r < n2 - 1; ++r) {
-      if (tid == 0) n_own = 0;
-      __syncthreads();
-      for (int k = tid; k < np; k += EIG_THREADS) {
-        int p = rr_player(k, r, n2), q = rr_player(n2 - 1 - k, r, n2);
-        if (p > q) { const int t = p; p = q; q = t; }
-        if (p % C != rank) continue;
-        double c = 1.0, s = 0.0;
-        if (q < n) {
-          const double apq = a[(p / C) * n + q];
-          if (fabs(apq) > thr) {
-            const double* ra = cl.map_shared_rank(a, q % C);
-            const double aqq = ra[(q / C) * n + q];
-            const double tau = (aqq - a[(p / C) * n + p]) / (2.0 * apq);
-            double t;
-            if (fabs(tau) > 1e150) t = 0.5 / tau;
-            else t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-            c = 1.0 / sqrt(1.0 + t * t);
-            s = t * c;
-            rot += 1.0;
-          }
-        }
-        par[2 * k] = c;
-        par[2 * k + 1] = s;
-        if (s != 0.0) own[atomicAdd(&n_own, 1)] = k;
-      }
-      cl.sync();
-      for (int k = tid; k < np; k += EIG_THREADS) {  // gather every pair's rotation
-        int p = rr_player(k, r, n2), q = rr_player(n2 - 1 - k, r, n2);
-        if (p > q) { const int t = p; p = q; q = t; }
-        const double* rp = cl.map_shared_rank(par, p % C);
-        allp[2 * k] = rp[2 * k];
-        allp[2 * k + 1] = rp[2 * k + 1];
-      }
-      const int no = n_own;
-      for (int e = tid; e < no * n; e += EIG_THREADS) {  // rows p (local) and q (remote) of owned pairs
-        const int k = own[e / n], j = e % n;
-        int p = rr_player(k, r, n2), q = rr_player(n2 - 1 - k, r, n2);
-        if (p > q) { const int t = p; p = q; q = t; }
-        const double c = par[2 * k], s = par[2 * k + 1];
-        double* rq = cl.map_shared_rank(a, q % C) + (size_t)(q / C) * n;
-        double* rowp = a + (size_t)(p / C) * n;
-        const double x = rowp[j], y = rq[j];
-        rowp[j] = c * x - s * y;
-        rq[j] = s * x + c * y;
-      }
-      cl.sync();
-      for (int e = tid; e < rows * np; e += EIG_THREADS) {  // columns p, q of own rows of A and V
-        const int li = e / np, k = e % np;
-        const double s = allp[2 * k + 1];
-        if (s == 0.0) continue;
-        const double c = allp[2 * k];
-        int p = rr_player(k, r, n2), q = rr_player(n2 - 1 - k, r, n2);
-        if (p > q) { const int t = p; p = q; q = t; }
-        double* ra = a + (size_t)li * n;
-        double* rv = v + (size_t)li * n;
-        const double x = ra[p], y = ra[q];
-        ra[p] = c * x - s * y;
-        ra[q] = s * x + c * y;
-        const double xv = rv[p], yv = rv[q];
-        rv[p] = c * xv - s * yv;
-        rv[q] = s * xv + c * yv;
-      }
-      cl.sync();
+  // this block's pairs: slots k0 .. k0 + m - 1 of the top row and the ones facing them
+  const int Ca = eig_active_blocks(np, C);
+  const int base = np / Ca, rem = np % Ca, mmax = base + (rem > 0);
+  const int m = rank < Ca ? base + (rank < rem) : 0;
+  const int k0 = rank < Ca ? rank * base + min(rank, rem) : np;
+  const int ncol = 2 * mmax + 2;
+  double2* allp = reinterpret_cast<double2*>(sm);     // [2][np] (c, s) of this round and the next
+  double* a = sm + 4 * np;                            // [ncol][n] columns of A
+  double* v = a + (size_t)ncol * n;                   // [ncol][n] columns of V
+  double* dg = v + (size_t)ncol * n;                  // [n] diagonal (final ordering)
+  int* rk = reinterpret_cast<int*>(dg + n);           // [n]
+  int* top = rk + n;                                  // [2][mmax] column of each top slot, this round and the next
+  int* bot = top + 2 * mmax;                          // [2][mmax] of the slot facing it
+  int* spare = bot + 2 * mmax;                        // [2][2] where a column from the right, the left goes
+  short2* rows = reinterpret_cast<short2*>(spare + 4);  // [2][np] (p, q) of each pair, this round and the next
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  for (int e = tid; e < 2 * m * n; e += EIGC_THREADS) {
+    const int i = e / (2 * m), lc = e % (2 * m);
+    const int j = lc < m ? k0 + lc : n2 - 1 - (k0 + lc - m);  // the player of a slot before the first round
+    if (j < n) {
+      a[(size_t)lc * n + i] = jb.A[(int64_t)i * n + j];
+      v[(size_t)lc * n + i] = i == j ? 1.0 : 0.0;
     }
-    if (cluster_sum(rot) == 0.0) break;  // every block leaves together
   }
-  // decreasing order: every block gathers the diagonal, ranks it, and writes its own rows of V
-  for (int i = tid; i < n; i += EIG_THREADS) {
-    const double* ra = cl.map_shared_rank(a, i % C);
-    dg[i] = ra[(i / C) * n + i];
+  for (int kk = tid; kk < m; kk += EIGC_THREADS) {
+    top[kk] = kk;
+    bot[kk] = m + kk;
   }
-  __syncthreads();
-  for (int i = tid; i < n; i += EIG_THREADS) {
+  if (tid == 0) {
+    spare[0] = 2 * m;
+    spare[1] = 2 * m + 1;
+  }
+  // |A|_F^2 by the first EIG_THREADS threads, summed as in k_eig
+  double fro = 0.0;
+  if (tid < EIG_THREADS)
+    for (int e = tid; e < n * n; e += EIG_THREADS) {
+      const double x = jb.A[e];
+      fro = fma(x, x, fro);
+    }
+  const double thr = 4.0 * 2.220446049250313e-16 * sqrt(eig_block_sum(fro, red));
+  // the pairs of round r, and its rotations from the columns in place (tables
+  // tp, bt), published to every block
+  double rot = 0.0;  // rotations this thread computed
+  auto rotations = [&](int r, const int* tp, const int* bt, double2* out, short2* pq) {
+    for (int k = tid; k < np; k += EIGC_THREADS) {
+      const int pt = rr_player(k, r, n2), pb = rr_player(n2 - 1 - k, r, n2);
+      pq[k] = make_short2((short)min(pt, pb), (short)max(pt, pb));
+    }
+    for (int kk = tid; kk < m; kk += EIGC_THREADS) {
+      const int k = k0 + kk;
+      const int pt = rr_player(k, r, n2), pb = rr_player(n2 - 1 - k, r, n2);
+      const int p = min(pt, pb), q = max(pt, pb);
+      double c = 1.0, s = 0.0;
+      if (q < n) {
+        const double* ap = a + (size_t)(pt < pb ? tp[kk] : bt[kk]) * n;
+        const double* aq = a + (size_t)(pt < pb ? bt[kk] : tp[kk]) * n;
+        const double apq = aq[p];
+        if (fabs(apq) > thr) {
+          const double tau = (aq[q] - ap[p]) / (2.0 * apq);
+          double t;
+          if (fabs(tau) > 1e150) t = 0.5 / tau;
+          else t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
+          c = 1.0 / sqrt(1.0 + t * t);
+          s = t * c;
+          rot += 1.0;
+        }
+      }
+      const double2 cs = make_double2(c, s);
+      for (int b = 0; b < Ca; ++b) cl.map_shared_rank(out, b)[k] = cs;
+    }
+  };
+  cl.sync();
+  if (n > 1) rotations(0, top, bot, allp, rows);
+  cl.sync();
+  int par = 0;
+  for (int sweep = 0; n > 1 && sweep < 40; ++sweep) {
+    double done = 0.0;  // rotations of this sweep
+    for (int r = 0; r < n2 - 1; ++r) {
+      const int* tp = top + par * mmax;
+      const int* bt = bot + par * mmax;
+      const int* sp = spare + par * 2;
+      const double2* cs = allp + (size_t)par * np;
+      const short2* pq = rows + (size_t)par * np;
+      const int nch = (np + 31) / 32;
+      for (int task = wid; task < m * nch; task += EIGC_WARPS) {  // A: a column pair's elements of 32 row pairs
+        const int kk = task / nch, kr = (task - kk * nch) * 32 + lane;
+        if (kr >= np) continue;
+        const double2 col = cs[k0 + kk], row = cs[kr];
+        const bool rcol = nonzero(col.y), rrow = nonzero(row.y);
+        if (!rcol && !rrow) continue;
+        const short2 own = pq[k0 + kk], rr = pq[kr];
+        const bool tf = rr_player(k0 + kk, r, n2) == own.x;
+        double* ap = a + (size_t)(tf ? tp[kk] : bt[kk]) * n;
+        double* aq = a + (size_t)(tf ? bt[kk] : tp[kk]) * n;
+        const bool hasq = own.y < n;  // else column p has no partner this round
+        const int rp = rr.x, rq = rr.y;
+        const bool hasr = rq < n;
+        double x11 = ap[rp], x21 = hasr ? ap[rq] : 0.0;
+        double x12 = hasq ? aq[rp] : 0.0, x22 = hasq && hasr ? aq[rq] : 0.0;
+        if (rrow) {
+          const double c = row.x, s = row.y;
+          const double x = x11, y = x21;
+          x11 = c * x - s * y;
+          x21 = s * x + c * y;
+          const double x2 = x12, y2 = x22;
+          x12 = c * x2 - s * y2;
+          x22 = s * x2 + c * y2;
+        }
+        if (rcol) {
+          const double c = col.x, s = col.y;
+          const double x = x11, y = x12;
+          x11 = c * x - s * y;
+          x12 = s * x + c * y;
+          const double x2 = x21, y2 = x22;
+          x21 = c * x2 - s * y2;
+          x22 = s * x2 + c * y2;
+        }
+        ap[rp] = x11;
+        if (hasr) ap[rq] = x21;
+        if (hasq) {
+          aq[rp] = x12;
+          if (hasr) aq[rq] = x22;
+        }
+      }
+      __syncthreads();
+      // the players move on: tops down by one slot, facing slots up, around
+      // the ends; the columns sent away are the next spares
+      const bool left = np > 1 && rank > 0 && rank < Ca, right = np > 1 && rank < Ca - 1;
+      int* nt = top + (par ^ 1) * mmax;
+      int* nb = bot + (par ^ 1) * mmax;
+      for (int kk = tid; kk < m; kk += EIGC_THREADS) {
+        nt[kk] = k0 + kk == 0 ? tp[0] : (kk < m - 1 ? tp[kk + 1] : (right ? sp[0] : bt[m - 1]));
+        nb[kk] = np == 1 ? bt[0] : (kk > 0 ? bt[kk - 1] : (left ? sp[1] : tp[1]));
+      }
+      if (tid == 0 && m > 0) {
+        spare[(par ^ 1) * 2] = left ? tp[0] : bt[m - 1];
+        spare[(par ^ 1) * 2 + 1] = right ? bt[m - 1] : tp[0];
+      }
+      const size_t to_left = left ? (size_t)cl.map_shared_rank(spare, rank - 1)[par * 2] * n : 0;
+      const size_t to_right = right ? (size_t)cl.map_shared_rank(spare, rank + 1)[par * 2 + 1] * n : 0;
+      auto move = [&](double* cols) {
+        if (left) {
+          double* dst = cl.map_shared_rank(cols, rank - 1) + to_left;
+          const double* src = cols + (size_t)tp[0] * n;
+          for (int i = tid; i < n; i += EIGC_THREADS) dst[i] = src[i];
+        }
+        if (right) {
+          double* dst = cl.map_shared_rank(cols, rank + 1) + to_right;
+          const double* src = cols + (size_t)bt[m - 1] * n;
+          for (int i = tid; i < n; i += EIGC_THREADS) dst[i] = src[i];
+        }
+      };
+      move(a);
+      cl.sync();  // A's columns are where the next round wants them
+      done += rot;
+      rot = 0.0;
+      rotations(r + 1 < n2 - 1 ? r + 1 : 0, nt, nb, allp + (size_t)(par ^ 1) * np,
+                rows + (size_t)(par ^ 1) * np);
+      const int nchv = (n + 31) / 32;
+      for (int task = wid; task < m * nchv; task += EIGC_WARPS) {  // V, beside the next rotations
+        const int kk = task / nchv, i = (task - kk * nchv) * 32 + lane;
+        const double2 col = cs[k0 + kk];
+        if (i >= n || !nonzero(col.y)) continue;
+        const bool tf = rr_player(k0 + kk, r, n2) == pq[k0 + kk].x;
+        double* vp = v + (size_t)(tf ? tp[kk] : bt[kk]) * n;
+        double* vq = v + (size_t)(tf ? bt[kk] : tp[kk]) * n;
+        const double c = col.x, s = col.y;
+        const double xv = vp[i], yv = vq[i];
+        vp[i] = c * xv - s * yv;
+        vq[i] = s * xv + c * yv;
+      }
+      __syncthreads();
+      move(v);
+      par ^= 1;
+      cl.sync();  // the next rotations and V's columns are everywhere
+    }
+    done = eig_block_sum(done, red);
+    if (tid == 0) sums[0] = done;
+    cl.sync();
+    double all = 0.0;
+    for (int b = 0; b < C; ++b) all += cl.map_shared_rank(sums, b)[0];
+    cl.sync();  // read before any block writes the next one
+    if (all == 0.0) break;  // every block leaves together
+  }
+  // decreasing order (ties by index): every block gathers the diagonal and
+  // ranks it, and writes its own columns of V
+  auto slot_col = [&](int lc, int& j) -> int {  // local column lc < 2 m: its index in A and its place
+    j = lc < m ? k0 + lc : n2 - 1 - (k0 + lc - m);
+    return lc < m ? top[par * mmax + lc] : bot[par * mmax + lc - m];
+  };
+  for (int lc = tid; lc < 2 * m; lc += EIGC_THREADS) {
+    int j;
+    const int col = slot_col(lc, j);
+    if (j >= n) continue;
+    const double d = a[(size_t)col * n + j];
+    for (int b = 0; b < Ca; ++b) cl.map_shared_rank(dg, b)[j] = d;
+  }
+  cl.sync();
+  if (m == 0) return;
+  for (int i = tid; i < n; i += EIGC_THREADS) {
     const double wi = dg[i];
     int r2 = 0;
     for (int j = 0; j < n; ++j) r2 += (dg[j] > wi) || (dg[j] == wi && j < i);
@@ -443,31 +560,45 @@ __global__ void __launch_bounds__(EIG_THREADS) k_eig_cluster(const EigJob* __res
   }
   __syncthreads();
   if (rank == 0)
-    for (int i = tid; i < n; i += EIG_THREADS) jb.w[rk[i]] = dg[i];
-  for (int e = tid; e < rows * n; e += EIG_THREADS) {
-    const int li = e / n, j = e % n, i = rank + C * li;
-    jb.V[(int64_t)i * n + rk[j]] = v[li * n + j];
+    for (int i = tid; i < n; i += EIGC_THREADS) jb.w[rk[i]] = dg[i];
+  for (int e = tid; e < 2 * m * n; e += EIGC_THREADS) {
+    const int i = e / (2 * m), lc = e % (2 * m);
+    int j;
+    const int col = slot_col(lc, j);
+    if (j < n) jb.V[(int64_t)i * n + rk[j]] = v[(size_t)col * n + i];
   }
-  cl.sync();  // no block leaves while others may still read its shared memory
 }
 
-size_t eig_cluster_smem(int n) {
-  const size_t R = (size_t)(n + EIG_CLUSTER - 1) / EIG_CLUSTER, np = (size_t)(n + 1) / 2;
-  return 2 * R * n * sizeof(double) + 4 * np * sizeof(double) + n * sizeof(double) + (np + n) * sizeof(int);
+size_t eig_cluster_smem(int n, int C) {
+  const size_t np = (size_t)(n + 1) / 2;
+  const size_t Ca = (size_t)eig_active_blocks((int)np, C), mmax = (np + Ca - 1) / Ca;
+  return (4 * np + 2 * (2 * mmax + 2) * n + n) * sizeof(double) + (n + 4 * mmax + 4 + 2 * np) * sizeof(int);
 }
 
 // largest n the cluster kernel takes (A and V in the cluster's shared memory)
 constexpr int EIG_CLUSTER_MAX_N = 448;
 
+// Blocks per cluster for matrices up to n (> EIG_ONE_BLOCK_N): the float64 work
+// of a round, 3 n^2 cycles of one SM, against the cluster's barriers.
+int eig_cluster_blocks(int n) { return n > 64 ? EIG_CLUSTER : 8; }
+
+// Up to here one block is faster: the square roots and divisions of a round are
+// most of it, and the cluster adds its barriers (n = 16 369 / 538 us, n = 32 1.07
+// / 1.21 ms, n = 40 1.90 / 1.60 ms).
+constexpr int EIG_ONE_BLOCK_N = 32;
+
 // -1: not tried, 0: unavailable on this device, 1: available
 int g_cluster_ok = -1;
 
-bool launch_eig_cluster(const std::vector<EigJob>& jobs, cudaStream_t st) {
+// one launch, the largest matrices first; false if the device has no such clusters
+bool launch_eig_cluster(std::vector<EigJob> jobs, cudaStream_t st) {
   if (jobs.empty()) return true;
-  size_t smem = 0;
-  for (const EigJob& j : jobs) smem = std::max(smem, eig_cluster_smem(j.n));
-  smem = (smem + 15) & ~(size_t)15;
   if (g_cluster_ok == 0) return false;
+  std::stable_sort(jobs.begin(), jobs.end(), [](const EigJob& x, const EigJob& y) { return x.n > y.n; });
+  const int C = eig_cluster_blocks(jobs[0].n);
+  size_t smem = 0;
+  for (const EigJob& j : jobs) smem = std::max(smem, eig_cluster_smem(j.n, C));
+  smem = (smem + 15) & ~(size_t)15;
   if (cudaFuncSetAttribute(k_eig_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
       cudaFuncSetAttribute(k_eig_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
     cudaGetLastError();
@@ -475,13 +606,13 @@ bool launch_eig_cluster(const std::vector<EigJob>& jobs, cudaStream_t st) {
     return false;
   }
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)(EIG_CLUSTER * jobs.size()));
-  cfg.blockDim = dim3(EIG_THREADS);
+  cfg.gridDim = dim3((unsigned)(C * jobs.size()));
+  cfg.blockDim = dim3(EIGC_THREADS);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = EIG_CLUSTER;
+  attr[0].val.clusterDim.x = C;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
@@ -502,15 +633,21 @@ bool launch_eig_cluster(const std::vector<EigJob>& jobs, cudaStream_t st) {
 
 void launch_eig(const std::vector<EigJob>& all, cudaStream_t st) {
   if (all.empty()) return;
-  // sizes between the one-block shared-memory limit and the cluster limit go to
-  // the cluster kernel when the device runs it; the rest to the one-block kernel
-  std::vector<EigJob> mid, jobs;
-  for (const EigJob& j : all) (j.n > EIG_SMEM_MAX_N && j.n <= EIG_CLUSTER_MAX_N ? mid : jobs).push_back(j);
-  if (!launch_eig_cluster(mid, st))
-    for (const EigJob& j : mid) {
-      if (!j.work) throw std::logic_error("eigensolve: missing workspace");
-      jobs.push_back(j);
-    }
+  // everything up to the cluster limit goes to the cluster kernel when the
+  // device runs it (matrices that fit one block's shared memory in a launch of
+  // their own: the larger ones' shared memory would leave one block per SM);
+  // the rest to the one-block kernel
+  std::vector<EigJob> mid, small, jobs;
+  for (const EigJob& j : all)
+    if (j.n > 0) (j.n > EIG_CLUSTER_MAX_N ? jobs : j.n > EIG_SMEM_MAX_N ? mid : small).push_back(j);
+  int widest = 0;
+  for (const EigJob& j : small) widest = std::max(widest, j.n);
+  for (std::vector<EigJob>* set : {&mid, &small})
+    if ((set == &small && widest <= EIG_ONE_BLOCK_N) || !launch_eig_cluster(*set, st))
+      for (const EigJob& j : *set) {
+        if (j.n > EIG_SMEM_MAX_N && !j.work) throw std::logic_error("eigensolve: missing workspace");
+        jobs.push_back(j);
+      }
   if (jobs.empty()) return;
   size_t smem = 0;
   for (const EigJob& j : jobs) {

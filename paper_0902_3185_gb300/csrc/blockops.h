@@ -35,7 +35,7 @@ struct GemmJob {
 void launch_gemm(const std::vector<GemmJob>& jobs, cudaStream_t st);
 
 // Eigen-decomposition of symmetric n x n matrices by cyclic Jacobi rotations
-// (one block per matrix): w (n) in decreasing order, V (n x n row-major, column
+// (a thread-block cluster per matrix, or one block): w (n) in decreasing order, V (n x n row-major, column
 // j the eigenvector of w[j]).  A is not modified.  work: 2 n (n + 1) doubles of
 // device memory per job whose n exceeds the shared-memory limit (else unused).
 struct EigJob {
