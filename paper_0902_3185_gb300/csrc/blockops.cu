@@ -13,6 +13,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <stdexcept>
 #include <string>
 
@@ -24,17 +25,39 @@ namespace dmrg {
 
 namespace {
 
-template <class T>
-T* upload_async(const std::vector<T>& h, cudaStream_t st) {
-  void* p = nullptr;
-  cudaError_t e = cudaMallocAsync(&p, std::max<size_t>(1, h.size()) * sizeof(T), st);
-  if (e != cudaSuccess) throw std::runtime_error(std::string("cudaMallocAsync: ") + cudaGetErrorString(e));
-  if (!h.empty()) {
-    e = cudaMemcpyAsync(p, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice, st);
+// The job lists of one launch on the device: one allocation (from the calling
+// thread's pool, else on the stream) and one copy for both arrays, released in
+// stream order after the launch.
+struct Upload {
+  char* p = nullptr;
+  size_t bytes = 0;
+  cudaStream_t st;
+  DevPool* pool;
+  template <class A, class B>
+  Upload(const std::vector<A>& a, const std::vector<B>& b, const A** da, const B** db, cudaStream_t s)
+      : st(s), pool(DevPool::current()) {
+    const size_t na = (a.size() * sizeof(A) + 15) & ~(size_t)15, nb = b.size() * sizeof(B);
+    bytes = std::max<size_t>(na + nb, 16);
+    std::vector<char> host(bytes);
+    if (!a.empty()) memcpy(host.data(), a.data(), a.size() * sizeof(A));
+    if (!b.empty()) memcpy(host.data() + na, b.data(), nb);
+    cudaError_t e = cudaSuccess;
+    if (pool) p = static_cast<char*>(pool->get(bytes));
+    else e = cudaMallocAsync(reinterpret_cast<void**>(&p), bytes, st);
+    if (e != cudaSuccess) throw std::runtime_error(std::string("cudaMallocAsync: ") + cudaGetErrorString(e));
+    e = cudaMemcpyAsync(p, host.data(), bytes, cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) throw std::runtime_error(std::string("cudaMemcpyAsync: ") + cudaGetErrorString(e));
+    *da = reinterpret_cast<const A*>(p);
+    *db = reinterpret_cast<const B*>(p + na);
   }
-  return static_cast<T*>(p);
-}
+  ~Upload() {
+    if (!p) return;
+    if (pool) pool->put(p, bytes);
+    else cudaFreeAsync(p, st);
+  }
+  Upload(const Upload&) = delete;
+  Upload& operator=(const Upload&) = delete;
+};
 
 void check_launch(const char* what) {
   const cudaError_t e = cudaGetLastError();
@@ -46,6 +69,44 @@ struct Tile {
 };
 
 }  // namespace
+
+// --------------------------------------------------------------------- pool
+namespace {
+thread_local DevPool* g_pool = nullptr;
+int size_class(size_t bytes) {
+  int c = 12;
+  while (((size_t)1 << c) < bytes) ++c;
+  return c;
+}
+}  // namespace
+
+DevPool* DevPool::current() { return g_pool; }
+DevPool* DevPool::set_current(DevPool* p) {
+  DevPool* old = g_pool;
+  g_pool = p;
+  return old;
+}
+void* DevPool::get(size_t bytes) {
+  const int c = size_class(bytes);
+  if (c <= MAX_CLASS && !free_[c].empty()) {
+    void* p = free_[c].back();
+    free_[c].pop_back();
+    return p;
+  }
+  void* p = nullptr;
+  const cudaError_t e = cudaMalloc(&p, c <= MAX_CLASS ? (size_t)1 << c : bytes);
+  if (e != cudaSuccess) throw std::runtime_error(std::string("cudaMalloc: ") + cudaGetErrorString(e));
+  return p;
+}
+void DevPool::put(void* p, size_t bytes) {
+  const int c = size_class(bytes);
+  if (c <= MAX_CLASS && free_[c].size() < MAX_KEPT) free_[c].push_back(p);
+  else cudaFree(p);
+}
+DevPool::~DevPool() {
+  for (std::vector<void*>& l : free_)
+    for (void* p : l) cudaFree(p);
+}
 
 // ------------------------------------------------------------------ scatter
 // One 32 x 32 destination tile per block (32 x 8 threads); a transposed
@@ -83,12 +144,11 @@ void launch_scatter(const std::vector<ScatJob>& jobs, cudaStream_t st) {
     for (int i0 = 0; i0 < jobs[q].rows; i0 += 32)
       for (int j0 = 0; j0 < jobs[q].cols; j0 += 32) tiles.push_back({(int32_t)q, i0, j0, 0});
   if (tiles.empty()) return;
-  ScatJob* dj = upload_async(jobs, st);
-  Tile* dt = upload_async(tiles, st);
+  const ScatJob* dj;
+  const Tile* dt;
+  const Upload up(jobs, tiles, &dj, &dt, st);
   k_scatter<<<(unsigned)tiles.size(), dim3(32, 8), 0, st>>>(dj, dt);
   check_launch("k_scatter");
-  cudaFreeAsync(dj, st);
-  cudaFreeAsync(dt, st);
 }
 
 // ------------------------------------------------------------------- gemm
@@ -162,12 +222,11 @@ void launch_gemm(const std::vector<GemmJob>& jobs, cudaStream_t st) {
       for (int n0 = 0; n0 < j.N; n0 += 64) tiles.push_back({(int32_t)q, m0, n0, 0});
   }
   if (tiles.empty()) return;
-  GemmJob* dj = upload_async(jobs, st);
-  Tile* dt = upload_async(tiles, st);
+  const GemmJob* dj;
+  const Tile* dt;
+  const Upload up(jobs, tiles, &dj, &dt, st);
   k_gemm<<<(unsigned)tiles.size(), 256, 0, st>>>(dj, dt);
   check_launch("k_gemm");
-  cudaFreeAsync(dj, st);
-  cudaFreeAsync(dt, st);
 }
 
 // ---------------------------------------------------------------- eigen
@@ -624,10 +683,11 @@ bool launch_eig_cluster(std::vector<EigJob> jobs, cudaStream_t st) {
     return false;
   }
   g_cluster_ok = 1;
-  EigJob* dj = upload_async(jobs, st);
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_eig_cluster, (const EigJob*)dj);
+  const EigJob* dj;
+  const char* none;
+  const Upload up(jobs, std::vector<char>(), &dj, &none, st);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_eig_cluster, dj);
   if (e != cudaSuccess) throw std::runtime_error(std::string("k_eig_cluster: ") + cudaGetErrorString(e));
-  cudaFreeAsync(dj, st);
   return true;
 }
 
@@ -661,10 +721,11 @@ void launch_eig(const std::vector<EigJob>& all, cudaStream_t st) {
   smem = (smem + 15) & ~(size_t)15;
   cudaError_t e = cudaFuncSetAttribute(k_eig, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) throw std::runtime_error(std::string("k_eig smem: ") + cudaGetErrorString(e));
-  EigJob* dj = upload_async(jobs, st);
+  const EigJob* dj;
+  const char* none;
+  const Upload up(jobs, std::vector<char>(), &dj, &none, st);
   k_eig<<<(unsigned)jobs.size(), EIG_THREADS, smem, st>>>(dj);
   check_launch("k_eig");
-  cudaFreeAsync(dj, st);
 }
 
 // -------------------------------------------------------------- selection

@@ -11,6 +11,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <initializer_list>
 #include <new>
 #include <stdexcept>
 #include <numeric>
@@ -53,13 +54,82 @@ long fail_alloc_at() {
   return at;
 }
 
+void count_alloc() {
+  if (fail_alloc_at() > 0 && ++g_alloc_count == fail_alloc_at()) throw CudaError{cudaErrorMemoryAllocation, "cudaMalloc (injected)"};
+}
+
 template <class T>
 T* dalloc(size_t n) {
   if (n == 0) n = 1;
   void* p = nullptr;
-  if (fail_alloc_at() > 0 && ++g_alloc_count == fail_alloc_at()) throw CudaError{cudaErrorMemoryAllocation, "cudaMalloc (injected)"};
+  count_alloc();
   CK(cudaMalloc(&p, n * sizeof(T)));
   return static_cast<T*>(p);
+}
+
+// One device allocation for many small arrays: a superblock has some fifty
+// (task lists, tables, solver vectors), and a DMRG step makes a superblock, so
+// an allocation, a copy and a release for each had cost more than the
+// solves of a short chain.  Arrays are asked for first (with their contents or
+// without), then allocated and filled together; large ones stay on their own.
+class Slab {
+ public:
+  static constexpr size_t LARGE = 1 << 20;
+  template <class T>
+  void array(T*& d, size_t n, const T* h = nullptr) {
+    count_alloc();
+    const size_t bytes = std::max<size_t>(n, 1) * sizeof(T);
+    if (bytes > LARGE) {
+      CK(cudaMalloc(reinterpret_cast<void**>(&d), bytes));
+      if (h && n) CK(cudaMemcpy(d, h, n * sizeof(T), cudaMemcpyHostToDevice));
+      return;
+    }
+    std::vector<Want>& w = h ? filled_ : empty_;
+    w.push_back({reinterpret_cast<void**>(&d), bytes, {}});
+    if (h && n) w.back().data.assign(reinterpret_cast<const char*>(h), reinterpret_cast<const char*>(h) + n * sizeof(T));
+  }
+  template <class T>
+  void array(T*& d, const std::vector<T>& h) {
+    static const T none{};
+    array(d, h.size(), h.empty() ? &none : h.data());
+  }
+  // allocate and fill; *slab, *size: the allocation (released by its owner)
+  void make(char** slab, size_t* size) {
+    size_t at = 0;
+    for (auto* w : {&filled_, &empty_})
+      for (Want& x : *w) at += (x.bytes + 255) & ~(size_t)255;
+    CK(cudaMalloc(reinterpret_cast<void**>(slab), std::max<size_t>(at, 256)));
+    *size = at;
+    std::vector<char> host;
+    at = 0;
+    for (auto* w : {&filled_, &empty_})
+      for (Want& x : *w) {
+        *x.p = *slab + at;
+        if (w == &filled_) {
+          host.resize(at + x.bytes);
+          std::copy(x.data.begin(), x.data.end(), host.begin() + at);
+        }
+        at += (x.bytes + 255) & ~(size_t)255;
+      }
+    if (!host.empty()) CK(cudaMemcpy(*slab, host.data(), host.size(), cudaMemcpyHostToDevice));
+  }
+
+ private:
+  struct Want {
+    void** p;
+    size_t bytes;
+    std::vector<char> data;
+  };
+  std::vector<Want> filled_, empty_;
+};
+
+// release an array unless it lies in one of the superblock's slabs
+void dfree(const dmrg_sb* sb, void* p) {
+  const char* c = static_cast<char*>(p);
+  if (!c) return;
+  if (sb->slab && c >= sb->slab && c < sb->slab + std::max<size_t>(sb->slab_bytes, 1)) return;
+  if (sb->lz_slab && c >= sb->lz_slab && c < sb->lz_slab + std::max<size_t>(sb->lz_slab_bytes, 1)) return;
+  cudaFree(p);
 }
 
 template <class T>
@@ -193,35 +263,40 @@ std::vector<TileF64> cut_tiles(const TaskListF64& tl, const std::vector<TileF64>
   int64_t t16 = 0;
   for (const TileF64& o : outs) t16 += (int64_t)((o.M + 15) / 16) * ((o.N + 15) / 16);
   const bool few = t16 * batch < SEG_FEW_TILES;
-  std::vector<TileF64> tiles;
-  std::vector<int32_t> from;
-  std::vector<int64_t> w;
+  // all tiles of an output weigh the same: the outputs are sorted, then cut
+  struct Cut {
+    int64_t w;
+    int32_t i, shape;
+  };
+  std::vector<Cut> cuts;
+  cuts.reserve(outs.size());
+  size_t total = 0;
   for (size_t i = 0; i < outs.size(); ++i) {
-    TileF64 t = outs[i];
+    const TileF64& t = outs[i];
     if (t.M <= 0 || t.N <= 0) continue;
     int64_t k = 0, chunks = 0;
     for (int32_t q = t.seg_begin; q < t.seg_end; ++q) {
       k += tl.h_segs[q].K;
       chunks += (tl.h_segs[q].K + 15) / 16;
     }
-    t.shape = seg_shape(t.M, t.N, k, chunks, few, df);
+    const int32_t shape = seg_shape(t.M, t.N, k, chunks, few, df);
+    const int32_t bm = 8 * (shape & 0xff), bn = 8 * (shape >> 8);
+    cuts.push_back({k * bm * bn, (int32_t)i, shape});
+    total += (size_t)((t.M + bm - 1) / bm) * ((t.N + bn - 1) / bn);
+  }
+  std::stable_sort(cuts.begin(), cuts.end(), [](const Cut& x, const Cut& y) { return x.w > y.w; });
+  std::vector<TileF64> out;
+  out.reserve(total);
+  if (which) which->clear();
+  for (const Cut& c : cuts) {
+    TileF64 t = outs[c.i];
+    t.shape = c.shape;
     const int32_t bm = 8 * (t.shape & 0xff), bn = 8 * (t.shape >> 8);
     for (t.m0 = 0; t.m0 < t.M; t.m0 += bm)
       for (t.n0 = 0; t.n0 < t.N; t.n0 += bn) {
-        tiles.push_back(t);
-        from.push_back((int32_t)i);
-        w.push_back(k * bm * bn);
+        out.push_back(t);
+        if (which) which->push_back(c.i);
       }
-  }
-  std::vector<int64_t> perm(tiles.size());
-  std::iota(perm.begin(), perm.end(), 0);
-  std::stable_sort(perm.begin(), perm.end(), [&](int64_t a, int64_t b) { return w[a] > w[b]; });
-  std::vector<TileF64> out;
-  out.reserve(tiles.size());
-  if (which) which->clear();
-  for (int64_t p : perm) {
-    out.push_back(tiles[p]);
-    if (which) which->push_back(from[p]);
   }
   if ((int64_t)out.size() * batch > INT32_MAX) throw Invalid{"too many product tiles"};
   return out;
@@ -248,15 +323,15 @@ std::vector<TileF64> list_outputs(const TaskListF64& tl) {
   return outs;
 }
 
-void finish(TaskListF64& tl) {
+void finish(TaskListF64& tl, Slab& slab) {
   tl.n_tiles = (int64_t)tl.h_tiles.size();
-  upload(tl.d_tiles, tl.h_tiles);
-  upload(tl.d_segs, tl.h_segs);
+  slab.array(tl.d_tiles, tl.h_tiles);
+  slab.array(tl.d_segs, tl.h_segs);
 }
 
-void free_tl(TaskListF64& tl) {
-  if (tl.d_tiles) cudaFree(tl.d_tiles);
-  if (tl.d_segs) cudaFree(tl.d_segs);
+void free_tl(const dmrg_sb* sb, TaskListF64& tl) {
+  dfree(sb, tl.d_tiles);
+  dfree(sb, tl.d_segs);
   if (tl.d_tiles_df) cudaFree(tl.d_tiles_df);
   tl.d_tiles_df = nullptr;
   tl.d_tiles = nullptr;
@@ -370,7 +445,7 @@ int64_t layout_T(const dmrg_sb* sb, const std::vector<GPair>& P, std::vector<int
 // The partials of a dot list per (member, term), in list order: item i, of
 // term terms[i], has SEG_DOT_PARTS for every member.
 void upload_dot_lists(const dmrg_sb* sb, const std::vector<int32_t>& terms, int32_t*& d_ptr, int32_t*& d_idx,
-                      double*& d_part) {
+                      double*& d_part, Slab* slab = nullptr) {
   const int64_t per = (int64_t)sb->batch * SEG_DOT_PARTS;
   if ((int64_t)terms.size() * per > INT32_MAX) throw Invalid{"too many product segments for the per-term dots"};
   std::vector<std::vector<int32_t>> items((size_t)sb->n_terms);
@@ -382,10 +457,17 @@ void upload_dot_lists(const dmrg_sb* sb, const std::vector<int32_t>& terms, int3
         for (int w = 0; w < SEG_DOT_PARTS; ++w) idx.push_back((int32_t)((i * (int64_t)sb->batch + b) * SEG_DOT_PARTS + w));
       ptr.push_back((int32_t)idx.size());
     }
+  const size_t parts = (size_t)std::max<int64_t>(1, (int64_t)terms.size() * per);
+  if (slab) {
+    slab->array(d_ptr, ptr);
+    slab->array(d_idx, idx);
+    slab->array(d_part, parts);
+    return;
+  }
   upload(d_ptr, ptr);
   upload(d_idx, idx);
   if (d_part) cudaFree(d_part);
-  d_part = dalloc<double>((size_t)std::max<int64_t>(1, (int64_t)terms.size() * per));
+  d_part = dalloc<double>(parts);
 }
 
 // number the (tile, segment) items of TM_STORE_DOTS tiles; returns their terms
@@ -398,7 +480,7 @@ std::vector<int32_t> number_segments(const TaskListF64& tl, std::vector<TileF64>
   return terms;
 }
 
-void build_f64_tasks(dmrg_sb* sb) {
+void build_f64_tasks(dmrg_sb* sb, Slab& slab) {
   const auto& r = sb->r;
   const auto& c = sb->c;
   std::vector<GPair> fw, bw;
@@ -420,8 +502,7 @@ void build_f64_tasks(dmrg_sb* sb) {
   const int64_t Tm = std::max(Tf, Tb);
   sb->T_elems = Tm * sb->batch;
   sb->T_fwd_elems = Tf > 0 ? Tm * (sb->batch - 1) + Tf : 0;  // member b's forward intermediates at b Tm + [0, Tf)
-  if (sb->d_T) cudaFree(sb->d_T);
-  sb->d_T = dalloc<double>((size_t)sb->T_elems);
+  slab.array(sb->d_T, (size_t)sb->T_elems);
 
   make_tiles(sb->f64_fwd1, phase1_outs(sb, fw, toff_f, Tm, true), sb->batch);
   make_tiles(sb->f64_fwd2, phase2_outs(sb, fw, toff_f, Tm, true), sb->batch);
@@ -443,18 +524,18 @@ void build_f64_tasks(dmrg_sb* sb) {
     make_tiles(sb->f64_dot2, outs, sb->batch, &which);
     std::vector<int32_t> terms;
     for (int32_t i : which) terms.push_back(fw[i].term);
-    upload_dot_lists(sb, terms, sb->d_dot_red_ptr, sb->d_dot_red_idx, sb->d_dot_partial);
+    upload_dot_lists(sb, terms, sb->d_dot_red_ptr, sb->d_dot_red_idx, sb->d_dot_partial, &slab);
   }
   {  // H psi with the per-term dots <psi, (A_k x B_k) psi> in one pass: the
      // output launch of the product with unscaled segments (after f64_dot1's
      // unscaled intermediates); the tiles apply c(member, term) themselves
     make_tiles(sb->f64_pdot2, phase2_outs(sb, fw, toff_f, Tm, false, true), sb->batch);
     upload_dot_lists(sb, number_segments(sb->f64_pdot2, sb->f64_pdot2.h_tiles), sb->d_pdot_ptr, sb->d_pdot_idx,
-                     sb->d_pdot_partial);
+                     sb->d_pdot_partial, &slab);
   }
   for (TaskListF64* tl : {&sb->f64_fwd1, &sb->f64_fwd2, &sb->f64_dot1, &sb->f64_dot2, &sb->f64_bwd1, &sb->f64_bwd2,
                           &sb->f64_pdot2})
-    finish(*tl);
+    finish(*tl, slab);
 }
 
 // ------------------------------------------------------------- products
@@ -532,18 +613,17 @@ void lz_free(dmrg_sb* sb) {
       sb->lz_graphs[i] = nullptr;
       sb->lz_graph_key[i] = 0;
     }
-  for (double* p : {sb->lz_V, sb->lz_w, sb->lz_vcur, sb->lz_partial, sb->lz_h, sb->lz_npart, sb->lz_ab, sb->lz_s,
-                    sb->lz_out, sb->rf_q, sb->rf_sc, sb->rf_diag, sb->rf_part})
-    if (p) cudaFree(p);
-  for (float* p : {sb->rf_res, sb->rf_p, sb->rf_hp, sb->rf_t, sb->rf_psi32, sb->rf_minv})
-    if (p) cudaFree(p);
-  if (sb->lz_ctl) cudaFree(sb->lz_ctl);
-  if (sb->lz_gate) cudaFree(sb->lz_gate);
-  if (sb->rf_ctl) cudaFree(sb->rf_ctl);
+  for (void* p : std::initializer_list<void*>{sb->lz_V, sb->lz_w, sb->lz_vcur, sb->lz_partial, sb->lz_h, sb->lz_npart,
+                                              sb->lz_ab, sb->lz_s, sb->lz_out, sb->rf_q, sb->rf_sc, sb->rf_diag,
+                                              sb->rf_part, sb->rf_res, sb->rf_p, sb->rf_hp, sb->rf_t, sb->rf_psi32,
+                                              sb->rf_minv, sb->lz_ctl, sb->lz_gate, sb->rf_ctl})
+    dfree(sb, p);
+  if (sb->lz_slab) cudaFree(sb->lz_slab);
+  sb->lz_slab = nullptr;
   sb->rf_q = sb->rf_sc = sb->rf_diag = sb->rf_part = nullptr;
   sb->rf_res = sb->rf_p = sb->rf_hp = sb->rf_t = sb->rf_psi32 = sb->rf_minv = nullptr;
   sb->rf_ctl = nullptr;
-  if (sb->h_ctl) cudaFreeHost(sb->h_ctl);
+  delete[] sb->h_ctl;
   sb->lz_V = sb->lz_w = sb->lz_vcur = sb->lz_partial = sb->lz_h = sb->lz_npart = sb->lz_ab = sb->lz_s =
       sb->lz_out = nullptr;
   sb->lz_ctl = sb->lz_gate = nullptr;
@@ -556,34 +636,32 @@ void lz_alloc(dmrg_sb* sb, int cap) {
   lz_free(sb);
   const int64_t D = sb->D, B = sb->batch;
   sb->lz_nchunk = lz_nchunk(D);
-  sb->lz_V = dalloc<double>((size_t)(cap * B * D));
-  sb->lz_w = dalloc<double>((size_t)(B * D));
-  sb->lz_vcur = dalloc<double>((size_t)(B * D));
+  Slab slab;
+  slab.array(sb->lz_V, (size_t)(cap * B * D));
+  slab.array(sb->lz_w, (size_t)(B * D));
+  slab.array(sb->lz_vcur, (size_t)(B * D));
   // per-chunk partials of the vector kernels, or per-warp dot partials of every Krylov row
-  sb->lz_partial = dalloc<double>((size_t)B * std::max(sb->lz_nchunk, lz_dot_nparts(sb->D)) * cap);
-  sb->lz_h = dalloc<double>((size_t)(3 * B * cap));
-  sb->lz_npart = dalloc<double>((size_t)(3 * B * sb->lz_nchunk));
-  sb->lz_gate = dalloc<int32_t>((size_t)(2 * B));  // the gates, then the block counts of k_norm_gate
-  CK(cudaMemset(sb->lz_gate, 0, sizeof(int32_t) * 2 * B));
-  sb->lz_ab = dalloc<double>((size_t)(2 * B * cap));
-  sb->lz_s = dalloc<double>((size_t)(B * cap));
-  sb->lz_out = dalloc<double>((size_t)(4 * B + 1));
-  sb->lz_ctl = dalloc<int32_t>((size_t)lz_ctl_words(B));
-  void* hp = nullptr;
-  CK(cudaMallocHost(&hp, sizeof(int32_t) * (LZ_CTL_MEMBER + 2 * B)));
-  sb->h_ctl = static_cast<int32_t*>(hp);
-  CK(cudaMemset(sb->lz_ab, 0, sizeof(double) * 2 * B * cap));
-  sb->rf_res = dalloc<float>((size_t)(B * D));
-  sb->rf_p = dalloc<float>((size_t)(B * D));
-  sb->rf_q = dalloc<double>((size_t)(B * D));
-  sb->rf_hp = dalloc<float>((size_t)(B * D));
-  sb->rf_t = dalloc<float>((size_t)(B * D));
-  sb->rf_psi32 = dalloc<float>((size_t)(B * D));
-  sb->rf_sc = dalloc<double>((size_t)(RF_NSC * B + 2));
-  sb->rf_ctl = dalloc<int32_t>((size_t)(2 * B + 2));
-  sb->rf_diag = dalloc<double>((size_t)(B * D));
-  sb->rf_minv = dalloc<float>((size_t)(B * D));
-  sb->rf_part = dalloc<double>((size_t)(4 * B * sb->lz_nchunk));
+  slab.array(sb->lz_partial, (size_t)B * std::max(sb->lz_nchunk, lz_dot_nparts(sb->D)) * cap);
+  slab.array(sb->lz_h, (size_t)(3 * B * cap));
+  slab.array(sb->lz_npart, (size_t)(3 * B * sb->lz_nchunk));
+  slab.array(sb->lz_gate, std::vector<int32_t>((size_t)(2 * B), 0));  // the gates, then the block counts of k_norm_gate
+  slab.array(sb->lz_ab, std::vector<double>((size_t)(2 * B * cap), 0.0));
+  slab.array(sb->lz_s, (size_t)(B * cap));
+  slab.array(sb->lz_out, (size_t)(4 * B + 1));
+  slab.array(sb->lz_ctl, (size_t)lz_ctl_words(B));
+  sb->h_ctl = new int32_t[LZ_CTL_MEMBER + 2 * B]();
+  slab.array(sb->rf_res, (size_t)(B * D));
+  slab.array(sb->rf_p, (size_t)(B * D));
+  slab.array(sb->rf_q, (size_t)(B * D));
+  slab.array(sb->rf_hp, (size_t)(B * D));
+  slab.array(sb->rf_t, (size_t)(B * D));
+  slab.array(sb->rf_psi32, (size_t)(B * D));
+  slab.array(sb->rf_sc, (size_t)(RF_NSC * B + 2));
+  slab.array(sb->rf_ctl, (size_t)(2 * B + 2));
+  slab.array(sb->rf_diag, (size_t)(B * D));
+  slab.array(sb->rf_minv, (size_t)(B * D));
+  slab.array(sb->rf_part, (size_t)(4 * B * sb->lz_nchunk));
+  slab.make(&sb->lz_slab, &sb->lz_slab_bytes);
   sb->lz_cap = cap;
 }
 
@@ -665,6 +743,19 @@ cudaGraphExec_t lz_graph(dmrg_sb* sb, int prec, int K) {
   return ge;
 }
 
+// Whether K captured iterations pay at once: capturing and instantiating a
+// graph costs some 0.4 ms of host time, as much as a whole short solve, so the
+// first solve of a kind on a superblock (the only one, in a DMRG step) launches
+// its first iterations directly (LZ_DIRECT_ITERS of them: a direct one costs
+// the GPU about 12 us more) and the graph is made if it needs more.
+constexpr int LZ_DIRECT_ITERS = 32;
+bool graph_pays(dmrg_sb* sb, int key) {
+  for (int k : sb->lz_used)
+    if (k == key) return true;
+  sb->lz_used.push_back(key);
+  return false;
+}
+
 struct LzRun {
   std::vector<int32_t> code, iters, restarts;
   std::vector<double> theta, resid;
@@ -702,10 +793,13 @@ LzRun lz_run(dmrg_sb* sb, const double* psi0, double* psi_out, int prec, double 
   CK(cudaMemcpyAsync(sb->lz_out + 4 * B, &tol, sizeof(double), cudaMemcpyHostToDevice, st));
   CK(cudaStreamSynchronize(st));  // host vectors above are stack memory
   const int K = std::max(1, std::min(graph_iters, max_iter));
-  cudaGraphExec_t ge = lz_graph(sb, prec, K);
+  cudaGraphExec_t ge = graph_pays(sb, 1 + prec * 1024 + K) ? lz_graph(sb, prec, K) : nullptr;
   int launched = 0;
   for (;;) {
-    CK(cudaGraphLaunch(ge, st));
+    if (!ge && launched >= LZ_DIRECT_ITERS) ge = lz_graph(sb, prec, K);
+    if (ge) CK(cudaGraphLaunch(ge, st));
+    else
+      for (int k = 0; k < K; ++k) lz_enqueue_iteration(sb, prec, st);
     launched += K;
     CK(cudaMemcpyAsync(sb->h_ctl, sb->lz_ctl, sizeof(int32_t) * (LZ_CTL_MEMBER + 2 * B), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
@@ -871,6 +965,7 @@ RfRun rf_solve(dmrg_sb* sb, double* psi, int prec, int rprec, double tol, int ma
   std::vector<int32_t> hctl(2 * B + 2, 0), mask(B, 0);
   std::vector<uint8_t> conv(B, 0);
   const int Kg = std::max(1, K);
+  const bool graphs = graph_pays(sb, (1 << 20) + 1 + prec * 1024 + Kg);
   rf_launch_diag(sb->d_dg, sb->d_dg_terms, (int)sb->dg_terms.size(), sb->d_coeffs, sb->n_terms, sb->rf_diag, D, B,
                  st);
   ++r.launches;
@@ -939,10 +1034,13 @@ RfRun rf_solve(dmrg_sb* sb, double* psi, int prec, int rprec, double tol, int ma
     CK(cudaMemcpyAsync(sb->rf_ctl, hctl.data(), sizeof(int32_t) * (2 * B + 2), cudaMemcpyHostToDevice, st));
     CK(cudaMemcpyAsync(sb->rf_sc + RF_NSC * B, &eps, sizeof(double), cudaMemcpyHostToDevice, st));
     CK(cudaStreamSynchronize(st));
-    cudaGraphExec_t ge = rf_graph(sb, prec, Kg);
+    cudaGraphExec_t ge = graphs ? rf_graph(sb, prec, Kg) : nullptr;
     int launched = 0;
     for (;;) {
-      CK(cudaGraphLaunch(ge, st));
+      if (!ge && launched >= LZ_DIRECT_ITERS) ge = rf_graph(sb, prec, Kg);
+      if (ge) CK(cudaGraphLaunch(ge, st));
+      else
+        for (int k = 0; k < Kg; ++k) rf_enqueue_inner(sb, prec, st);
       launched += Kg;
       r.launches += (int64_t)Kg * (RF_KERNELS_PER_ITER + matvec_launches(sb, prec));
       int32_t stop = 0;
@@ -979,7 +1077,7 @@ dmrg_status code_to_status(int code) {
   }
 }
 
-void validate_and_copy(dmrg_sb* sb, const dmrg_sb_desc* d, int32_t batch) {
+void validate_and_copy(dmrg_sb* sb, const dmrg_sb_desc* d, int32_t batch, Slab& slab) {
   if (!d) throw Invalid{"null descriptor"};
   if (batch < 1) throw Invalid{"batch must be >= 1"};
   if (d->n_sectors < 0 || d->n_terms < 1 || d->n_pairs < 0) throw Invalid{"bad counts"};
@@ -1071,8 +1169,7 @@ void validate_and_copy(dmrg_sb* sb, const dmrg_sb_desc* d, int32_t batch) {
     }
     sb->pairs.push_back(h);
   }
-  sb->d_ops = dalloc<double>((size_t)std::max<int64_t>(ops, 1));
-  if (ops) CK(cudaMemcpy(sb->d_ops, host.data(), ops * sizeof(double), cudaMemcpyHostToDevice));
+  slab.array(sb->d_ops, host);
   // diagonal of every term with diagonal blocks (s_out == s_in): the
   // refinement's preconditioner sums them with the member's coefficients
   {
@@ -1096,16 +1193,15 @@ void validate_and_copy(dmrg_sb* sb, const dmrg_sb_desc* d, int32_t batch) {
       }
     }
     if (!sb->dg_terms.empty()) {
-      upload(sb->d_dg, dg);
-      upload(sb->d_dg_terms, sb->dg_terms);
+      slab.array(sb->d_dg, dg);
+      slab.array(sb->d_dg_terms, sb->dg_terms);
     }
   }
   sb->h_ops = std::move(host);
-  sb->d_tc_err = dalloc<int32_t>(1);
-  CK(cudaMemset(sb->d_tc_err, 0, sizeof(int32_t)));
-  upload(sb->d_coeffs, sb->coeffs);
-  sb->d_scratch = dalloc<double>((size_t)(4 * batch + 16));
-  sb->d_red = dalloc<double>((size_t)batch * lz_nchunk(sb->D));
+  slab.array(sb->d_tc_err, std::vector<int32_t>(1, 0));
+  slab.array(sb->d_coeffs, sb->coeffs);
+  slab.array(sb->d_scratch, (size_t)(4 * batch + 16));
+  slab.array(sb->d_red, (size_t)batch * lz_nchunk(sb->D));
 }
 
 void destroy(dmrg_sb* sb) {
@@ -1114,17 +1210,14 @@ void destroy(dmrg_sb* sb) {
   tc_free(sb);
   for (TaskListF64* tl : {&sb->f64_fwd1, &sb->f64_fwd2, &sb->f64_dot1, &sb->f64_dot2, &sb->f64_bwd1, &sb->f64_bwd2,
                           &sb->f64_pdot2})
-    free_tl(*tl);
-  for (double* p : {sb->d_coeffs, sb->d_ops, sb->d_T, sb->d_dot_partial, sb->d_scratch, sb->d_red, sb->d_dg,
-                    sb->d_pdot_partial, sb->d_pdot_partial_df, sb->d_ops_df, sb->d_x_df})
-    if (p) cudaFree(p);
-  for (int32_t* p : {sb->d_pdot_ptr, sb->d_pdot_idx, sb->d_pdot_ptr_df, sb->d_pdot_idx_df})
-    if (p) cudaFree(p);
-  if (sb->d_dg_terms) cudaFree(sb->d_dg_terms);
-  if (sb->d_tc_err) cudaFree(sb->d_tc_err);
+    free_tl(sb, *tl);
+  for (void* p : std::initializer_list<void*>{
+           sb->d_coeffs, sb->d_ops, sb->d_T, sb->d_dot_partial, sb->d_scratch, sb->d_red, sb->d_dg, sb->d_pdot_partial,
+           sb->d_pdot_partial_df, sb->d_ops_df, sb->d_x_df, sb->d_pdot_ptr, sb->d_pdot_idx, sb->d_pdot_ptr_df,
+           sb->d_pdot_idx_df, sb->d_dg_terms, sb->d_tc_err, sb->d_dot_red_ptr, sb->d_dot_red_idx})
+    dfree(sb, p);
+  if (sb->slab) cudaFree(sb->slab);
   if (sb->h_coeffs_pinned) cudaFreeHost(sb->h_coeffs_pinned);
-  if (sb->d_dot_red_ptr) cudaFree(sb->d_dot_red_ptr);
-  if (sb->d_dot_red_idx) cudaFree(sb->d_dot_red_idx);
   delete sb;
 }
 
@@ -1139,8 +1232,10 @@ dmrg_status dmrg_create_superblock(const dmrg_sb_desc* d, int32_t batch, dmrg_sb
   dmrg_sb* sb = new (std::nothrow) dmrg_sb();
   if (!sb) return DMRG_ENOMEM;
   const dmrg_status st = guard(sb, [&] {
-    validate_and_copy(sb, d, batch);
-    build_f64_tasks(sb);
+    Slab slab;
+    validate_and_copy(sb, d, batch, slab);
+    build_f64_tasks(sb, slab);
+    slab.make(&sb->slab, &sb->slab_bytes);
     tc_build(sb);
     sb->h_ops.clear();
     sb->h_ops.shrink_to_fit();
@@ -1180,7 +1275,8 @@ dmrg_status dmrg_set_coeffs(dmrg_sb* sb, const double* coeffs, void* stream) {
   return guard(sb, [&] {
     cudaStream_t st = (cudaStream_t)stream;
     const size_t n = (size_t)sb->batch * sb->n_terms;
-    sb->coeffs.assign(coeffs, coeffs + n);
+    // the table that is set already (written and waited for by the call that set it)
+    if (memcmp(sb->coeffs.data(), coeffs, n * sizeof(double)) == 0) return DMRG_OK;
     // through a pinned staging copy, ordered on the caller's stream after the
     // products already queued there (which read the old table); the stream is
     // synchronised so that the staging copy is free for the next call
@@ -1192,6 +1288,7 @@ dmrg_status dmrg_set_coeffs(dmrg_sb* sb, const double* coeffs, void* stream) {
     memcpy(sb->h_coeffs_pinned, coeffs, n * sizeof(double));
     CK(cudaMemcpyAsync(sb->d_coeffs, sb->h_coeffs_pinned, n * sizeof(double), cudaMemcpyHostToDevice, st));
     CK(cudaStreamSynchronize(st));
+    sb->coeffs.assign(coeffs, coeffs + n);
     if (tc_set_coeffs(sb))  // tensor-core panels with folded coefficients were rebuilt
       for (int i = 0; i < 8; ++i)
         if (sb->lz_graphs[i]) {

@@ -50,32 +50,45 @@ struct Bad {
   std::string msg;
 };
 
-// owned device array of doubles
-struct DBuf {
-  double* p = nullptr;
-  size_t n = 0;
-  explicit DBuf(size_t n_) {
-    n = std::max<size_t>(n_, 1);
-    SYS_CK(cudaMalloc(&p, n * sizeof(double)));
-  }
-  ~DBuf() {
-    if (p) cudaFree(p);
-  }
-  DBuf(const DBuf&) = delete;
-  DBuf& operator=(const DBuf&) = delete;
-};
-using DBufP = std::shared_ptr<DBuf>;
-
+// owned device array of a plain type, from the run's pool (the calling
+// thread's; without one from the driver)
 template <class T>
-struct DArr {  // owned device array of a plain type
+struct DArr {
   T* p = nullptr;
-  explicit DArr(size_t n) { SYS_CK(cudaMalloc(&p, std::max<size_t>(n, 1) * sizeof(T))); }
+  size_t n = 0;
+  std::shared_ptr<DevPool> pool;
+  explicit DArr(size_t n_);
   ~DArr() {
-    if (p) cudaFree(p);
+    if (!p) return;
+    if (pool) pool->put(p, n * sizeof(T));
+    else cudaFree(p);
   }
   DArr(const DArr&) = delete;
   DArr& operator=(const DArr&) = delete;
 };
+
+// the pool of the run whose call this thread is in
+thread_local std::shared_ptr<DevPool> t_pool;
+struct PoolScope {
+  std::shared_ptr<DevPool> old_owner;
+  DevPool* old;
+  explicit PoolScope(std::shared_ptr<DevPool> p) : old_owner(std::move(t_pool)) {
+    t_pool = std::move(p);
+    old = DevPool::set_current(t_pool.get());
+  }
+  ~PoolScope() {
+    DevPool::set_current(old);
+    t_pool = std::move(old_owner);
+  }
+};
+
+template <class T>
+DArr<T>::DArr(size_t n_) : n(std::max<size_t>(n_, 1)), pool(t_pool) {
+  if (pool) p = static_cast<T*>(pool->get(n * sizeof(T)));
+  else SYS_CK(cudaMalloc(&p, n * sizeof(T)));
+}
+using DBuf = DArr<double>;
+using DBufP = std::shared_ptr<DBuf>;
 
 struct Basis {
   std::vector<int64_t> q;
@@ -673,34 +686,44 @@ double host_ms() {
   return std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now().time_since_epoch()).count();
 }
 
-// Keep the m most probable states of the grown block G (side S: rows of the
-// target blocks, rho = Psi Psi^T; side E: columns, rho = Psi^T Psi) and carry
-// H and the operators of end distance >= keep_from to the new basis.
-TruncOut truncate(const Model& M, const Blk& G, bool sideS, const SbView& V, const double* psi, int m,
-                  double tie_tol, int keep_from, cudaStream_t st) {
+// The density matrices of one side and their eigensolves: the arrays, and the
+// jobs that fill them.
+struct Densities {
+  std::vector<int64_t> roff, coff, woff;
+  std::unique_ptr<DBuf> rho, lam, work;
+  DBufP Vv;
+};
+
+// The density matrices of the grown block G (side S: rows of the target
+// blocks, rho = Psi Psi^T; side E: columns, rho = Psi^T Psi).  The jobs are
+// appended, so that both sides of a step share the launches.
+Densities densities(const Blk& G, bool sideS, const SbView& V, const double* psi, std::vector<GemmJob>& gj,
+                    std::vector<EigJob>& ej, cudaStream_t st) {
   const Basis& b = G.bs;
   const int nz = b.size();
-  std::vector<int64_t> roff(nz + 1, 0), coff(nz + 1, 0), woff(nz + 1, 0);
+  Densities d;
+  d.roff.assign(nz + 1, 0);
+  d.coff.assign(nz + 1, 0);
+  d.woff.assign(nz + 1, 0);
+  std::vector<int64_t>&roff = d.roff, &coff = d.coff, &woff = d.woff;
   for (int z = 0; z < nz; ++z) {
     const int64_t n = b.dim[z];
     roff[z + 1] = roff[z] + n * n;
     coff[z + 1] = coff[z] + n;
     woff[z + 1] = woff[z] + (n > EIG_SMEM_MAX_N ? 2 * n * (n + 1) : 0);
   }
-  const int64_t ncand = coff[nz];
-  const double t0 = host_ms();
-  DBuf rho((size_t)roff[nz]);
-  auto Vv = std::make_shared<DBuf>((size_t)roff[nz]);
-  DBuf lam((size_t)ncand), work((size_t)std::max<int64_t>(woff[nz], 1));
-  SYS_CK(cudaMemsetAsync(rho.p, 0, roff[nz] * sizeof(double), st));
-  std::vector<GemmJob> gj;
+  d.rho = std::make_unique<DBuf>((size_t)roff[nz]);
+  d.Vv = std::make_shared<DBuf>((size_t)roff[nz]);
+  d.lam = std::make_unique<DBuf>((size_t)coff[nz]);
+  d.work = std::make_unique<DBuf>((size_t)std::max<int64_t>(woff[nz], 1));
+  SYS_CK(cudaMemsetAsync(d.rho->p, 0, roff[nz] * sizeof(double), st));
   for (int z = 0; z < nz; ++z) {
     const int s = sideS ? V.tsecS[z] : V.tsecE[z];
     if (s < 0) continue;
     const int r = V.r[s], c = V.c[s];
     GemmJob j{};
     j.A = j.B = psi + V.off[s];
-    j.C = rho.p + roff[z];
+    j.C = d.rho->p + roff[z];
     j.alpha = 1.0;
     j.beta = 0.0;
     j.lda = j.ldb = c;
@@ -719,19 +742,27 @@ TruncOut truncate(const Model& M, const Blk& G, bool sideS, const SbView& V, con
     }
     gj.push_back(j);
   }
-  launch_gemm(gj, st);
-  std::vector<EigJob> ej;
   for (int z = 0; z < nz; ++z) {
     EigJob j{};
-    j.A = rho.p + roff[z];
-    j.V = Vv->p + roff[z];
-    j.w = lam.p + coff[z];
-    j.work = b.dim[z] > EIG_SMEM_MAX_N ? work.p + woff[z] : nullptr;
+    j.A = d.rho->p + roff[z];
+    j.V = d.Vv->p + roff[z];
+    j.w = d.lam->p + coff[z];
+    j.work = b.dim[z] > EIG_SMEM_MAX_N ? d.work->p + woff[z] : nullptr;
     j.n = b.dim[z];
     ej.push_back(j);
   }
-  launch_eig(ej, st);
-  SYS_CK(cudaStreamSynchronize(st));
+  return d;
+}
+
+// Keep the m most probable states of the grown block G, whose density matrices
+// have been diagonalised (d, enqueued on st), and carry H and the operators of
+// end distance >= keep_from to the new basis.
+TruncOut truncate(const Blk& G, const Densities& d, int m, double tie_tol, int keep_from, cudaStream_t st) {
+  const Basis& b = G.bs;
+  const int nz = b.size();
+  const std::vector<int64_t>&roff = d.roff, &coff = d.coff;
+  const int64_t ncand = coff[nz];
+  const DBufP& Vv = d.Vv;
   const double t1 = host_ms();
   // global selection
   std::vector<int32_t> hsec((size_t)ncand), hidx((size_t)ncand);
@@ -745,7 +776,7 @@ TruncOut truncate(const Model& M, const Blk& G, bool sideS, const SbView& V, con
   SYS_CK(cudaMemcpyAsync(dsec.p, hsec.data(), ncand * sizeof(int32_t), cudaMemcpyHostToDevice, st));
   SYS_CK(cudaMemcpyAsync(didx.p, hidx.data(), ncand * sizeof(int32_t), cudaMemcpyHostToDevice, st));
   const int meff = (int)std::min<int64_t>(m, ncand);
-  launch_select(lam.p, dsec.p, didx.p, (int32_t)ncand, meff, tie_tol, dkeep.p, stats.p, scr.p, nullptr, st);
+  launch_select(d.lam->p, dsec.p, didx.p, (int32_t)ncand, meff, tie_tol, dkeep.p, stats.p, scr.p, nullptr, st);
   std::vector<int32_t> keep((size_t)ncand);
   double hst[2] = {0.0, 0.0};
   SYS_CK(cudaMemcpyAsync(keep.data(), dkeep.p, ncand * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
@@ -831,13 +862,39 @@ TruncOut truncate(const Model& M, const Blk& G, bool sideS, const SbView& V, con
   SYS_CK(cudaStreamSynchronize(st));
   N->trunc = tr;
   TruncOut out;
-  out.ms_eig = t1 - t0;
   out.ms_select = t2 - t1;
   out.ms_transform = host_ms() - t2;
   out.blk = N;
   out.eps = std::max(0.0, hst[0]);
   out.gap = hst[1];
   out.kept = meff;
+  return out;
+}
+
+// The truncation of one or both grown blocks of a step: all density matrices in
+// one launch, all eigensolves in one (two blocks' worth of small matrices take
+// as long as one's), then the choice and the change of basis per block.
+struct TruncSide {
+  const Blk* G;
+  bool sideS;
+  int keep_from;
+};
+std::vector<TruncOut> truncate_sides(const std::vector<TruncSide>& sides, const SbView& V, const double* psi, int m,
+                                     double tie_tol, cudaStream_t st) {
+  const double t0 = host_ms();
+  std::vector<GemmJob> gj;
+  std::vector<EigJob> ej;
+  std::vector<Densities> ds;
+  for (const TruncSide& s : sides) ds.push_back(densities(*s.G, s.sideS, V, psi, gj, ej, st));
+  launch_gemm(gj, st);
+  launch_eig(ej, st);
+  SYS_CK(cudaStreamSynchronize(st));
+  const double ms_eig = host_ms() - t0;
+  std::vector<TruncOut> out;
+  for (size_t i = 0; i < sides.size(); ++i) {
+    out.push_back(truncate(*sides[i].G, ds[i], m, tie_tol, sides[i].keep_from, st));
+    out.back().ms_eig = ms_eig / (double)sides.size();
+  }
   return out;
 }
 
@@ -1085,6 +1142,7 @@ struct dmrg_sys {
   std::vector<double> psi_host;
   int last_nS = 0, last_L = 0;
   Prev prev;  // the previous step, for the wavefunction transformation
+  std::shared_ptr<DevPool> pool = std::make_shared<DevPool>();
   std::string err;
 };
 
@@ -1174,6 +1232,7 @@ int max_dim(const Blk& b) {
 
 template <class F>
 dmrg_status sys_guard(dmrg_sys* sys, F&& fn) {
+  const PoolScope scope(sys ? sys->pool : nullptr);
   try {
     return fn();
   } catch (const Bad& b) {
@@ -1249,8 +1308,10 @@ dmrg_status dmrg_sys_infinite(dmrg_sys* sys, dmrg_step_info* steps, int32_t* n_s
       solve_step(sys, Sp, Ep, Lk, 0, info, nullptr, st);
       const double* psi = sys->prev.psi->p;
       const double t2 = now_ms();
-      TruncOut ts = truncate(M, *Sp, true, sys->view, psi, sys->m, sys->opts.tie_tol, Sp->n - M.reach, st);
-      TruncOut te = truncate(M, *Ep, false, sys->view, psi, sys->m, sys->opts.tie_tol, Ep->n - M.reach, st);
+      const std::vector<TruncOut> both =
+          truncate_sides({{Sp.get(), true, Sp->n - M.reach}, {Ep.get(), false, Ep->n - M.reach}}, sys->view, psi, sys->m,
+                         sys->opts.tie_tol, st);
+      const TruncOut &ts = both[0], &te = both[1];
       info.ms_truncate = now_ms() - t2;
       info.ms_eig = ts.ms_eig + te.ms_eig;
       info.ms_select = ts.ms_select + te.ms_select;
@@ -1330,7 +1391,8 @@ dmrg_status dmrg_sys_sweeps(dmrg_sys* sys, int32_t n_sweeps, dmrg_step_info* ste
       const double t2 = now_ms();
       info.max_sector = dir > 0 ? max_dim(*Sp) : max_dim(*Ep);
       if (dir > 0) {
-        TruncOut ts = truncate(M, *Sp, true, sys->view, psi, sys->m, sys->opts.tie_tol, Sp->n - M.reach, st);
+        const TruncOut ts =
+            truncate_sides({{Sp.get(), true, Sp->n - M.reach}}, sys->view, psi, sys->m, sys->opts.tie_tol, st)[0];
         sys->left[Sp->n] = ts.blk;
         info.ms_eig = ts.ms_eig;
         info.ms_select = ts.ms_select;
@@ -1339,7 +1401,8 @@ dmrg_status dmrg_sys_sweeps(dmrg_sys* sys, int32_t n_sweeps, dmrg_step_info* ste
         info.gap_S = ts.gap;
         info.kept_S = ts.kept;
       } else {
-        TruncOut te = truncate(M, *Ep, false, sys->view, psi, sys->m, sys->opts.tie_tol, Ep->n - M.reach, st);
+        const TruncOut te =
+            truncate_sides({{Ep.get(), false, Ep->n - M.reach}}, sys->view, psi, sys->m, sys->opts.tie_tol, st)[0];
         sys->right[Ep->n] = te.blk;
         info.ms_eig = te.ms_eig;
         info.ms_select = te.ms_select;

@@ -141,7 +141,7 @@ struct dmrg_sb {
   double* lz_s = nullptr;        // Ritz vector [batch][lz_cap]
   double* lz_out = nullptr;      // per member: theta, resid
   int32_t* lz_ctl = nullptr;     // device control words
-  int32_t* h_ctl = nullptr;      // pinned host mirror
+  int32_t* h_ctl = nullptr;      // host mirror
   int32_t lz_nchunk = 0;
   // float64 refinement (Newton step with mixed CG) buffers, allocated with Lanczos
   float* rf_res = nullptr;       // [batch][D] inner CG vectors (float32)
@@ -161,6 +161,10 @@ struct dmrg_sb {
   double* d_dg = nullptr;
   void* lz_graphs[8] = {};       // cached cudaGraphExec_t per (prec, K) slot
   int32_t lz_graph_key[8] = {};
+  std::vector<int32_t> lz_used;  // keys of the solves that have run once (their graphs are made at the second)
+  // the allocations that hold the small arrays of the superblock and of its solver buffers
+  char *slab = nullptr, *lz_slab = nullptr;
+  size_t slab_bytes = 0, lz_slab_bytes = 0;
 
   void* tc = nullptr;            // tensor-core path state (matvec_tc.cu)
   int32_t* d_tc_err = nullptr;   // set by a tensor-core kernel whose bounded wait gave up
