@@ -90,7 +90,7 @@ __device__ __forceinline__ int first_row(int j, int win) { return win ? max(0, j
 // reduction.
 // GB300 issues float64 at 1/64 of the float32 rate, so the reduction must not
 // cost more float64 work than the dot products: every thread keeps
-// LZ_DOT_EPT elements of w in registers, takes 8 rows at a time, and the 8
+// LZ_DOT_EPT elements of w in registers, takes RG = 8 rows at a time, and the 8
 // row sums are reduced across the warp by a butterfly that halves the values
 // per lane at each step (4+2+1+1+1 shuffle-adds for 8 rows, not 8 x 5).
 // With h_pre != NULL the previous pass's update (the three-term step,
@@ -99,12 +99,13 @@ __device__ __forceinline__ int first_row(int j, int win) { return win ? max(0, j
 // one sweep instead of an update sweep followed by a dot sweep (blocks of
 // LZ_THREADS, one row of blocks).
 // The warps of a chunk are independent: a short vector, which would leave most
-// SMs without a block, takes blocks of one warp and splits the groups of 8
-// rows over blockIdx.z (the update then has a kernel of its own,
-// k_update_local); each partial is the same sum either way.  Float64 pass B of
-// the 32-site chain at m = 200 (D = 13 596, 4 chunks, j = 40 on average): 50 us
-// with the update inside, now 3.9 + 9 us.
-template <bool PAIR>
+// SMs without a block, takes blocks of one warp and splits the groups of rows
+// over blockIdx.z, two rows each in float64 where that makes more warps (the
+// update then has a kernel of its own, k_update_local); each partial is the
+// same sum either way.  Float64 pass B of the 32-site chain at m = 200 (D = 13 596,
+// 4 chunks, j = 40): 50 us with the update inside, 4.1 + 11.4 us with groups of
+// 8 rows, 4.1 + 3.9 us with two.
+template <bool PAIR, int RG>
 __global__ void __launch_bounds__(LZ_THREADS, PAIR ? 2 : 3)
 k_multidot(const double* __restrict__ V, double* __restrict__ w, double* __restrict__ partial,
            const int32_t* __restrict__ ctl, int64_t D, int batch, int cap, int nchunk, int win,
@@ -116,7 +117,7 @@ k_multidot(const double* __restrict__ V, double* __restrict__ w, double* __restr
   const int lane = threadIdx.x & 31;
   const int vw = blockIdx.x * (int)(blockDim.x >> 5) + (int)(threadIdx.x >> 5);  // warp of the member
   const int chunk = vw / LZ_DOT_WARPS, wid = vw % LZ_DOT_WARPS;
-  const int row0 = first_row(j, win) + 8 * (int)blockIdx.z;
+  const int row0 = first_row(j, win) + RG * (int)blockIdx.z;
   if (row0 > j) return;
   double wv[LZ_DOT_EPT];  // w (float64 basis)
   float2 wf[LZ_DOT_EPT];  // w split into double-float pairs (pair basis)
@@ -156,12 +157,12 @@ k_multidot(const double* __restrict__ V, double* __restrict__ w, double* __restr
     }
   }
   const bool full = base + (LZ_DOT_EPT - 1) * LZ_THREADS < D;
-  for (int i0 = row0; i0 <= j; i0 += 8 * (int)gridDim.z) {
-    // per-thread sums of 8 rows: float64, or double-float pairs (pair basis)
-    double p[8];
-    float2 p2[8];
+  for (int i0 = row0; i0 <= j; i0 += RG * (int)gridDim.z) {
+    // per-thread sums of RG rows: float64, or double-float pairs (pair basis)
+    double p[RG];
+    float2 p2[RG];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
+    for (int q = 0; q < RG; ++q) {
       const int i = i0 + q;
       const double* v = V + ((int64_t)i * batch + b) * D + base;
       if (PAIR) {  // double-float dot of the stored pairs with the split w
@@ -191,58 +192,40 @@ k_multidot(const double* __restrict__ V, double* __restrict__ w, double* __restr
         }
       }
     }
-    // butterfly: after the step with offset 16 a lane holds 4 partial rows,
-    // after 8 two rows, after 4 one row; offsets 2 and 1 finish that row.
-    // The pair basis adds pairs (float32 work: float64 issues at 1/64 of the
-    // float32 rate, and float64 adds here had cost a third of the sweep).
-    const int row = ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
-    if (PAIR) {
+    // butterfly: every step halves the rows a lane holds (each half of the
+    // lanes keeps half of them) until it holds one; the remaining offsets
+    // finish that row.  The pair basis adds pairs (float32 work: float64 issues
+    // at 1/64 of the float32 rate, and float64 adds here had cost a third of
+    // the sweep).
+    int row = 0;
 #pragma unroll
-      for (int h = 4; h >= 1; h >>= 1) {  // offsets 16, 8, 4: halve the rows held
-        const int off = 4 * h;
+    for (int off = 16, held = RG; off >= 1; off >>= 1) {
+      if (held > 1) {
+        held >>= 1;
         const bool up = lane & off;
+        row = row * 2 + (up ? 1 : 0);
 #pragma unroll
-        for (int q = 0; q < h; ++q) {
-          const float2 send = up ? p2[q] : p2[q + h];
-          const float2 keep = up ? p2[q + h] : p2[q];
-          const float2 got = make_float2(__shfl_xor_sync(0xffffffffu, send.x, off),
-                                         __shfl_xor_sync(0xffffffffu, send.y, off));
-          p2[q] = df_add(keep, got);
+        for (int q = 0; q < RG / 2; ++q) {
+          if (q >= held) break;
+          if (PAIR) {
+            const float2 send = up ? p2[q] : p2[q + held];
+            const float2 keep = up ? p2[q + held] : p2[q];
+            p2[q] = df_add(keep, make_float2(__shfl_xor_sync(0xffffffffu, send.x, off),
+                                             __shfl_xor_sync(0xffffffffu, send.y, off)));
+          } else {
+            const double send = up ? p[q] : p[q + held];
+            const double keep = up ? p[q + held] : p[q];
+            p[q] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+          }
         }
-      }
-#pragma unroll
-      for (int off = 2; off >= 1; off >>= 1)
+      } else if (PAIR) {
         p2[0] = df_add(p2[0], make_float2(__shfl_xor_sync(0xffffffffu, p2[0].x, off),
                                           __shfl_xor_sync(0xffffffffu, p2[0].y, off)));
-    } else {
-      {
-        const bool up = lane & 16;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const double send = up ? p[q] : p[q + 4];
-          const double keep = up ? p[q + 4] : p[q];
-          p[q] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-        }
+      } else {
+        p[0] += __shfl_xor_sync(0xffffffffu, p[0], off);
       }
-      {
-        const bool up = lane & 8;
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const double send = up ? p[q] : p[q + 2];
-          const double keep = up ? p[q + 2] : p[q];
-          p[q] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-        }
-      }
-      {
-        const bool up = lane & 4;
-        const double send = up ? p[0] : p[1];
-        const double keep = up ? p[1] : p[0];
-        p[0] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
-      }
-      p[0] += __shfl_xor_sync(0xffffffffu, p[0], 2);
-      p[0] += __shfl_xor_sync(0xffffffffu, p[0], 1);
     }
-    if ((lane & 3) == 0 && i0 + row <= j)
+    if ((lane & (32 / RG - 1)) == 0 && i0 + row <= j)
       partial[((int64_t)b * cap + i0 + row) * ((int64_t)nchunk * LZ_DOT_WARPS) + chunk * LZ_DOT_WARPS + wid] =
           PAIR ? df_value(p2[0].x, p2[0].y) : p[0];
   }
@@ -442,7 +425,7 @@ k_multiaxpy(const double* __restrict__ V, double* __restrict__ w, const double* 
     const int64_t d = d0 + e * T;
     wv[e] = d < D ? w[(int64_t)b * D + d] : 0.0;
   }
-#pragma unroll (EPT == 1 ? 8 : 2)
+#pragma unroll (EPT == 1 ? (PAIR ? 8 : 16) : 2)
   for (int i = i0; i <= j; ++i) {
     const double* vi = V + ((int64_t)i * batch + b) * D + d0;
     if (PAIR) {  // sum_i V[i] h[i] in double-float arithmetic
@@ -1254,8 +1237,9 @@ void lz_launch_cfrac(const double* norm2, const double* alpha, const double* bet
   k_cfrac<<<dim3((n_z + 127) / 128, batch), 128, 0, st>>>(norm2, alpha, beta, n, ld, zr, zi, n_z, gr, gi);
 }
 // blocks of a dot pass: LZ_DOT_WARPS warps each (one row of blocks), or for a
-// short vector single warps with the row groups over z, up to about 16 warps per SM
-static void dot_grid(int64_t D, int batch, int cap, dim3& g, int& threads) {
+// short vector single warps with the row groups (rg rows) over z, up to about
+// 16 warps per SM
+static void dot_grid(int64_t D, int batch, int cap, int rg, dim3& g, int& threads) {
   const int nch = lz_dot_nchunk(D);
   if (!lz_short(D, batch)) {
     g = dim3(nch, batch);
@@ -1263,28 +1247,31 @@ static void dot_grid(int64_t D, int batch, int cap, dim3& g, int& threads) {
     return;
   }
   const int warps = nch * LZ_DOT_WARPS;
-  const int z = std::min((cap + 7) / 8, std::max(1, 152 * 16 / (warps * batch)));
+  const int z = std::min((cap + rg - 1) / rg, std::max(1, 152 * 16 / (warps * batch)));
   g = dim3(warps, batch, z);
   threads = 32;
 }
 void lz_launch_multidot(const double* V, double* w, double* partial, const int32_t* ctl, int64_t D,
                         int batch, int cap, int win, const int32_t* gate, cudaStream_t st, const double* h_pre,
                         double* npart_pre, bool pair) {
-  dim3 g(lz_dot_nchunk(D), batch);
+  const int nch = lz_dot_nchunk(D);
+  // two rows per warp while that still leaves every SM at most 16 warps for 64 rows
+  const bool fine = !h_pre && !pair && (int64_t)nch * LZ_DOT_WARPS * batch * 32 <= 152 * 16;
+  dim3 g(nch, batch);
   int threads = LZ_THREADS;
-  if (!h_pre) dot_grid(D, batch, cap, g, threads);
+  if (!h_pre) dot_grid(D, batch, cap, fine ? 2 : 8, g, threads);
   if (pair)
-    k_multidot<true><<<g, threads, 0, st>>>(V, w, partial, ctl, D, batch, cap, lz_dot_nchunk(D), win, gate, h_pre,
-                                            npart_pre);
+    k_multidot<true, 8><<<g, threads, 0, st>>>(V, w, partial, ctl, D, batch, cap, nch, win, gate, h_pre, npart_pre);
+  else if (fine)
+    k_multidot<false, 2><<<g, threads, 0, st>>>(V, w, partial, ctl, D, batch, cap, nch, win, gate, h_pre, npart_pre);
   else
-    k_multidot<false><<<g, threads, 0, st>>>(V, w, partial, ctl, D, batch, cap, lz_dot_nchunk(D), win, gate, h_pre,
-                                             npart_pre);
+    k_multidot<false, 8><<<g, threads, 0, st>>>(V, w, partial, ctl, D, batch, cap, nch, win, gate, h_pre, npart_pre);
 }
 void lz_launch_dots_local(const double* V, const double* w, double* partial, const int32_t* ctl, int64_t D,
                           int batch, int cap, cudaStream_t st, bool pair) {
   dim3 g;
   int threads;
-  dot_grid(D, batch, 1, g, threads);
+  dot_grid(D, batch, 1, 8, g, threads);
   if (pair)
     k_dots_local<true><<<g, threads, 0, st>>>(V, w, partial, ctl, D, batch, cap, lz_dot_nchunk(D));
   else
