@@ -26,9 +26,9 @@
 //
 // Bound: instruction issue (80 % of the slots on wide sectors, 66-73 % on the
 // ladder).  Measured against 64 x 64 tiles of 256 threads: the 32-site chain
-// at m = 1000 472 -> 277 us, 16 sectors 16..512 wide 4.92 -> 4.27 ms, the 2 x 32
-// ladder at m = 1000 (16 members) 3.14 -> 3.17 ms, with the per-term dots 4.21
-// -> 3.68 ms.  Tiles of 32 x 32 (16 sums a thread) were slower: 6.4 ms on the
+// at m = 1000 472 -> 273 us, 16 sectors 16..512 wide 4.92 -> 4.23 ms, the 2 x 32
+// ladder at m = 1000 (16 members) 3.14 -> 3.11 ms, with the per-term dots 4.21
+// -> 3.62 ms.  Tiles of 32 x 32 (16 sums a thread) were slower: 6.4 ms on the
 // wide sectors, too few warps for their registers.
 
 #include <algorithm>

@@ -12,9 +12,9 @@
 //
 // Measured against 64 x 64 tiles of 256 threads with one chunk in flight and
 // the two output groups in launches of their own: one product of the 12-site
-// ladder at m = 60 (2 members) 145 -> 29 us, of the 32-site chain at m = 200
-// 108 -> 29 us, at m = 1000 1429 -> 749 us, of the 2 x 32 ladder at m = 400 (4
-// members) 707 -> 217 us, of 16 sectors 16..512 wide 17.3 -> 14.1 ms (1.14
+// ladder at m = 60 (2 members) 145 -> 26 us, of the 32-site chain at m = 200
+// 108 -> 27 us, at m = 1000 1429 -> 743 us, of the 2 x 32 ladder at m = 400 (4
+// members) 707 -> 212 us, of 16 sectors 16..512 wide 17.3 -> 14.1 ms (1.14
 // TFLOP/s; the float64 unit is 95-97 % busy).
 
 #include "internal.h"
