@@ -32,6 +32,14 @@
 // share their wavefunction operand run as one "pieced" tile: their operator
 // panels side by side along N behind one L tile.
 //
+// A launch ends with its longest block, and an output's chain of K chunks
+// (0.4 us each, nearly independent of the tile's width) can be several times
+// the mean work of an SM.  The tiles are dealt to the blocks by their modelled
+// length, and the longest ones split along N first.  Measured against a
+// round-robin deal of the sorted, unsplit tiles: 64 sectors 16..512 wide
+// 363 -> 328 us, 16 such sectors 173 -> 161 us, the m = 1000 chain 57 -> 52 us, the
+// m = 1000 ladder (16 members) 191 -> 186 us, the m = 400 ladder 61 -> 56 us.
+//
 // Eight draining warps rather than twelve: the block then gets 168 registers
 // a thread without spills (at 448 threads the cap of 128 spilled inside the
 // producer's and the MMA warp's loops), and fewer warps share the issue slots
@@ -45,7 +53,9 @@
 #include <array>
 #include <cmath>
 #include <cstring>
+#include <functional>
 #include <map>
+#include <queue>
 #include <stdexcept>
 #include <vector>
 
@@ -237,7 +247,8 @@ __device__ __forceinline__ bool tile_done(const TcTile& tl, const int32_t* __res
 
 template <int PREC>
 __global__ void __launch_bounds__(TC_THREADS, 1)
-tc_gemm_kernel(const TcTile* __restrict__ tiles, int n_tiles, const TcSeg* __restrict__ segs,
+tc_gemm_kernel(const TcTile* __restrict__ tiles, int n_tiles, const int32_t* __restrict__ cta_begin,
+               const TcSeg* __restrict__ segs,
                const TcOut* __restrict__ seg_outs, double* __restrict__ y, int64_t D, const double* __restrict__ coef, int n_terms, int n_coef,
                int accumulate, const int32_t* __restrict__ skip, const int32_t* __restrict__ member_done,
                int32_t* __restrict__ err, int stages, int stage_bytes, int r_tile_bytes, int tmem_cols,
@@ -285,6 +296,10 @@ tc_gemm_kernel(const TcTile* __restrict__ tiles, int n_tiles, const TcSeg* __res
   __syncthreads();
   tc::tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  // this block's tiles: its own run of the list, or every gridDim.x-th
+  const int t_first = cta_begin ? cta_begin[blockIdx.x] : (int)blockIdx.x;
+  const int t_end = cta_begin ? cta_begin[blockIdx.x + 1] : n_tiles;
+  const int t_step = cta_begin ? 1 : (int)gridDim.x;
 
   if (warp == 0) {
     // ------------------------------------------------------------ producer
@@ -295,21 +310,21 @@ tc_gemm_kernel(const TcTile* __restrict__ tiles, int n_tiles, const TcSeg* __res
       uint32_t issued_par = 0;
       // descriptors are fetched one segment (and one tile) ahead, so that
       // their load latency overlaps the copies of the current segment
-      int t = blockIdx.x;
+      int t = t_first;
       TcTile tl{}, tl_n{};
-      if (t < n_tiles) tl_n = tiles[t];
+      if (t < t_end) tl_n = tiles[t];
       TcSeg sg_n{};
       int sg_n_idx = -1;
-      for (; t < n_tiles; t += gridDim.x) {
+      for (; t < t_end; t += t_step) {
         tl = tl_n;
-        const int tn = t + gridDim.x;
-        if (tn < n_tiles) tl_n = tiles[tn];
+        const int tn = t + t_step;
+        if (tn < t_end) tl_n = tiles[tn];
         if (tile_done(tl, member_done)) continue;
         const uint32_t lb = (uint32_t)tl.la * ATOM_BYTES, rb = (uint32_t)tl.ra * ATOM_BYTES;
         if (tl.pieced) {
           // one L tile and every piece's R rows per K chunk
           const TcSeg sg = sg_n_idx == tl.seg_begin ? sg_n : segs[tl.seg_begin];
-          if (tn < n_tiles && tl_n.seg_begin < tl_n.seg_end) {
+          if (tn < t_end && tl_n.seg_begin < tl_n.seg_end) {
             sg_n = segs[tl_n.seg_begin];
             sg_n_idx = tl_n.seg_begin;
           }
@@ -342,7 +357,7 @@ tc_gemm_kernel(const TcTile* __restrict__ tiles, int n_tiles, const TcSeg* __res
           if (s + 1 < tl.seg_end) {
             sg_n = segs[s + 1];
             sg_n_idx = s + 1;
-          } else if (tn < n_tiles && tl_n.seg_begin < tl_n.seg_end) {
+          } else if (tn < t_end && tl_n.seg_begin < tl_n.seg_end) {
             sg_n = segs[tl_n.seg_begin];
             sg_n_idx = tl_n.seg_begin;
           }
@@ -388,11 +403,11 @@ tc_gemm_kernel(const TcTile* __restrict__ tiles, int n_tiles, const TcSeg* __res
       int kk = 0;  // tiles with products so far: tile kk uses accumulator buffer kk % n_acc
       constexpr uint32_t fmt = PREC == DMRG_TF32 ? tc::FMT_TF32 : tc::FMT_BF16;
       TcTile tl_n{};
-      if (blockIdx.x < n_tiles) tl_n = tiles[blockIdx.x];
+      if (t_first < t_end) tl_n = tiles[t_first];
       int nt_seg = -1, nt_kch = 0, nt_slot = 0;  // the next tile's first segment, loaded during this tile
-      for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
+      for (int t = t_first; t < t_end; t += t_step) {
         const TcTile tl = tl_n;
-        if (t + (int)gridDim.x < n_tiles) tl_n = tiles[t + gridDim.x];  // one tile ahead
+        if (t + t_step < t_end) tl_n = tiles[t + t_step];  // one tile ahead
         if (tl.seg_begin == tl.seg_end || tile_done(tl, member_done)) continue;
         int kch_n = nt_seg == tl.seg_begin ? nt_kch : segs[tl.seg_begin].kchunks;
         int slot_n = nt_seg == tl.seg_begin ? nt_slot : segs[tl.seg_begin].slot;
@@ -411,7 +426,7 @@ tc_gemm_kernel(const TcTile* __restrict__ tiles, int n_tiles, const TcSeg* __res
           if (s + 1 < s_end) {  // one segment ahead
             kch_n = segs[s + 1].kchunks;
             slot_n = segs[s + 1].slot;
-          } else if (t + (int)gridDim.x < n_tiles && tl_n.seg_begin < tl_n.seg_end) {
+          } else if (t + t_step < t_end && tl_n.seg_begin < tl_n.seg_end) {
             nt_seg = tl_n.seg_begin;  // the next tile's first: in flight during this last segment
             nt_kch = segs[nt_seg].kchunks;
             nt_slot = segs[nt_seg].slot;
@@ -476,10 +491,10 @@ tc_gemm_kernel(const TcTile* __restrict__ tiles, int n_tiles, const TcSeg* __res
     double* stg = epi_stage + (warp - 2) * (epi_bytes / (8 * TC_EPI_WARPS));  // this warp's staging
     int kk = 0;  // tiles with products so far (same count as the MMA warp's)
     TcTile tl_n{};
-    if (blockIdx.x < n_tiles) tl_n = tiles[blockIdx.x];
-    for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
+    if (t_first < t_end) tl_n = tiles[t_first];
+    for (int t = t_first; t < t_end; t += t_step) {
       const TcTile tl = tl_n;
-      if (t + (int)gridDim.x < n_tiles) tl_n = tiles[t + gridDim.x];  // one tile ahead
+      if (t + t_step < t_end) tl_n = tiles[t + t_step];  // one tile ahead
       if (tile_done(tl, member_done)) continue;
       const TcOut& o = tl.o;
       const bool empty_tile = tl.seg_begin == tl.seg_end;
@@ -725,6 +740,7 @@ int64_t pad8(int64_t a) { return cdiv(a, 8) * 8; }  // member stride of stacked 
 
 struct Launch {  // one grouped GEMM launch
   TcTile* tiles = nullptr;
+  int32_t* cta_begin = nullptr;     // per block: its first tile (+ end); null: every grid-th tile
   TcTile* tiles_by_out = nullptr;   // the same tiles grouped by output block
   std::vector<int> out_begin;       // per output: first tile in tiles_by_out (+ end)
   TcSeg* segs = nullptr;
@@ -761,7 +777,7 @@ struct EPair {
 
 struct Tune {         // picked by dmrg_autotune
   int max_ntile = 0;  // widest MMA N of a tile (0: default per precision)
-  int heavy_first = 1;  // deal the heaviest tiles first (else build order)
+  int heavy_first = 1;  // balance the blocks by the modelled length of the tiles (else build order)
   int per_block = 0;  // baseline: one launch per output block instead of one persistent launch
   int pieces = 1;     // phase 1: pack pairs sharing their L operand side by side (pieced tiles)
 };
@@ -778,7 +794,7 @@ struct State {
 };
 
 void free_launch(Launch& l) {
-  for (void* p : {(void*)l.tiles, (void*)l.tiles_by_out, (void*)l.segs, (void*)l.seg_outs})
+  for (void* p : {(void*)l.tiles, (void*)l.cta_begin, (void*)l.tiles_by_out, (void*)l.segs, (void*)l.seg_outs})
     if (p) cudaFree(p);
   l = Launch{};
 }
@@ -1000,6 +1016,14 @@ static int64_t build_set(const dmrg_sb* sb, int prec, const std::vector<EPair>& 
     g.kchunks = (int32_t)cdiv(Lp.K, kce);
     return g;
   };
+  // Modelled clocks of a tile, fitted to the measured launches: a K chunk takes
+  // about 700 clocks however narrow the tile is and 2 more per column, or its
+  // copies at 64 bytes a clock; a tile at least its epilogue, and 300 beside it.
+  auto clocks = [&](const TcTile& t, int64_t kchunks) {
+    const int64_t mma = kchunks * (700 + 2 * t.ntile);
+    const int64_t copy = kchunks * (t.la + t.ra) * ATOM_BYTES * (prec == DMRG_BF16X3 ? 2 : 1) / 64;
+    return std::max({mma, copy, (int64_t)t.ntile * 8}) + 300;
+  };
   auto add_out = [&](Build& B, const TcOut& o, const std::vector<TcSeg>& sg, const std::vector<int>& slot_terms) {
     for (const TcSeg& g : sg) {
       check(g.l_atoms == cdiv(o.M, 8) && g.r_atoms == cdiv(o.N, 8), "operand rows differ from the output");
@@ -1046,7 +1070,7 @@ static int64_t build_set(const dmrg_sb* sb, int prec, const std::vector<EPair>& 
         check(t.ntile % 16 == 0 && t.ntile >= 16 && t.ntile <= 256 && t.ra * 8 <= t.ntile, "MMA N");
         B.ntile_max = std::max(B.ntile_max, t.ntile);
         B.tiles.push_back(t);
-        B.weight.push_back(kw * (int64_t)t.ntile + 64);
+        B.weight.push_back(clocks(t, kw));
       }
   };
   // phase 1: the output (an operand panel of phase 2) of a two-GEMM pair
@@ -1156,7 +1180,7 @@ static int64_t build_set(const dmrg_sb* sb, int prec, const std::vector<EPair>& 
         L1.acc_cols = std::max(L1.acc_cols, col);
         L1.ntile_max = std::max(L1.ntile_max, col);
         L1.tiles.push_back(t);
-        L1.weight.push_back((int64_t)sg[0].kchunks * col + 64);
+        L1.weight.push_back(clocks(t, sg[0].kchunks));
       }
     }
   }
@@ -1217,29 +1241,72 @@ static int64_t build_set(const dmrg_sb* sb, int prec, const std::vector<EPair>& 
     }
   }
   auto finish = [&](Build& B, Launch& L) {
-    // heaviest first, dealt round-robin over the persistent CTAs, by groups of
-    // the tiles of one output and first row: the N tiles of a row of tiles
-    // share their L operand tiles, the rows of one output their R operands, so
-    // a group's tiles (and the rows of one output, of equal group weight) stay
-    // neighbours in the order and run on neighbouring CTAs at about the same
-    // time, where the second read of a shared operand tile hits L2
-    std::vector<size_t> perm(B.tiles.size());
-    for (size_t i = 0; i < perm.size(); ++i) perm[i] = i;
+    // Longest first, each tile to the block with the least work so far, by
+    // the modelled clocks (weight).  The tiles of one output come in sequence
+    // of the order: they share operands (the N tiles of a row their L tiles,
+    // the rows their R tiles), so that they run at about the same time and the
+    // second read of a shared operand hits L2.
+    std::vector<TcTile> t;
+    t.reserve(B.tiles.size());
+    std::vector<int32_t> begin;
+    // A launch lasts at least as long as its longest tile: tiles above 1.3
+    // times the mean work of an SM are split along N, down to 32 columns.  Each
+    // part repeats the L copies: splits down to the mean, or to 0.7 of it, cost
+    // wide sectors more than the balance gave (16 sectors 16..512 wide: 163 us,
+    // against 175 and 192).  An element's sum keeps its order in any width.
+    std::vector<TcTile> all;
+    std::vector<int64_t> weight;
     if (tune.heavy_first) {
-      std::map<std::pair<int, int>, int64_t> gw;
-      for (size_t i = 0; i < B.tiles.size(); ++i) gw[{B.tiles[i].out, B.tiles[i].m0}] += B.weight[i];
-      std::vector<int64_t> w(B.tiles.size());
-      for (size_t i = 0; i < B.tiles.size(); ++i) w[i] = gw[{B.tiles[i].out, B.tiles[i].m0}];
-      std::stable_sort(perm.begin(), perm.end(), [&](size_t a, size_t b) { return w[a] > w[b]; });
-      // CTA c takes positions c, c + G, c + 2G, ... (G CTAs): reversing every
-      // second round of G deals the sorted tiles back and forth (a snake), so
-      // that no CTA takes the heavier tile of every round
+      int64_t sum = 0;
+      for (int64_t w : B.weight) sum += w;
+      const int64_t most = std::max<int64_t>(sum / n_sms * 13 / 10, 1);
+      for (size_t i = 0; i < B.tiles.size(); ++i) {
+        const TcTile& u = B.tiles[i];
+        const int parts = (int)std::min<int64_t>(cdiv(B.weight[i], most), u.ntile / 32);
+        if (u.pieced || parts < 2) {
+          all.push_back(u);
+          weight.push_back(B.weight[i]);
+          continue;
+        }
+        int64_t kw = 0;
+        for (int32_t q = u.seg_begin; q < u.seg_end; ++q) kw += B.segs[q].kchunks;
+        const int width = (int)cdiv(cdiv(u.ntile, parts), 16) * 16;
+        for (int n = 0; n < u.ntile; n += width) {
+          TcTile v = u;
+          v.n0 = u.n0 + n;
+          v.ntile = std::min(width, u.ntile - n);
+          v.ra = (int)std::min<int64_t>(v.ntile / 8, cdiv(u.o.N - v.n0, 8));
+          check(v.n0 % 8 == 0 && v.ra >= 1 && v.ntile >= 16 && v.n0 / 8 + v.ra <= cdiv(u.o.N, 8), "part of a tile");
+          all.push_back(v);
+          weight.push_back(clocks(v, kw));
+        }
+      }
+      std::vector<size_t> perm(all.size());
+      for (size_t i = 0; i < perm.size(); ++i) perm[i] = i;
+      std::vector<int64_t> top(B.outs.size(), 0);  // an output's heaviest tile
+      for (size_t i = 0; i < all.size(); ++i)
+        top[all[i].out] = std::max(top[all[i].out], weight[i]);
+      std::stable_sort(perm.begin(), perm.end(),
+                       [&](size_t a, size_t b) { return top[all[a].out] > top[all[b].out]; });
       const size_t G = (size_t)std::max(1, std::min(n_sms, (int)perm.size()));
-      for (size_t r0 = G; r0 < perm.size(); r0 += 2 * G)
-        std::reverse(perm.begin() + r0, perm.begin() + std::min(perm.size(), r0 + G));
+      std::vector<std::vector<size_t>> of(G);
+      std::priority_queue<std::pair<int64_t, size_t>, std::vector<std::pair<int64_t, size_t>>, std::greater<>> load;
+      for (size_t c = 0; c < G; ++c) load.push({0, c});
+      for (size_t i : perm) {
+        auto [w, c] = load.top();
+        load.pop();
+        of[c].push_back(i);
+        load.push({w + weight[i], c});
+      }
+      for (const auto& l : of) {
+        begin.push_back((int32_t)t.size());
+        for (size_t i : l) t.push_back(all[i]);
+      }
+      begin.push_back((int32_t)t.size());
+      L.cta_begin = up(begin);
+    } else {
+      t = B.tiles;
     }
-    std::vector<TcTile> t(B.tiles.size());
-    for (size_t i = 0; i < perm.size(); ++i) t[i] = B.tiles[perm[i]];
     L.tiles = up(t);
     // tiles are built output by output: record where each output starts
     L.tiles_by_out = up(B.tiles);
@@ -1446,13 +1513,13 @@ static void run_gemm(const State* s, const Launch& L, double* y, const dmrg_sb* 
     for (size_t o = 0; o + 1 < L.out_begin.size(); ++o) {
       const int b0 = L.out_begin[o], n = L.out_begin[o + 1] - b0;
       tc_gemm_kernel<PREC><<<std::min(n, s->num_sms), TC_THREADS, smem, st>>>(
-          L.tiles_by_out + b0, n, L.segs, L.seg_outs, y, sb->D, sb->d_coeffs, sb->n_terms, sb->batch * sb->n_terms, accumulate, skip,
+          L.tiles_by_out + b0, n, nullptr, L.segs, L.seg_outs, y, sb->D, sb->d_coeffs, sb->n_terms, sb->batch * sb->n_terms, accumulate, skip,
           member_done, sb->d_tc_err, stages, stage_bytes, r_tile, tmem_cols, epi, L.acc_cols, n_acc, 0, sb->test_stall);
     }
     return;
   }
   const int grid = std::min(L.n_tiles, s->num_sms);
-  tc_gemm_kernel<PREC><<<grid, TC_THREADS, smem, st>>>(L.tiles, L.n_tiles, L.segs, L.seg_outs, y, sb->D,
+  tc_gemm_kernel<PREC><<<grid, TC_THREADS, smem, st>>>(L.tiles, L.n_tiles, L.cta_begin, L.segs, L.seg_outs, y, sb->D,
                                                        sb->d_coeffs, sb->n_terms, sb->batch * sb->n_terms,
                                                        accumulate, skip, member_done,
                                                        sb->d_tc_err, stages, stage_bytes, r_tile, tmem_cols, epi,
