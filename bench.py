@@ -660,14 +660,14 @@ def main():
         pk_r, name_r = pkdf, "df64"
         src_r = (f"{FP32_OPS_PER_CLK} float32 ops/clock / {DF_OPS_PER_FMA} per double-float FMA x 2 x "
                  f"{sm_mhz:.0f} MHz (median SM clock of the timed region)")
-        kern_r = "grouped double-float product, seg_gemm_df_kernel (3 launches per product)"
-        kern_d = ("double-float product with the per-term dots (unscaled intermediates + seg_gemm_df_dots_kernel, "
+        kern_r = "grouped double-float product, seg_gemm_df_kernel (2 launches per product)"
+        kern_d = ("double-float product with the per-term dots (unscaled intermediates + seg_gemm_df_kernel<DOTS>, "
                   "the refinement's residual expected to be the last)")
     else:
         pk_r, name_r = pk64, "fp64"
         src_r = f"304 float64 FMA/clock x 2 x {sm_mhz:.0f} MHz (median SM clock of the timed region)"
-        kern_r = "grouped float64 product, seg_gemm_f64_kernel (3 launches per dmrg_apply_H)"
-        kern_d = ("float64 product with the per-term dots (unscaled intermediates + seg_gemm_f64_dots_kernel, "
+        kern_r = "grouped float64 product, seg_gemm_f64_kernel (2 launches per dmrg_apply_H)"
+        kern_d = ("float64 product with the per-term dots (unscaled intermediates + seg_gemm_f64_kernel<DOTS>, "
                   "the refinement's residual expected to be the last)")
     a_r = flops_mv / (mvr_ms / 1e3) / 1e12
     kernels[f"{name_r}_product"] = {

@@ -173,7 +173,8 @@ dmrg_status dmrg_apply_H_backward(dmrg_sb* sb, const double* psi, const double* 
  * Lanczos with float64 scalars and full reorthogonalisation (every step
  * against every Krylov vector: the three-term step, one classical
  * Gram-Schmidt pass, and a second pass where the norm fell below 1/sqrt(2)),
- * the iteration captured in CUDA graphs.  A member stops when a float32
+ * the iteration captured in CUDA graphs (the first ones of a superblock's
+ * first solve are launched directly).  A member stops when a float32
  * estimate of its residual passes at half the tolerance; the float64 test
  * after the loop confirms it, and a member that misses it restarts from its
  * Ritz vector with the iterations it has left (DMRG_ENOCONV only at max_iter).
@@ -244,7 +245,7 @@ dmrg_status dmrg_continued_fraction(const double* norm2, const double* alpha, co
 /* Autotuner of the tensor-core product (no paper counterpart; the paper's
  * block loop has no tuning): times the product of this superblock, `reps`
  * launches per candidate after a warm-up, for every tile width (64, 128,
- * 256), tile order (heaviest first, or as built) and phase-1
+ * 256), tile order (balanced by modelled length, or as built) and phase-1
  * packing (pairs sharing their wavefunction operand side by side in one
  * tile, or one tile set per pair), keeps the fastest, and also times the
  * baseline that launches one kernel per output block.  Rebuilds task lists and operand panels (allocates); invalidates

@@ -150,7 +150,7 @@ dmrg_status dmrg_sys_last_superblock(dmrg_sys* sys, dmrg_sys_superblock_view* ou
  * row-major, not modified) the eigenvalues w[i] (device [n[i]], decreasing)
  * and eigenvectors V[i] (device n[i] x n[i] row-major, column j for w[i][j]),
  * by cyclic Jacobi rotations in float64: one thread block per matrix up to
- * n = 110 (in its shared memory), a cluster of 16 blocks up to n = 448 (in
+ * n = 32 (in its shared memory), a cluster of 16 blocks up to n = 448 (in
  * their distributed shared memory), one block over global memory above that
  * (n <= 4096).  n, A, V, w: host arrays of [count]; stream-ordered (workspace
  * is allocated on the stream).  DMRG_EINVAL for n[i] < 0 or > 4096 or NULL
