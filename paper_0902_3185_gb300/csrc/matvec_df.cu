@@ -28,8 +28,10 @@
 // ladder).  Measured against 64 x 64 tiles of 256 threads: the 32-site chain
 // at m = 1000 472 -> 273 us, 16 sectors 16..512 wide 4.92 -> 4.23 ms, the 2 x 32
 // ladder at m = 1000 (16 members) 3.14 -> 3.11 ms, with the per-term dots 4.21
-// -> 3.62 ms.  Tiles of 32 x 32 (16 sums a thread) were slower: 6.4 ms on the
-// wide sectors, too few warps for their registers.
+// -> 3.62 ms; a real m = 1000 superblock (blocks up to 424 wide, 16 members) is
+// slower without the dots, 37.8 -> 40.0 ms, and 41.3 -> 40.5 ms with them.  Tiles of 32 x 32
+// (16 sums a thread) were slower: 6.4 ms on the wide sectors, too few warps for
+// their registers.
 
 #include <algorithm>
 
