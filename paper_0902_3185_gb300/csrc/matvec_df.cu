@@ -24,13 +24,20 @@
 // writes as its renormalised (s, c) sums (48 bits, no rounding to float64
 // between the two GEMMs).
 //
+// The two groups of an output's segments are chains of their own, added in
+// float64: one chain over both carries the first group's rounding through the
+// second (error of a product against float64, relative to |y|: 6.4e-14 with
+// one chain, 4.7e-14 with two on a real m = 1000 superblock, 1.3e-14 and 5.6e-15 on
+// the 32-site chain at m = 1000; it costs 0.3 to 2 % of the time, 6 % on the
+// 2 x 32 ladder at m = 400).
+//
 // Bound: instruction issue (80 % of the slots on wide sectors, 66-73 % on the
 // ladder).  Measured against 64 x 64 tiles of 256 threads: the 32-site chain
-// at m = 1000 472 -> 273 us, 16 sectors 16..512 wide 4.92 -> 4.23 ms, the 2 x 32
-// ladder at m = 1000 (16 members) 3.14 -> 3.11 ms, with the per-term dots 4.21
+// at m = 1000 472 -> 276 us, 16 sectors 16..512 wide 4.94 -> 4.25 ms, the 2 x 32
+// ladder at m = 1000 (16 members) 3.14 ms both ways, with the per-term dots 4.21
 // -> 3.62 ms; a real m = 1000 superblock (blocks up to 424 wide, 16 members) is
-// slower without the dots, 37.8 -> 40.0 ms, and 41.3 -> 40.5 ms with them.  Tiles of 32 x 32
-// (16 sums a thread) were slower: 6.4 ms on the wide sectors, too few warps for
+// slower without the dots, 37.8 -> 40.2 ms, and 41.3 -> 40.5 ms with them.  Tiles of
+// 32 x 32 (16 sums a thread) were slower: 6.4 ms on the wide sectors, too few warps for
 // their registers.
 
 #include <algorithm>
@@ -55,7 +62,7 @@ struct ArDF {
   using Acc = float2;   // double-float sum (s, c)
   using Coef = float2;
   using Dot = double;
-  static constexpr bool groups = false;
+  static constexpr bool unrolled_tail = false;
   static __device__ __forceinline__ float2 zero() { return make_float2(0.0f, 0.0f); }
   static __device__ __forceinline__ void fma(double a, double b, float2& c) { df_fma(df_bits(a), df_bits(b), c.x, c.y); }
   // renormalise (fast two-sum, |c| << |s|): c restarts near ulp(s) / 2, so

@@ -32,7 +32,7 @@ struct ArF64 {
     bool unit;
   };
   using Dot = double;
-  static constexpr bool groups = true;
+  static constexpr bool unrolled_tail = true;
   static __device__ __forceinline__ double zero() { return 0.0; }
   static __device__ __forceinline__ void fma(double a, double b, double& c) { c = ::fma(a, b, c); }
   static __device__ __forceinline__ void end_chunk(double&) {}

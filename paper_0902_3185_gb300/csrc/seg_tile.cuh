@@ -21,9 +21,10 @@
 // scales one operand: each thread scales the elements it copied itself, after
 // its own copies have landed and before the barrier that publishes them.
 //
-// Every output element is one chain over the segments in list order and over
-// k in increasing order (float64: one chain per group of segments, then their
-// sum), whatever the tile shape, the same chain on every call.
+// Every output element is one chain per group of segments, over the group's
+// segments in list order and over k in increasing order, and the two chains'
+// values are added in float64, whatever the tile shape, the same chains on
+// every call.
 #pragma once
 
 #include <cstdint>
@@ -179,15 +180,16 @@ __device__ __forceinline__ void seg_tile(const TileF64& t, int member, int batch
     sm.segs[i] = seg_view(segs[t.seg_begin + i], t, member, sm.base, coef, n_terms);
   __syncthreads();
   SegCopier<BM, BN, SMEM> cp(t, segs, coef, n_terms, sm, member);
-  constexpr bool TWO = AR::groups && !DOTS;  // the two groups' sums kept apart (held: the first group's)
-  Acc acc[NI][NJ], held[TWO ? NI : 1][TWO ? NJ : 1];
+  constexpr bool TWO = !DOTS;  // the two groups' sums kept apart (held: the first group's value)
+  Acc acc[NI][NJ];
+  double held[TWO ? NI : 1][TWO ? NJ : 1];
   double sum[DOTS ? NI : 1][DOTS ? NJ : 1];
 #pragma unroll
   for (int i = 0; i < NI; ++i)
 #pragma unroll
     for (int j = 0; j < NJ; ++j) {
       acc[i][j] = AR::zero();
-      if (TWO) held[TWO ? i : 0][TWO ? j : 0] = AR::zero();
+      if (TWO) held[TWO ? i : 0][TWO ? j : 0] = 0.0;
       if (DOTS) sum[DOTS ? i : 0][DOTS ? j : 0] = 0.0;
     }
   // the output block of this member; (m, n) at m * ldc + n
@@ -216,7 +218,7 @@ __device__ __forceinline__ void seg_tile(const TileF64& t, int member, int batch
       for (int i = 0; i < NI; ++i)
 #pragma unroll
         for (int j = 0; j < NJ; ++j) {
-          held[TWO ? i : 0][TWO ? j : 0] = acc[i][j];
+          held[TWO ? i : 0][TWO ? j : 0] = AR::value(acc[i][j]);
           acc[i][j] = AR::zero();
         }
     }
@@ -259,7 +261,7 @@ __device__ __forceinline__ void seg_tile(const TileF64& t, int member, int batch
       if (kmax == SEG_BK) {
 #pragma unroll
         for (int k = 0; k < SEG_BK; ++k) step(k);
-      } else if (!AR::groups) {
+      } else if (!AR::unrolled_tail) {
         for (int k = 0; k < kmax; ++k) step(k);
       } else {
         int k = 0;
@@ -339,7 +341,7 @@ __device__ __forceinline__ void seg_tile(const TileF64& t, int member, int batch
       }
       // the first group's sum, then the second's (each a chain of its own)
       const bool both = TWO && first && second;
-      const double v1 = AR::value(both ? held[TWO ? i : 0][TWO ? j : 0] : acc[i][j]);
+      const double v1 = both ? held[TWO ? i : 0][TWO ? j : 0] : AR::value(acc[i][j]);
       double y = accumulate ? *p + v1 : v1;
       if (both) y += AR::value(acc[i][j]);
       *p = y;
