@@ -136,7 +136,9 @@ dmrg_status dmrg_query(const dmrg_sb* sb, dmrg_sb_info* info);
  * coupling sweeps and finite differences.  The device copy is written on
  * `stream` (through a pinned staging copy), after the work already queued on
  * that stream, and the call returns once it is written (it synchronises
- * `stream`).  Work on other streams that reads this superblock must be
+ * `stream`, also when the table is the one already set and nothing is
+ * written).  After a call that failed the table is unspecified until a call
+ * succeeds.  Work on other streams that reads this superblock must be
  * ordered before the call by the caller. */
 dmrg_status dmrg_set_coeffs(dmrg_sb* sb, const double* coeffs, void* stream);
 
@@ -284,7 +286,8 @@ dmrg_status dmrg_sync_status(dmrg_sb* sb, void* stream);
  * report DMRG_ETIMEOUT through dmrg_sync_status; what = 2 makes the float32
  * convergence test of the next Lanczos solve pass at its first check, so
  * that the float64 test after the loop fails and the restart from the Ritz
- * vector runs; what = 0 clears both.  No memory is touched out of bounds and
+ * vector runs; what = 3 makes the next build of tensor-core operand panels
+ * report that memory has run out; what = 0 clears them.  No memory is touched out of bounds and
  * every wait ends after its limit. */
 dmrg_status dmrg_test_inject(dmrg_sb* sb, int32_t what);
 

@@ -23,6 +23,17 @@
 
 using namespace dmrg;
 
+namespace dmrg {
+void lz_drop_graphs(dmrg_sb* sb) {
+  for (int i = 0; i < 8; ++i)
+    if (sb->lz_graphs[i]) {
+      cudaGraphExecDestroy((cudaGraphExec_t)sb->lz_graphs[i]);
+      sb->lz_graphs[i] = nullptr;
+      sb->lz_graph_key[i] = 0;
+    }
+}
+}  // namespace dmrg
+
 namespace {
 
 struct CudaError {
@@ -607,12 +618,7 @@ void term_dots(dmrg_sb* sb, const double* psi, const double* g, double* dc, cuda
 
 // --------------------------------------------------------------- Lanczos
 void lz_free(dmrg_sb* sb) {
-  for (int i = 0; i < 8; ++i)
-    if (sb->lz_graphs[i]) {
-      cudaGraphExecDestroy((cudaGraphExec_t)sb->lz_graphs[i]);
-      sb->lz_graphs[i] = nullptr;
-      sb->lz_graph_key[i] = 0;
-    }
+  lz_drop_graphs(sb);
   for (void* p : std::initializer_list<void*>{sb->lz_V, sb->lz_w, sb->lz_vcur, sb->lz_partial, sb->lz_h, sb->lz_npart,
                                               sb->lz_ab, sb->lz_s, sb->lz_out, sb->rf_q, sb->rf_sc, sb->rf_diag,
                                               sb->rf_part, sb->rf_res, sb->rf_p, sb->rf_hp, sb->rf_t, sb->rf_psi32,
@@ -1275,8 +1281,11 @@ dmrg_status dmrg_set_coeffs(dmrg_sb* sb, const double* coeffs, void* stream) {
   return guard(sb, [&] {
     cudaStream_t st = (cudaStream_t)stream;
     const size_t n = (size_t)sb->batch * sb->n_terms;
-    // the table that is set already (written and waited for by the call that set it)
-    if (memcmp(sb->coeffs.data(), coeffs, n * sizeof(double)) == 0) return DMRG_OK;
+    // the table that is set already, by a call that went through: nothing to write
+    if (sb->coeffs_set && memcmp(sb->coeffs.data(), coeffs, n * sizeof(double)) == 0) {
+      CK(cudaStreamSynchronize(st));
+      return DMRG_OK;
+    }
     // through a pinned staging copy, ordered on the caller's stream after the
     // products already queued there (which read the old table); the stream is
     // synchronised so that the staging copy is free for the next call
@@ -1285,17 +1294,13 @@ dmrg_status dmrg_set_coeffs(dmrg_sb* sb, const double* coeffs, void* stream) {
       CK(cudaMallocHost(&hp, n * sizeof(double)));
       sb->h_coeffs_pinned = static_cast<double*>(hp);
     }
+    sb->coeffs_set = false;  // until the copy and the panels are done
     memcpy(sb->h_coeffs_pinned, coeffs, n * sizeof(double));
     CK(cudaMemcpyAsync(sb->d_coeffs, sb->h_coeffs_pinned, n * sizeof(double), cudaMemcpyHostToDevice, st));
     CK(cudaStreamSynchronize(st));
     sb->coeffs.assign(coeffs, coeffs + n);
-    if (tc_set_coeffs(sb))  // tensor-core panels with folded coefficients were rebuilt
-      for (int i = 0; i < 8; ++i)
-        if (sb->lz_graphs[i]) {
-          cudaGraphExecDestroy((cudaGraphExec_t)sb->lz_graphs[i]);
-          sb->lz_graphs[i] = nullptr;
-          sb->lz_graph_key[i] = 0;
-        }
+    tc_set_coeffs(sb);  // tensor-core panels with folded coefficients are rebuilt
+    sb->coeffs_set = true;
     return DMRG_OK;
   });
 }
@@ -1355,13 +1360,6 @@ dmrg_status dmrg_autotune(dmrg_sb* sb, int32_t prec, int32_t reps, void* stream,
   return guard(sb, [&] {
     double out[7] = {};
     tc_autotune(sb, prec, reps, (cudaStream_t)stream, out);
-    // captured graphs hold the old task lists
-    for (int i = 0; i < 8; ++i)
-      if (sb->lz_graphs[i]) {
-        cudaGraphExecDestroy((cudaGraphExec_t)sb->lz_graphs[i]);
-        sb->lz_graphs[i] = nullptr;
-        sb->lz_graph_key[i] = 0;
-      }
     if (info) {
       info->best_ms = out[0];
       info->default_ms = out[1];
@@ -1393,13 +1391,17 @@ dmrg_status dmrg_sync_status(dmrg_sb* sb, void* stream) {
 }
 
 dmrg_status dmrg_test_inject(dmrg_sb* sb, int32_t what) {
-  if (!sb || what < 0 || what > 2) return DMRG_EINVAL;
+  if (!sb || what < 0 || what > 3) return DMRG_EINVAL;
   if (what == 2) {
     sb->test_force_pending = 1;
     return DMRG_OK;
   }
+  if (what == 3) {
+    sb->test_fail_panels = 1;
+    return DMRG_OK;
+  }
   sb->test_stall = what;
-  sb->test_force_pending = 0;
+  sb->test_force_pending = sb->test_fail_panels = 0;
   return DMRG_OK;
 }
 

@@ -98,6 +98,7 @@ struct dmrg_sb {
   std::vector<int64_t> off;  // [S+1]
   int64_t D = 0;
   std::vector<double> coeffs;  // host [batch][n_terms]
+  bool coeffs_set = true;      // false from the start of a dmrg_set_coeffs until it has gone through
   double* d_coeffs = nullptr;  // device [batch][n_terms]
   double* h_coeffs_pinned = nullptr;  // pinned staging copy of coeffs for dmrg_set_coeffs
   std::vector<dmrg::PairH> pairs;
@@ -169,8 +170,14 @@ struct dmrg_sb {
   void* tc = nullptr;            // tensor-core path state (matvec_tc.cu)
   int32_t* d_tc_err = nullptr;   // set by a tensor-core kernel whose bounded wait gave up
   int32_t test_stall = 0;        // testing hook: the next tensor-core product issues no copies
+  int32_t test_fail_panels = 0;  // testing hook: the next build of tensor-core panels reports out of memory
   int32_t test_force_pending = 0;  // testing hook: the next Lanczos solve's float32 test passes at its first check
   std::vector<double> h_ops;     // host copy of the float64 arena during creation only
 
   std::string err;
 };
+
+namespace dmrg {
+// forget the captured Lanczos and CG iterations (the memory they name is about to be replaced)
+void lz_drop_graphs(dmrg_sb* sb);
+}  // namespace dmrg

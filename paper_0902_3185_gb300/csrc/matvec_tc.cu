@@ -1367,9 +1367,9 @@ static void build_fmt(dmrg_sb* sb, State* s, int fi);
 // time: the panels are rebuilt when the set of such terms or their values
 // change.  Returns true when it rebuilt (captured graphs then hold stale task
 // lists).
-bool tc_set_coeffs(dmrg_sb* sb) {
+void tc_set_coeffs(dmrg_sb* sb) {
   State* s = st_of(sb);
-  if (!s || !s->ok) return false;
+  if (!s || !s->ok) return;
   const int nt = sb->n_terms;
   const int64_t nb = sb->batch;
   auto uniform = [&](const std::vector<double>& cf, int term) {
@@ -1377,7 +1377,6 @@ bool tc_set_coeffs(dmrg_sb* sb) {
       if (cf[(size_t)b * nt + term] != cf[term]) return false;
     return true;
   };
-  bool rebuilt = false;
   for (int fi = 0; fi < 2; ++fi) {
     const Fmt& F = s->f[fi];
     if (!F.built) continue;  // built later with the coefficients current then
@@ -1388,9 +1387,7 @@ bool tc_set_coeffs(dmrg_sb* sb) {
     }
     if (same) continue;
     build_fmt(sb, s, fi);
-    rebuilt = true;
   }
-  return rebuilt;
 }
 
 void tc_prepare(dmrg_sb* sb, int prec) {
@@ -1411,10 +1408,15 @@ int tc_launches(const dmrg_sb* sb, int prec) {
 static void build_fmt(dmrg_sb* sb, State* s, int fi) {
   const int prec = fi == 0 ? DMRG_TF32 : DMRG_BF16X3;
   Fmt& F = s->f[fi];
+  if (F.built) lz_drop_graphs(sb);  // captured products hold the old panels and lists
   free_set(F.fwd);
   free_set(F.bwd);
   if (F.arena) cudaFree(F.arena);
   F = Fmt{};
+  if (sb->test_fail_panels) {
+    sb->test_fail_panels = 0;
+    throw CudaFail("cudaMalloc (injected)");
+  }
   // sizes depend only on shapes: a dry run lays the arena out first
   std::vector<uint8_t> hi, lo;
   {

@@ -15,7 +15,7 @@ void tc_build(dmrg_sb* sb);      // pair lists (no-op when unsupported); panels 
 void tc_prepare(dmrg_sb* sb, int prec);
 void tc_free(dmrg_sb* sb);
 bool tc_available(const dmrg_sb* sb);
-bool tc_set_coeffs(dmrg_sb* sb);  // true: operand panels rebuilt (captured graphs are stale)
+void tc_set_coeffs(dmrg_sb* sb);  // rebuilds the operand panels that hold coefficients which changed
 double tc_operand_bytes(const dmrg_sb* sb);
 int tc_launches(const dmrg_sb* sb, int prec);  // kernels one product launches
 // member_done (device [batch], may be null): members whose flag is nonzero are
