@@ -46,14 +46,19 @@ struct Upload {
     else e = cudaMallocAsync(reinterpret_cast<void**>(&p), bytes, st);
     if (e != cudaSuccess) throw std::runtime_error(std::string("cudaMallocAsync: ") + cudaGetErrorString(e));
     e = cudaMemcpyAsync(p, host.data(), bytes, cudaMemcpyHostToDevice, st);
-    if (e != cudaSuccess) throw std::runtime_error(std::string("cudaMemcpyAsync: ") + cudaGetErrorString(e));
+    if (e != cudaSuccess) {
+      release();
+      throw std::runtime_error(std::string("cudaMemcpyAsync: ") + cudaGetErrorString(e));
+    }
     *da = reinterpret_cast<const A*>(p);
     *db = reinterpret_cast<const B*>(p + na);
   }
-  ~Upload() {
+  ~Upload() { release(); }
+  void release() {
     if (!p) return;
     if (pool) pool->put(p, bytes);
     else cudaFreeAsync(p, st);
+    p = nullptr;
   }
   Upload(const Upload&) = delete;
   Upload& operator=(const Upload&) = delete;
@@ -69,44 +74,6 @@ struct Tile {
 };
 
 }  // namespace
-
-// --------------------------------------------------------------------- pool
-namespace {
-thread_local DevPool* g_pool = nullptr;
-int size_class(size_t bytes) {
-  int c = 12;
-  while (((size_t)1 << c) < bytes) ++c;
-  return c;
-}
-}  // namespace
-
-DevPool* DevPool::current() { return g_pool; }
-DevPool* DevPool::set_current(DevPool* p) {
-  DevPool* old = g_pool;
-  g_pool = p;
-  return old;
-}
-void* DevPool::get(size_t bytes) {
-  const int c = size_class(bytes);
-  if (c <= MAX_CLASS && !free_[c].empty()) {
-    void* p = free_[c].back();
-    free_[c].pop_back();
-    return p;
-  }
-  void* p = nullptr;
-  const cudaError_t e = cudaMalloc(&p, c <= MAX_CLASS ? (size_t)1 << c : bytes);
-  if (e != cudaSuccess) throw std::runtime_error(std::string("cudaMalloc: ") + cudaGetErrorString(e));
-  return p;
-}
-void DevPool::put(void* p, size_t bytes) {
-  const int c = size_class(bytes);
-  if (c <= MAX_CLASS && free_[c].size() < MAX_KEPT) free_[c].push_back(p);
-  else cudaFree(p);
-}
-DevPool::~DevPool() {
-  for (std::vector<void*>& l : free_)
-    for (void* p : l) cudaFree(p);
-}
 
 // ------------------------------------------------------------------ scatter
 // One 32 x 32 destination tile per block (32 x 8 threads); a transposed

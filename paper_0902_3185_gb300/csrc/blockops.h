@@ -9,27 +9,9 @@
 #include <cstdint>
 #include <vector>
 
+#include "devpool.h"
+
 namespace dmrg {
-
-// Device memory of one DMRG run, kept between its steps: blocks of a power of
-// two bytes up to 4 MiB (larger ones come from and go back to the driver), at
-// most 64 spare blocks of each size, released with the run.  A block put back
-// is handed out again at once, so everything that uses the pool runs on one
-// stream (the run's, the legacy default stream); a run's calls do not overlap.
-// `current` is the calling thread's pool, set for the length of a call.
-class DevPool {
- public:
-  static constexpr int MAX_CLASS = 22;
-  static constexpr size_t MAX_KEPT = 64;
-  void* get(size_t bytes);
-  void put(void* p, size_t bytes);
-  ~DevPool();
-  static DevPool* current();
-  static DevPool* set_current(DevPool* p);  // returns the previous one
-
- private:
-  std::vector<void*> free_[MAX_CLASS + 1];
-};
 
 // dst[i][j] += scale * S(i, j) for a rows x cols destination rectangle;
 // S(i, j) = src[i*ld_src + j] (trans 0), src[j*ld_src + i] (trans 1), or

@@ -16,6 +16,7 @@
 #include <stdexcept>
 #include <numeric>
 
+#include "devpool.h"
 #include "internal.h"
 #include "lanczos.h"
 #include "refine.h"
@@ -74,7 +75,7 @@ T* dalloc(size_t n) {
   if (n == 0) n = 1;
   void* p = nullptr;
   count_alloc();
-  CK(cudaMalloc(&p, n * sizeof(T)));
+  CK(dev_malloc(&p, n * sizeof(T)));
   return static_cast<T*>(p);
 }
 
@@ -91,7 +92,7 @@ class Slab {
     count_alloc();
     const size_t bytes = std::max<size_t>(n, 1) * sizeof(T);
     if (bytes > LARGE) {
-      CK(cudaMalloc(reinterpret_cast<void**>(&d), bytes));
+      CK(dev_malloc(reinterpret_cast<void**>(&d), bytes));
       if (h && n) CK(cudaMemcpy(d, h, n * sizeof(T), cudaMemcpyHostToDevice));
       return;
     }
@@ -109,7 +110,7 @@ class Slab {
     size_t at = 0;
     for (auto* w : {&filled_, &empty_})
       for (Want& x : *w) at += (x.bytes + 255) & ~(size_t)255;
-    CK(cudaMalloc(reinterpret_cast<void**>(slab), std::max<size_t>(at, 256)));
+    CK(dev_malloc(reinterpret_cast<void**>(slab), std::max<size_t>(at, 256)));
     *size = at;
     std::vector<char> host;
     at = 0;

@@ -61,6 +61,7 @@
 
 #include <cuda_bf16.h>
 
+#include "devpool.h"
 #include "internal.h"
 #include "tc.h"
 #include "tc_kernel.cuh"
@@ -705,7 +706,7 @@ template <class T>
 T* up(const std::vector<T>& h) {
   void* p = nullptr;
   const size_t n = std::max<size_t>(1, h.size());
-  TCK(cudaMalloc(&p, n * sizeof(T)));
+  TCK(dev_malloc(&p, n * sizeof(T)));
   if (!h.empty()) TCK(cudaMemcpy(p, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice));
   return static_cast<T*>(p);
 }
@@ -1426,7 +1427,7 @@ static void build_fmt(dmrg_sb* sb, State* s, int fi) {
     F.bytes = (size_t)(a + b2);
   }
   const size_t total = F.bytes * (prec == DMRG_BF16X3 ? 2 : 1);
-  TCK(cudaMalloc(&F.arena, std::max<size_t>(total, 1024)));
+  TCK(dev_malloc(reinterpret_cast<void**>(&F.arena), std::max<size_t>(total, 1024)));
   TCK(cudaMemset(F.arena, 0, std::max<size_t>(total, 1024)));
   const int64_t lo_delta = prec == DMRG_BF16X3 ? (int64_t)F.bytes : 0;
   const int64_t a = build_set(sb, prec, s->fw, 0, hi, lo, F.arena, lo_delta, F.fwd, false, s->tune[fi], s->num_sms);
