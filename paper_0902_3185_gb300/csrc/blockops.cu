@@ -356,8 +356,6 @@ __global__ void __launch_bounds__(EIG_THREADS) k_eig(const EigJob* __restrict__ 
 // float64 unit of the cluster's SMs is 43 % busy (a sweep is 18 million cycles
 // of it per 1000 rounds, 9 to 10 sweeps); 512 threads per block were faster
 // for one wide matrix (51 ms) but slower for many (24 of n = 110 15.5 ms).
-constexpr int EIG_CLUSTER = 16;
-
 // x != 0 by its bits (a float64 compare runs on the float64 unit)
 __device__ __forceinline__ bool nonzero(double x) {
   return ((__double2hiint(x) & 0x7fffffff) | __double2loint(x)) != 0;
@@ -604,15 +602,6 @@ size_t eig_cluster_smem(int n, int C) {
 // largest n the cluster kernel takes (A and V in the cluster's shared memory)
 constexpr int EIG_CLUSTER_MAX_N = 448;
 
-// Blocks per cluster for matrices up to n (> EIG_ONE_BLOCK_N): the float64 work
-// of a round, 3 n^2 cycles of one SM, against the cluster's barriers.
-int eig_cluster_blocks(int n) { return n > 64 ? EIG_CLUSTER : 8; }
-
-// Up to here one block is faster: the square roots and divisions of a round are
-// most of it, and the cluster adds its barriers (n = 16 369 / 538 us, n = 32 1.07
-// / 1.21 ms, n = 40 1.90 / 1.60 ms).
-constexpr int EIG_ONE_BLOCK_N = 32;
-
 // -1: not tried, 0: unavailable on this device, 1: available
 int g_cluster_ok = -1;
 
@@ -660,17 +649,17 @@ bool launch_eig_cluster(std::vector<EigJob> jobs, cudaStream_t st) {
 
 void launch_eig(const std::vector<EigJob>& all, cudaStream_t st) {
   if (all.empty()) return;
-  // everything up to the cluster limit goes to the cluster kernel when the
-  // device runs it (matrices that fit one block's shared memory in a launch of
-  // their own: the larger ones' shared memory would leave one block per SM);
-  // the rest to the one-block kernel
+  // what exceeds one block's shared memory goes to the cluster kernel, up to its
+  // limit and when the device runs it; smaller matrices where that is faster
+  // (eig_clusters_pay), in a launch of their own: the larger ones' shared memory
+  // would leave one block per SM.  The rest goes to the one-block kernel
   std::vector<EigJob> mid, small, jobs;
   for (const EigJob& j : all)
     if (j.n > 0) (j.n > EIG_CLUSTER_MAX_N ? jobs : j.n > EIG_SMEM_MAX_N ? mid : small).push_back(j);
-  int widest = 0;
-  for (const EigJob& j : small) widest = std::max(widest, j.n);
+  std::vector<int> sizes;
+  for (const EigJob& j : small) sizes.push_back(j.n);
   for (std::vector<EigJob>* set : {&mid, &small})
-    if ((set == &small && widest <= EIG_ONE_BLOCK_N) || !launch_eig_cluster(*set, st))
+    if ((set == &small && !eig_clusters_pay(sizes)) || !launch_eig_cluster(*set, st))
       for (const EigJob& j : *set) {
         if (j.n > EIG_SMEM_MAX_N && !j.work) throw std::logic_error("eigensolve: missing workspace");
         jobs.push_back(j);

@@ -37,8 +37,8 @@ struct GemmJob {
 void launch_gemm(const std::vector<GemmJob>& jobs, cudaStream_t st);
 
 // Eigen-decomposition of symmetric n x n matrices by cyclic Jacobi rotations
-// (a thread-block cluster per matrix, or one block): w (n) in decreasing order, V (n x n row-major, column
-// j the eigenvector of w[j]).  A is not modified.  work: 2 n (n + 1) doubles of
+// (a thread-block cluster per matrix, or one block): w (n) in decreasing order,
+// V (n x n row-major, column j the eigenvector of w[j]).  A is not modified.  work: 2 n (n + 1) doubles of
 // device memory per job whose n exceeds the shared-memory limit (else unused).
 struct EigJob {
   const double* A;
@@ -48,6 +48,34 @@ struct EigJob {
   int32_t n, pad;
 };
 constexpr int EIG_SMEM_MAX_N = 110;  // A and V in shared memory up to this size
+constexpr int EIG_CLUSTER = 16;      // blocks of a cluster, at most
+// Blocks per cluster for matrices up to n: the float64 work of a round, 3 n^2
+// cycles of one SM, against the cluster's barriers.
+inline int eig_cluster_blocks(int n) { return n > 64 ? EIG_CLUSTER : 8; }
+// Whether matrices of these sizes (up to EIG_SMEM_MAX_N) are faster one per
+// cluster, or one per block.  One block takes longer for a wide matrix, but
+// hundreds of them run side by side; clusters take turns.  Modelled times (ms)
+// of both, from measured ones:
+//   one matrix, one block / cluster: n = 16 0.37 / 0.54, 32 1.07 / 1.21, 40 1.86 /
+//   1.59, 64 5.2 / 2.7, 65 5.5 / 3.0, 80 9.3 / 3.8, 110 23.6 / 5.9 (the square roots and
+//   divisions of a round are most of a small one);
+//   24 matrices: 33 1.6 / 1.7, 40 2.2 / 2.0, 64 5.5 / 3.2, 110 24 / 10;
+//   64 wide: 60 matrices 5.6 / 4.2, 80 5.7 / 7.0; 65 wide: 40 6.1 / 7.3; 80 wide: 40
+//   10.1 / 10.0, 60 10.2 / 11.4;
+//   150 matrices: 33 2.2 / 4.9, 64 6.0 / 10.5, 65 6.6 / 20.5, 110 25 / 45; 600: 64 20 / 34,
+//   80 36 / 101.
+inline bool eig_clusters_pay(const std::vector<int>& sizes) {
+  int n = 0;
+  for (int s : sizes) n = s > n ? s : n;
+  if (n <= 32) return false;
+  const bool wide = eig_cluster_blocks(n) == EIG_CLUSTER;
+  const double block = 0.026 * n + 1.56e-5 * n * n * n;                       // the widest, alone in its block
+  const double cluster = wide ? 0.0346 * n + 1.7e-4 * n * n : 0.0415 * n;     // alone in its cluster
+  double share = 0.0;  // the clusters' time when they keep the device busy
+  for (int s : sizes) share += (wide ? 0.0028 : 0.0013) * s;
+  const double few = cluster + 0.4 * share;
+  return (few > share ? few : share) < block + 0.1 * share;
+}
 void launch_eig(const std::vector<EigJob>& jobs, cudaStream_t st);
 
 // Global selection of the m largest density-matrix eigenvalues over n
