@@ -175,8 +175,7 @@ dmrg_status dmrg_apply_H_backward(dmrg_sb* sb, const double* psi, const double* 
  * Lanczos with float64 scalars and full reorthogonalisation (every step
  * against every Krylov vector: the three-term step, one classical
  * Gram-Schmidt pass, and a second pass where the norm fell below 1/sqrt(2)),
- * the iteration captured in CUDA graphs (the first ones of a superblock's
- * first solve are launched directly).  A member stops when a float32
+ * the iteration captured in CUDA graphs.  A member stops when a float32
  * estimate of its residual passes at half the tolerance; the float64 test
  * after the loop confirms it, and a member that misses it restarts from its
  * Ritz vector with the iterations it has left (DMRG_ENOCONV only at max_iter).

@@ -750,19 +750,6 @@ cudaGraphExec_t lz_graph(dmrg_sb* sb, int prec, int K) {
   return ge;
 }
 
-// Whether K captured iterations pay at once: capturing and instantiating a
-// graph costs some 0.4 ms of host time, as much as a whole short solve, so the
-// first solve of a kind on a superblock (the only one, in a DMRG step) launches
-// its first iterations directly (LZ_DIRECT_ITERS of them: a direct one costs
-// the GPU about 12 us more) and the graph is made if it needs more.
-constexpr int LZ_DIRECT_ITERS = 32;
-bool graph_pays(dmrg_sb* sb, int key) {
-  for (int k : sb->lz_used)
-    if (k == key) return true;
-  sb->lz_used.push_back(key);
-  return false;
-}
-
 struct LzRun {
   std::vector<int32_t> code, iters, restarts;
   std::vector<double> theta, resid;
@@ -800,13 +787,15 @@ LzRun lz_run(dmrg_sb* sb, const double* psi0, double* psi_out, int prec, double 
   CK(cudaMemcpyAsync(sb->lz_out + 4 * B, &tol, sizeof(double), cudaMemcpyHostToDevice, st));
   CK(cudaStreamSynchronize(st));  // host vectors above are stack memory
   const int K = std::max(1, std::min(graph_iters, max_iter));
-  cudaGraphExec_t ge = graph_pays(sb, 1 + prec * 1024 + K) ? lz_graph(sb, prec, K) : nullptr;
+  // captured at the first solve already: launching the first 8, 16 or 32
+  // iterations one by one instead, for the 0.4 ms that capturing takes, was
+  // slower at every size (first solve of the 32-site chain at m = 200, mixed 5.3
+  // against 5.9 / 6.3 / 6.9 ms, float64 5.3 against 5.5 / 5.8 / 6.2; Heisenberg DMRG run
+  // at m = 32 23.5 against 24.9 / 27.4 / 29.0)
+  cudaGraphExec_t ge = lz_graph(sb, prec, K);
   int launched = 0;
   for (;;) {
-    if (!ge && launched >= LZ_DIRECT_ITERS) ge = lz_graph(sb, prec, K);
-    if (ge) CK(cudaGraphLaunch(ge, st));
-    else
-      for (int k = 0; k < K; ++k) lz_enqueue_iteration(sb, prec, st);
+    CK(cudaGraphLaunch(ge, st));
     launched += K;
     CK(cudaMemcpyAsync(sb->h_ctl, sb->lz_ctl, sizeof(int32_t) * (LZ_CTL_MEMBER + 2 * B), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
@@ -972,7 +961,6 @@ RfRun rf_solve(dmrg_sb* sb, double* psi, int prec, int rprec, double tol, int ma
   std::vector<int32_t> hctl(2 * B + 2, 0), mask(B, 0);
   std::vector<uint8_t> conv(B, 0);
   const int Kg = std::max(1, K);
-  const bool graphs = graph_pays(sb, (1 << 20) + 1 + prec * 1024 + Kg);
   rf_launch_diag(sb->d_dg, sb->d_dg_terms, (int)sb->dg_terms.size(), sb->d_coeffs, sb->n_terms, sb->rf_diag, D, B,
                  st);
   ++r.launches;
@@ -1041,13 +1029,10 @@ RfRun rf_solve(dmrg_sb* sb, double* psi, int prec, int rprec, double tol, int ma
     CK(cudaMemcpyAsync(sb->rf_ctl, hctl.data(), sizeof(int32_t) * (2 * B + 2), cudaMemcpyHostToDevice, st));
     CK(cudaMemcpyAsync(sb->rf_sc + RF_NSC * B, &eps, sizeof(double), cudaMemcpyHostToDevice, st));
     CK(cudaStreamSynchronize(st));
-    cudaGraphExec_t ge = graphs ? rf_graph(sb, prec, Kg) : nullptr;
+    cudaGraphExec_t ge = rf_graph(sb, prec, Kg);
     int launched = 0;
     for (;;) {
-      if (!ge && launched >= LZ_DIRECT_ITERS) ge = rf_graph(sb, prec, Kg);
-      if (ge) CK(cudaGraphLaunch(ge, st));
-      else
-        for (int k = 0; k < Kg; ++k) rf_enqueue_inner(sb, prec, st);
+      CK(cudaGraphLaunch(ge, st));
       launched += Kg;
       r.launches += (int64_t)Kg * (RF_KERNELS_PER_ITER + matvec_launches(sb, prec));
       int32_t stop = 0;

@@ -162,7 +162,6 @@ struct dmrg_sb {
   double* d_dg = nullptr;
   void* lz_graphs[8] = {};       // cached cudaGraphExec_t per (prec, K) slot
   int32_t lz_graph_key[8] = {};
-  std::vector<int32_t> lz_used;  // keys of the solves that have run once (their graphs are made at the second)
   // the allocations that hold the small arrays of the superblock and of its solver buffers
   char *slab = nullptr, *lz_slab = nullptr;
   size_t slab_bytes = 0, lz_slab_bytes = 0;

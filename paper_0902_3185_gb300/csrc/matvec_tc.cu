@@ -1366,8 +1366,7 @@ static void build_fmt(dmrg_sb* sb, State* s, int fi);
 // Coefficients are read from the shared table at run time, except those of
 // identity terms uniform over the batch, folded into operator panels at build
 // time: the panels are rebuilt when the set of such terms or their values
-// change.  Returns true when it rebuilt (captured graphs then hold stale task
-// lists).
+// change.
 void tc_set_coeffs(dmrg_sb* sb) {
   State* s = st_of(sb);
   if (!s || !s->ok) return;
