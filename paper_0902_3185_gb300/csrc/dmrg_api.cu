@@ -7,6 +7,7 @@
 // Lanczos needs only that product).
 
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -21,6 +22,7 @@
 #include "lanczos.h"
 #include "refine.h"
 #include "tc.h"
+#include "tiles.h"
 
 using namespace dmrg;
 
@@ -267,87 +269,92 @@ int32_t seg_shape(int32_t M, int32_t N, int64_t sumK, int64_t chunks, bool few, 
   return shape;
 }
 
-// Cut outputs (their descriptors with the segment range set, their segments in
-// tl.h_segs) into tiles, the heaviest first (one block per tile and member);
-// which[i] (optional) gets the output of tile i.
-std::vector<TileF64> cut_tiles(const TaskListF64& tl, const std::vector<TileF64>& outs, int batch, bool df,
-                               std::vector<int32_t>* which = nullptr) {
+// A list's outputs (their descriptors with the segment range set) in the order
+// of their tiles, the heaviest first (one block per tile and member).
+struct Cut {
+  std::vector<TileF64> outs;
+  std::vector<int32_t> first;  // first tile of every output (+ end)
+  int64_t tiles = 0, items = 0;  // tiles, (tile, segment) items
+};
+Cut cut_outputs(const std::vector<SegF64>& segs, const std::vector<TileF64>& protos, int batch, bool df) {
   int64_t t16 = 0;
-  for (const TileF64& o : outs) t16 += (int64_t)((o.M + 15) / 16) * ((o.N + 15) / 16);
+  for (const TileF64& o : protos) t16 += (int64_t)((o.M + 15) / 16) * ((o.N + 15) / 16);
   const bool few = t16 * batch < SEG_FEW_TILES;
-  // all tiles of an output weigh the same: the outputs are sorted, then cut
-  struct Cut {
+  // all tiles of an output weigh the same: the outputs are sorted, and cut on the device
+  struct Weight {
     int64_t w;
     int32_t i, shape;
   };
-  std::vector<Cut> cuts;
-  cuts.reserve(outs.size());
-  size_t total = 0;
-  for (size_t i = 0; i < outs.size(); ++i) {
-    const TileF64& t = outs[i];
+  std::vector<Weight> order;
+  order.reserve(protos.size());
+  for (size_t i = 0; i < protos.size(); ++i) {
+    const TileF64& t = protos[i];
     if (t.M <= 0 || t.N <= 0) continue;
     int64_t k = 0, chunks = 0;
     for (int32_t q = t.seg_begin; q < t.seg_end; ++q) {
-      k += tl.h_segs[q].K;
-      chunks += (tl.h_segs[q].K + 15) / 16;
+      k += segs[q].K;
+      chunks += (segs[q].K + 15) / 16;
     }
     const int32_t shape = seg_shape(t.M, t.N, k, chunks, few, df);
-    const int32_t bm = 8 * (shape & 0xff), bn = 8 * (shape >> 8);
-    cuts.push_back({k * bm * bn, (int32_t)i, shape});
-    total += (size_t)((t.M + bm - 1) / bm) * ((t.N + bn - 1) / bn);
+    order.push_back({k * (8 * (shape & 0xff)) * (8 * (shape >> 8)), (int32_t)i, shape});
   }
-  std::stable_sort(cuts.begin(), cuts.end(), [](const Cut& x, const Cut& y) { return x.w > y.w; });
-  std::vector<TileF64> out;
-  out.reserve(total);
-  if (which) which->clear();
-  for (const Cut& c : cuts) {
-    TileF64 t = outs[c.i];
-    t.shape = c.shape;
+  std::stable_sort(order.begin(), order.end(), [](const Weight& x, const Weight& y) { return x.w > y.w; });
+  Cut cut;
+  cut.outs.reserve(order.size());
+  cut.first.assign(1, 0);
+  cut.first.reserve(order.size() + 1);
+  for (const Weight& o : order) {
+    TileF64 t = protos[o.i];
+    t.shape = o.shape;
+    t.dot_base = (int32_t)cut.items;
     const int32_t bm = 8 * (t.shape & 0xff), bn = 8 * (t.shape >> 8);
-    for (t.m0 = 0; t.m0 < t.M; t.m0 += bm)
-      for (t.n0 = 0; t.n0 < t.N; t.n0 += bn) {
-        out.push_back(t);
-        if (which) which->push_back(c.i);
-      }
+    const int64_t n = (int64_t)((t.M + bm - 1) / bm) * ((t.N + bn - 1) / bn);
+    cut.tiles += n;
+    cut.items += n * (t.seg_end - t.seg_begin);
+    if (cut.tiles * batch > INT32_MAX) throw Invalid{"too many product tiles"};
+    cut.outs.push_back(t);
+    cut.first.push_back((int32_t)cut.tiles);
   }
-  if ((int64_t)out.size() * batch > INT32_MAX) throw Invalid{"too many product tiles"};
-  return out;
+  return cut;
 }
 
-void make_tiles(TaskListF64& tl, const std::vector<OutF64>& outs, int batch, std::vector<int32_t>* which = nullptr) {
+// A list's arrays: the segments, the outputs cut for float64 and (with_df) for
+// double-float arithmetic.  The float64 tiles are made when the slab is (the
+// launch that expands them follows it).  Returns both cuts, for the dot lists.
+std::array<Cut, 2> make_list(TaskListF64& tl, const std::vector<OutF64>& outs, int batch, bool with_df, Slab& slab,
+                             std::vector<SegF64>* segs_out = nullptr) {
   std::vector<TileF64> protos;
+  std::vector<SegF64> segs;
   for (const OutF64& o : outs) {
     TileF64 t = o.proto;
-    t.seg_begin = (int32_t)tl.h_segs.size();
+    t.seg_begin = (int32_t)segs.size();
     t.seg_mid = t.seg_begin + o.nM;
-    tl.h_segs.insert(tl.h_segs.end(), o.segs.begin(), o.segs.end());
-    t.seg_end = (int32_t)tl.h_segs.size();
+    segs.insert(segs.end(), o.segs.begin(), o.segs.end());
+    t.seg_end = (int32_t)segs.size();
     protos.push_back(t);
   }
-  tl.h_tiles = cut_tiles(tl, protos, batch, false, which);
-}
-
-// the outputs of a list: its tiles at the origin
-std::vector<TileF64> list_outputs(const TaskListF64& tl) {
-  std::vector<TileF64> outs;
-  for (const TileF64& t : tl.h_tiles)
-    if (t.m0 == 0 && t.n0 == 0) outs.push_back(t);
-  return outs;
-}
-
-void finish(TaskListF64& tl, Slab& slab) {
-  tl.n_tiles = (int64_t)tl.h_tiles.size();
-  slab.array(tl.d_tiles, tl.h_tiles);
-  slab.array(tl.d_segs, tl.h_segs);
+  slab.array(tl.d_segs, segs);
+  std::array<Cut, 2> cuts;
+  cuts[0] = cut_outputs(segs, protos, batch, false);
+  tl.n_outs = (int32_t)cuts[0].outs.size();
+  tl.n_tiles = cuts[0].tiles;
+  slab.array(tl.d_outs, cuts[0].outs);
+  slab.array(tl.d_first, cuts[0].first);
+  slab.array(tl.d_tiles, (size_t)tl.n_tiles);
+  if (with_df) {
+    cuts[1] = cut_outputs(segs, protos, batch, true);
+    tl.n_tiles_df = cuts[1].tiles;
+    slab.array(tl.d_outs_df, cuts[1].outs);
+    slab.array(tl.d_first_df, cuts[1].first);
+  }
+  if (segs_out) segs_out->swap(segs);
+  return cuts;
 }
 
 void free_tl(const dmrg_sb* sb, TaskListF64& tl) {
-  dfree(sb, tl.d_tiles);
-  dfree(sb, tl.d_segs);
-  if (tl.d_tiles_df) cudaFree(tl.d_tiles_df);
-  tl.d_tiles_df = nullptr;
-  tl.d_tiles = nullptr;
-  tl.d_segs = nullptr;
+  for (void* p : std::initializer_list<void*>{tl.d_segs, tl.d_outs, tl.d_first, tl.d_tiles, tl.d_outs_df, tl.d_first_df})
+    dfree(sb, p);
+  tl = TaskListF64{};
 }
 
 bool is_gemm_pair(int flags) { return (flags & (DMRG_ID_A | DMRG_ID_B)) == 0; }
@@ -454,42 +461,42 @@ int64_t layout_T(const dmrg_sb* sb, const std::vector<GPair>& P, std::vector<int
   return T;
 }
 
-// The partials of a dot list per (member, term), in list order: item i, of
-// term terms[i], has SEG_DOT_PARTS for every member.
-void upload_dot_lists(const dmrg_sb* sb, const std::vector<int32_t>& terms, int32_t*& d_ptr, int32_t*& d_idx,
-                      double*& d_part, Slab* slab = nullptr) {
-  const int64_t per = (int64_t)sb->batch * SEG_DOT_PARTS;
-  if ((int64_t)terms.size() * per > INT32_MAX) throw Invalid{"too many product segments for the per-term dots"};
-  std::vector<std::vector<int32_t>> items((size_t)sb->n_terms);
-  for (size_t i = 0; i < terms.size(); ++i) items[terms[i]].push_back((int32_t)i);
-  std::vector<int32_t> ptr(1, 0), idx;
-  for (int b = 0; b < sb->batch; ++b)
-    for (const std::vector<int32_t>& l : items) {
-      for (int32_t i : l)
-        for (int w = 0; w < SEG_DOT_PARTS; ++w) idx.push_back((int32_t)((i * (int64_t)sb->batch + b) * SEG_DOT_PARTS + w));
-      ptr.push_back((int32_t)idx.size());
-    }
-  const size_t parts = (size_t)std::max<int64_t>(1, (int64_t)terms.size() * per);
-  if (slab) {
-    slab->array(d_ptr, ptr);
-    slab->array(d_idx, idx);
-    slab->array(d_part, parts);
-    return;
-  }
-  upload(d_ptr, ptr);
-  upload(d_idx, idx);
-  if (d_part) cudaFree(d_part);
-  d_part = dalloc<double>(parts);
+// The term sums of a dot list: a run per output and segment (TM_STORE_DOTS), or
+// per output (TM_DOT: one segment, an item per tile).  with_partials: the
+// partials are part of the slab as well.
+int64_t dot_parts(const dmrg_sb* sb, int64_t items) {
+  const int64_t n = items * sb->batch * SEG_DOT_PARTS;
+  if (n > INT32_MAX) throw Invalid{"too many product segments for the per-term dots"};
+  return std::max<int64_t>(1, n);
 }
-
-// number the (tile, segment) items of TM_STORE_DOTS tiles; returns their terms
-std::vector<int32_t> number_segments(const TaskListF64& tl, std::vector<TileF64>& tiles) {
-  std::vector<int32_t> terms;
-  for (TileF64& t : tiles) {
-    t.dot_base = (int32_t)terms.size();
-    for (int32_t q = t.seg_begin; q < t.seg_end; ++q) terms.push_back(tl.h_segs[q].term);
+void make_dot_list(const dmrg_sb* sb, DotList& l, const Cut& cut, const std::vector<SegF64>& segs, bool with_partials,
+                   Slab& slab) {
+  std::vector<std::vector<DotRun>> by_term((size_t)sb->n_terms);
+  for (size_t o = 0; o < cut.outs.size(); ++o) {
+    const TileF64& t = cut.outs[o];
+    const int32_t n = cut.first[o + 1] - cut.first[o];
+    for (int32_t q = t.seg_begin; q < t.seg_end; ++q) {
+      std::vector<DotRun>& v = by_term[segs[q].term];
+      const int32_t at = v.empty() ? 0 : v.back().end;
+      if (t.mode == TM_DOT) v.push_back({cut.first[o], 1, at, at + n});
+      else v.push_back({t.dot_base + (q - t.seg_begin), t.seg_end - t.seg_begin, at, at + n});
+    }
   }
-  return terms;
+  std::vector<int32_t> ptr(1, 0);
+  std::vector<DotRun> runs;
+  for (const std::vector<DotRun>& v : by_term) {
+    runs.insert(runs.end(), v.begin(), v.end());
+    ptr.push_back((int32_t)runs.size());
+  }
+  l.n_items = cut.items;
+  slab.array(l.d_ptr, ptr);
+  slab.array(l.d_runs, runs);
+  if (with_partials) slab.array(l.d_partial, (size_t)dot_parts(sb, l.n_items));
+}
+void free_dots(const dmrg_sb* sb, DotList& l, bool partials) {
+  dfree(sb, l.d_ptr);
+  dfree(sb, l.d_runs);
+  if (partials) dfree(sb, l.d_partial);
 }
 
 void build_f64_tasks(dmrg_sb* sb, Slab& slab) {
@@ -516,12 +523,12 @@ void build_f64_tasks(dmrg_sb* sb, Slab& slab) {
   sb->T_fwd_elems = Tf > 0 ? Tm * (sb->batch - 1) + Tf : 0;  // member b's forward intermediates at b Tm + [0, Tf)
   slab.array(sb->d_T, (size_t)sb->T_elems);
 
-  make_tiles(sb->f64_fwd1, phase1_outs(sb, fw, toff_f, Tm, true), sb->batch);
-  make_tiles(sb->f64_fwd2, phase2_outs(sb, fw, toff_f, Tm, true), sb->batch);
-  make_tiles(sb->f64_bwd1, phase1_outs(sb, bw, toff_b, Tm, true), sb->batch);
-  make_tiles(sb->f64_bwd2, phase2_outs(sb, bw, toff_b, Tm, true), sb->batch);
-  make_tiles(sb->f64_dot1, phase1_outs(sb, fw, toff_f, Tm, false), sb->batch);
-
+  make_list(sb->f64_fwd1, phase1_outs(sb, fw, toff_f, Tm, true), sb->batch, true, slab);
+  make_list(sb->f64_fwd2, phase2_outs(sb, fw, toff_f, Tm, true), sb->batch, true, slab);
+  make_list(sb->f64_bwd1, phase1_outs(sb, bw, toff_b, Tm, true), sb->batch, false, slab);
+  make_list(sb->f64_bwd2, phase2_outs(sb, bw, toff_b, Tm, true), sb->batch, false, slab);
+  make_list(sb->f64_dot1, phase1_outs(sb, fw, toff_f, Tm, false), sb->batch, true, slab);
+  std::vector<SegF64> segs;
   {  // per-term dots: one output per pair, dotted with G
     std::vector<OutF64> outs;
     for (size_t i = 0; i < fw.size(); ++i) {
@@ -532,22 +539,27 @@ void build_f64_tasks(dmrg_sb* sb, Slab& slab) {
       o.nM = 1;
       outs.push_back(std::move(o));
     }
-    std::vector<int32_t> which;
-    make_tiles(sb->f64_dot2, outs, sb->batch, &which);
-    std::vector<int32_t> terms;
-    for (int32_t i : which) terms.push_back(fw[i].term);
-    upload_dot_lists(sb, terms, sb->d_dot_red_ptr, sb->d_dot_red_idx, sb->d_dot_partial, &slab);
+    const std::array<Cut, 2> cuts = make_list(sb->f64_dot2, outs, sb->batch, false, slab, &segs);
+    make_dot_list(sb, sb->dot, cuts[0], segs, true, slab);
   }
   {  // H psi with the per-term dots <psi, (A_k x B_k) psi> in one pass: the
      // output launch of the product with unscaled segments (after f64_dot1's
      // unscaled intermediates); the tiles apply c(member, term) themselves
-    make_tiles(sb->f64_pdot2, phase2_outs(sb, fw, toff_f, Tm, false, true), sb->batch);
-    upload_dot_lists(sb, number_segments(sb->f64_pdot2, sb->f64_pdot2.h_tiles), sb->d_pdot_ptr, sb->d_pdot_idx,
-                     sb->d_pdot_partial, &slab);
+    const std::array<Cut, 2> cuts =
+        make_list(sb->f64_pdot2, phase2_outs(sb, fw, toff_f, Tm, false, true), sb->batch, true, slab, &segs);
+    make_dot_list(sb, sb->pdot, cuts[0], segs, true, slab);
+    make_dot_list(sb, sb->pdot_df, cuts[1], segs, false, slab);
   }
-  for (TaskListF64* tl : {&sb->f64_fwd1, &sb->f64_fwd2, &sb->f64_dot1, &sb->f64_dot2, &sb->f64_bwd1, &sb->f64_bwd2,
-                          &sb->f64_pdot2})
-    finish(*tl, slab);
+}
+
+// the float64 tiles of every list, once the slab is there
+void expand_f64_tiles(dmrg_sb* sb, cudaStream_t st) {
+  ExpandArgs a;
+  for (const TaskListF64* tl : {&sb->f64_fwd1, &sb->f64_fwd2, &sb->f64_dot1, &sb->f64_dot2, &sb->f64_bwd1,
+                                &sb->f64_bwd2, &sb->f64_pdot2})
+    a.add(tl->d_outs, tl->d_first, tl->d_tiles, tl->n_outs);
+  launch_expand_tiles(a, st);
+  CK(cudaGetLastError());
 }
 
 // ------------------------------------------------------------- products
@@ -555,18 +567,32 @@ void build_f64_tasks(dmrg_sb* sb, Slab& slab) {
 // the first such product) and the input, split into a buffer of its own each
 // time; the intermediates are written and read as pairs.
 Bufs df_bufs(dmrg_sb* sb, const double* x, double* y, cudaStream_t st) {
-  if (!sb->d_ops_df) {
-    for (TaskListF64* tl : {&sb->f64_fwd1, &sb->f64_fwd2, &sb->f64_dot1, &sb->f64_pdot2}) {
-      std::vector<TileF64> tiles = cut_tiles(*tl, list_outputs(*tl), sb->batch, true);
-      if (tl == &sb->f64_pdot2)
-        upload_dot_lists(sb, number_segments(*tl, tiles), sb->d_pdot_ptr_df, sb->d_pdot_idx_df, sb->d_pdot_partial_df);
-      upload(tl->d_tiles_df, tiles);
-      tl->n_tiles_df = (int64_t)tiles.size();
+  if (!sb->df_mem) {  // one allocation for all that these products add to the superblock
+    TaskListF64* const lists[] = {&sb->f64_fwd1, &sb->f64_fwd2, &sb->f64_dot1, &sb->f64_pdot2};
+    const int64_t parts = dot_parts(sb, sb->pdot_df.n_items);
+    size_t at = 0;
+    auto place = [&](size_t bytes) {
+      const size_t p = at;
+      at += (bytes + 255) & ~(size_t)255;
+      return p;
+    };
+    size_t tiles[4];
+    for (int i = 0; i < 4; ++i) tiles[i] = place((size_t)lists[i]->n_tiles_df * sizeof(TileF64));
+    const size_t part = place((size_t)parts * sizeof(double));
+    const size_t ops = place((size_t)sb->ops_elems * sizeof(double));
+    const size_t xs = place((size_t)(sb->batch * sb->D) * sizeof(double));
+    sb->df_mem = dalloc<char>(at);
+    ExpandArgs a;
+    for (int i = 0; i < 4; ++i) {
+      lists[i]->d_tiles_df = reinterpret_cast<TileF64*>(sb->df_mem + tiles[i]);
+      a.add(lists[i]->d_outs_df, lists[i]->d_first_df, lists[i]->d_tiles_df, lists[i]->n_outs);
     }
-    sb->d_ops_df = dalloc<double>((size_t)std::max<int64_t>(sb->ops_elems, 1));
+    sb->pdot_df.d_partial = reinterpret_cast<double*>(sb->df_mem + part);
+    sb->d_ops_df = reinterpret_cast<double*>(sb->df_mem + ops);
+    sb->d_x_df = reinterpret_cast<double*>(sb->df_mem + xs);
+    launch_expand_tiles(a, st);
     launch_split_pairs(sb->d_ops, sb->d_ops_df, sb->ops_elems, st);
   }
-  if (!sb->d_x_df) sb->d_x_df = dalloc<double>((size_t)(sb->batch * sb->D));
   launch_split_pairs(x, sb->d_x_df, sb->batch * sb->D, st);
   return Bufs{{sb->d_x_df, y, sb->d_T, sb->d_ops_df, nullptr}};
 }
@@ -596,24 +622,22 @@ void matvec_f64_dots(dmrg_sb* sb, const double* psi, double* y, double* dc, cuda
   if (df) {
     const Bufs bufs = df_bufs(sb, psi, y, st);
     launch_seg_gemm_df(sb->f64_dot1, bufs, sb->d_coeffs, sb->n_terms, sb->batch, 0, st);
-    launch_seg_gemm_df_dots(sb->f64_pdot2, bufs, sb->d_coeffs, sb->n_terms, sb->batch, 0, sb->d_pdot_partial_df,
-                            st);
+    launch_seg_gemm_df_dots(sb->f64_pdot2, bufs, sb->d_coeffs, sb->n_terms, sb->batch, 0, sb->pdot_df.d_partial, st);
   } else {
     Bufs bufs{{const_cast<double*>(psi), y, sb->d_T, sb->d_ops, nullptr}};
     launch_seg_gemm_f64(sb->f64_dot1, bufs, sb->d_coeffs, sb->n_terms, sb->batch, 0, nullptr, nullptr, st);
-    launch_seg_gemm_f64_dots(sb->f64_pdot2, bufs, sb->d_coeffs, sb->n_terms, sb->batch, 0, sb->d_pdot_partial,
-                             nullptr, st);
+    launch_seg_gemm_f64_dots(sb->f64_pdot2, bufs, sb->d_coeffs, sb->n_terms, sb->batch, 0, sb->pdot.d_partial, nullptr,
+                             st);
   }
-  lz_launch_reduce_terms(df ? sb->d_pdot_partial_df : sb->d_pdot_partial, df ? sb->d_pdot_ptr_df : sb->d_pdot_ptr,
-                         df ? sb->d_pdot_idx_df : sb->d_pdot_idx, dc, sb->batch * sb->n_terms, st);
+  launch_reduce_terms(df ? sb->pdot_df : sb->pdot, dc, sb->batch, sb->n_terms, st);
   CK(cudaGetLastError());
 }
 
 void term_dots(dmrg_sb* sb, const double* psi, const double* g, double* dc, cudaStream_t st) {
   Bufs bufs{{const_cast<double*>(psi), nullptr, sb->d_T, sb->d_ops, const_cast<double*>(g)}};
   launch_seg_gemm_f64(sb->f64_dot1, bufs, sb->d_coeffs, sb->n_terms, sb->batch, 0, nullptr, nullptr, st);
-  launch_seg_gemm_f64(sb->f64_dot2, bufs, sb->d_coeffs, sb->n_terms, sb->batch, 0, sb->d_dot_partial, nullptr, st);
-  lz_launch_reduce_terms(sb->d_dot_partial, sb->d_dot_red_ptr, sb->d_dot_red_idx, dc, sb->batch * sb->n_terms, st);
+  launch_seg_gemm_f64(sb->f64_dot2, bufs, sb->d_coeffs, sb->n_terms, sb->batch, 0, sb->dot.d_partial, nullptr, st);
+  launch_reduce_terms(sb->dot, dc, sb->batch, sb->n_terms, st);
   CK(cudaGetLastError());
 }
 
@@ -1204,10 +1228,12 @@ void destroy(dmrg_sb* sb) {
                           &sb->f64_pdot2})
     free_tl(sb, *tl);
   for (void* p : std::initializer_list<void*>{
-           sb->d_coeffs, sb->d_ops, sb->d_T, sb->d_dot_partial, sb->d_scratch, sb->d_red, sb->d_dg, sb->d_pdot_partial,
-           sb->d_pdot_partial_df, sb->d_ops_df, sb->d_x_df, sb->d_pdot_ptr, sb->d_pdot_idx, sb->d_pdot_ptr_df,
-           sb->d_pdot_idx_df, sb->d_dg_terms, sb->d_tc_err, sb->d_dot_red_ptr, sb->d_dot_red_idx})
+           sb->d_coeffs, sb->d_ops, sb->d_T, sb->d_scratch, sb->d_red, sb->d_dg, sb->d_dg_terms, sb->d_tc_err})
     dfree(sb, p);
+  free_dots(sb, sb->dot, true);
+  free_dots(sb, sb->pdot, true);
+  free_dots(sb, sb->pdot_df, false);
+  if (sb->df_mem) cudaFree(sb->df_mem);
   if (sb->slab) cudaFree(sb->slab);
   if (sb->h_coeffs_pinned) cudaFreeHost(sb->h_coeffs_pinned);
   delete sb;
@@ -1228,6 +1254,7 @@ dmrg_status dmrg_create_superblock(const dmrg_sb_desc* d, int32_t batch, dmrg_sb
     validate_and_copy(sb, d, batch, slab);
     build_f64_tasks(sb, slab);
     slab.make(&sb->slab, &sb->slab_bytes);
+    expand_f64_tiles(sb, nullptr);
     tc_build(sb);
     sb->h_ops.clear();
     sb->h_ops.shrink_to_fit();

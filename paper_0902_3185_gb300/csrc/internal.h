@@ -53,18 +53,36 @@ struct TileF64 {
 };
 
 struct TaskListF64 {
-  std::vector<TileF64> h_tiles;
-  std::vector<SegF64> h_segs;
-  TileF64* d_tiles = nullptr;
   SegF64* d_segs = nullptr;
+  int32_t n_outs = 0;
+  TileF64* d_outs = nullptr;   // descriptors of the outputs, in the order of their tiles
+  int32_t* d_first = nullptr;  // first tile of every output (+ end)
+  TileF64* d_tiles = nullptr;
   int64_t n_tiles = 0;  // per member: a launch has n_tiles * batch blocks, block tile * batch + member
-  // the same outputs cut for double-float arithmetic (at the first such product)
+  // the same outputs cut for double-float arithmetic (tiles made at the first such product)
+  TileF64* d_outs_df = nullptr;
+  int32_t* d_first_df = nullptr;
   TileF64* d_tiles_df = nullptr;
   int64_t n_tiles_df = 0;
 };
 
 // dot partials per (tile, member), or per (tile, segment, member): one per warp of a block
 constexpr int SEG_DOT_PARTS = 2;
+
+// The partials of a dot list by term.  An item is a (tile, segment) of the list
+// (a tile of a TM_DOT list); item i of member b has the partials
+// (i * batch + b) * SEG_DOT_PARTS + part.  A run: the items of one output and
+// segment, item + u stride for its tiles u, elements first .. end - 1 of its
+// term's list.
+struct DotRun {
+  int32_t item, stride, first, end;
+};
+struct DotList {
+  int32_t* d_ptr = nullptr;    // runs of term k: ptr[k] .. ptr[k+1] - 1
+  DotRun* d_runs = nullptr;
+  double* d_partial = nullptr;
+  int64_t n_items = 0;
+};
 
 // skip: optional device flag; when *skip != 0 the launch does nothing
 void launch_seg_gemm_f64(const TaskListF64& tl, const Bufs& bufs, const double* coef, int n_terms, int batch,
@@ -103,6 +121,7 @@ struct dmrg_sb {
   double* h_coeffs_pinned = nullptr;  // pinned staging copy of coeffs for dmrg_set_coeffs
   std::vector<dmrg::PairH> pairs;
   double* d_ops = nullptr;     // FP64 operator arena
+  char* df_mem = nullptr;      // tiles, dot partials, d_ops_df and d_x_df of the double-float products (at the first)
   double* d_ops_df = nullptr;  // the same arena as double-float pairs (first double-float product)
   double* d_x_df = nullptr;    // [batch][D] the double-float product's input as pairs
   int64_t ops_elems = 0;
@@ -113,19 +132,10 @@ struct dmrg_sb {
   dmrg::TaskListF64 f64_bwd1, f64_bwd2;   // H^T g
   dmrg::TaskListF64 f64_dot1, f64_dot2;   // per-pair <g, A psi B^T>
   dmrg::TaskListF64 f64_pdot2;            // H psi and per-term <psi, (A_k x B_k) psi> in one pass (after f64_dot1)
-  int32_t* d_pdot_ptr = nullptr;          // term reduction of its segment partials, as d_dot_red_*
-  int32_t* d_pdot_idx = nullptr;
-  double* d_pdot_partial = nullptr;
-  int32_t* d_pdot_ptr_df = nullptr;       // the same for the double-float tiles
-  int32_t* d_pdot_idx_df = nullptr;
-  double* d_pdot_partial_df = nullptr;
+  dmrg::DotList dot, pdot, pdot_df;       // term sums of f64_dot2, of f64_pdot2, of its double-float tiles
   double* d_T = nullptr;                  // FP64 intermediate workspace
   int64_t T_elems = 0;
   int64_t T_fwd_elems = 0;               // the part of it the forward product uses
-  // term reduction of dot tiles: for (b, k): tile range [dot_red_ptr[bk], dot_red_ptr[bk+1])
-  int32_t* d_dot_red_ptr = nullptr;
-  int32_t* d_dot_red_idx = nullptr;
-  double* d_dot_partial = nullptr;
   double* d_scratch = nullptr;  // small reduction scratch (batch norms)
   double* d_red = nullptr;      // [batch][chunks] reduction partials outside Lanczos
 

@@ -96,7 +96,5 @@ void lz_launch_scale_unit(const double* x, const double* nrm2, double* y, double
 void lz_launch_ritz(const double* V, const double* s, const int32_t* ctl, double* out, int64_t D, int batch,
                     int cap, cudaStream_t st, bool pair);
 void lz_launch_div_rows(double* v, const double* nrm2, int n_terms, int batch, cudaStream_t st);
-void lz_launch_reduce_terms(const double* part, const int32_t* ptr, const int32_t* idx, double* out, int n,
-                            cudaStream_t st);
 
 }  // namespace dmrg
