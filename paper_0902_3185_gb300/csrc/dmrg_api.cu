@@ -244,20 +244,32 @@ TileF64 out_tile(int32_t buf, int64_t off, int64_t bs, int32_t ldc, int32_t M, i
 // output list, more in the intermediates': 279 / 285 us; 355 wide ones 413 /
 // 423 us), double-float 5 to 9 % in favour of 16.
 constexpr int64_t SEG_FEW_TILES = 152 * 6;
+// From this many 24 x 24 tiles (all members; three rounds of eight blocks per
+// SM) a list may use tiles up to 24 wide, if that saves at least a third of the
+// tiles (outputs wide enough to fill them).  An operand element is copied and
+// scaled once for 24 outputs instead of 16 or 8.  Both lists of a product 16
+// wide / by this rule: the real m = 1000 superblock (blocks up to 424 wide) with
+// 16 members float64 138.1 / 131.6, double-float 40.2 / 37.0 ms, with one 8.79 /
+// 8.61 and 2.59 / 2.55; 64 sectors 16..512 wide 47.1 / 46.8 and 14.2 / 14.1; the m = 1000
+// ladder with 16 members 7.63 / 7.43 and 3.14 / 2.90 ms.  Below it 24 wide is slower:
+// 757 tiles in the output list 742 / 878 us (32-site chain, m = 1000), 836 and 3040
+// in the intermediates' 243 / 253 us; so are 8784 tiles on blocks of at most 40
+// (211 / 214 us, m = 400 ladder).
+constexpr int64_t SEG_WIDE_TILES = 152 * 8 * 3;
 
 // Tile shape of an M x N output with `chunks` K chunks of sumK in all:
-// 8*ni x 8*nj of the least estimated cost.  A tile pays its area, padding
+// 8*ni x 8*nj, ni and nj up to `widest`, of the least estimated cost.  A tile pays its area, padding
 // included, for every k, and for every chunk a fixed cost (barrier, loop) and
 // its edges (copies).  In cycles of an SM: 0.5 per element and k in float64
 // (2 multiply-adds per clock), 0.1 in double-float (13 instructions, 128
 // lanes), 30 + 0.6 per edge element for a chunk (two warps' instructions on
 // four schedulers).  8 x 8 when the list has few tiles.
-int32_t seg_shape(int32_t M, int32_t N, int64_t sumK, int64_t chunks, bool few, bool df) {
+int32_t seg_shape(int32_t M, int32_t N, int64_t sumK, int64_t chunks, bool few, bool df, int widest) {
   if (few) return 1 | (1 << 8);
   double best = -1.0;
   int32_t shape = 1 | (1 << 8);
-  for (int32_t ni = 2; ni >= 1; --ni)
-    for (int32_t nj = 2; nj >= 1; --nj) {
+  for (int32_t ni = widest; ni >= 1; --ni)
+    for (int32_t nj = widest; nj >= 1; --nj) {
       const int32_t bm = 8 * ni, bn = 8 * nj;
       const double tiles = (double)((M + bm - 1) / bm) * ((N + bn - 1) / bn);
       const double cost = tiles * ((df ? 0.1 : 0.5) * sumK * bm * bn + chunks * (30.0 + 0.6 * (bm + bn)));
@@ -275,11 +287,17 @@ struct Cut {
   std::vector<TileF64> outs;
   std::vector<int32_t> first;  // first tile of every output (+ end)
   int64_t tiles = 0, items = 0;  // tiles, (tile, segment) items
+  bool wide = false;             // some are 24 wide
 };
 Cut cut_outputs(const std::vector<SegF64>& segs, const std::vector<TileF64>& protos, int batch, bool df) {
-  int64_t t16 = 0;
-  for (const TileF64& o : protos) t16 += (int64_t)((o.M + 15) / 16) * ((o.N + 15) / 16);
+  int64_t t16 = 0, t24 = 0;
+  for (const TileF64& o : protos) {
+    t16 += (int64_t)((o.M + 15) / 16) * ((o.N + 15) / 16);
+    t24 += (int64_t)((o.M + 23) / 24) * ((o.N + 23) / 24);
+  }
   const bool few = t16 * batch < SEG_FEW_TILES;
+  const bool dots = !protos.empty() && protos[0].mode != TM_STORE;
+  const int widest = !dots && t24 * batch >= SEG_WIDE_TILES && 2 * t16 >= 3 * t24 ? 3 : 2;
   // all tiles of an output weigh the same: the outputs are sorted, and cut on the device
   struct Weight {
     int64_t w;
@@ -295,7 +313,7 @@ Cut cut_outputs(const std::vector<SegF64>& segs, const std::vector<TileF64>& pro
       k += segs[q].K;
       chunks += (segs[q].K + 15) / 16;
     }
-    const int32_t shape = seg_shape(t.M, t.N, k, chunks, few, df);
+    const int32_t shape = seg_shape(t.M, t.N, k, chunks, few, df, widest);
     order.push_back({k * (8 * (shape & 0xff)) * (8 * (shape >> 8)), (int32_t)i, shape});
   }
   std::stable_sort(order.begin(), order.end(), [](const Weight& x, const Weight& y) { return x.w > y.w; });
@@ -310,6 +328,7 @@ Cut cut_outputs(const std::vector<SegF64>& segs, const std::vector<TileF64>& pro
     const int32_t bm = 8 * (t.shape & 0xff), bn = 8 * (t.shape >> 8);
     const int64_t n = (int64_t)((t.M + bm - 1) / bm) * ((t.N + bn - 1) / bn);
     cut.tiles += n;
+    if (bm > 16 || bn > 16) cut.wide = true;
     cut.items += n * (t.seg_end - t.seg_begin);
     if (cut.tiles * batch > INT32_MAX) throw Invalid{"too many product tiles"};
     cut.outs.push_back(t);
@@ -338,12 +357,14 @@ std::array<Cut, 2> make_list(TaskListF64& tl, const std::vector<OutF64>& outs, i
   cuts[0] = cut_outputs(segs, protos, batch, false);
   tl.n_outs = (int32_t)cuts[0].outs.size();
   tl.n_tiles = cuts[0].tiles;
+  tl.wide = cuts[0].wide;
   slab.array(tl.d_outs, cuts[0].outs);
   slab.array(tl.d_first, cuts[0].first);
   slab.array(tl.d_tiles, (size_t)tl.n_tiles);
   if (with_df) {
     cuts[1] = cut_outputs(segs, protos, batch, true);
     tl.n_tiles_df = cuts[1].tiles;
+    tl.wide_df = cuts[1].wide;
     slab.array(tl.d_outs_df, cuts[1].outs);
     slab.array(tl.d_first_df, cuts[1].first);
   }

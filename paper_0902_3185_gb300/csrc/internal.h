@@ -58,6 +58,7 @@ struct TaskListF64 {
   TileF64* d_outs = nullptr;   // descriptors of the outputs, in the order of their tiles
   int32_t* d_first = nullptr;  // first tile of every output (+ end)
   TileF64* d_tiles = nullptr;
+  bool wide = false, wide_df = false;  // tiles up to 24 wide (else 16), float64 and double-float
   int64_t n_tiles = 0;  // per member: a launch has n_tiles * batch blocks, block tile * batch + member
   // the same outputs cut for double-float arithmetic (tiles made at the first such product)
   TileF64* d_outs_df = nullptr;

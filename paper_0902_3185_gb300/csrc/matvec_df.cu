@@ -28,17 +28,17 @@
 // float64: one chain over both carries the first group's rounding through the
 // second (error of a product against float64, relative to |y|: 6.4e-14 with
 // one chain, 4.7e-14 with two on a real m = 1000 superblock, 1.3e-14 and 5.6e-15 on
-// the 32-site chain at m = 1000; it costs 0.3 to 2 % of the time, 6 % on the
+// the 32-site chain at m = 1000; it costs 0.3 to 2 % of the time, 5 % on the
 // 2 x 32 ladder at m = 400).
 //
 // Bound: instruction issue (80 % of the slots on wide sectors, 66-73 % on the
 // ladder).  Measured against 64 x 64 tiles of 256 threads: the 32-site chain
-// at m = 1000 472 -> 276 us, 16 sectors 16..512 wide 4.94 -> 4.25 ms, the 2 x 32
-// ladder at m = 1000 (16 members) 3.14 ms both ways, with the per-term dots 4.21
-// -> 3.62 ms; a real m = 1000 superblock (blocks up to 424 wide, 16 members) is
-// slower without the dots, 37.8 -> 40.2 ms, and 41.3 -> 40.5 ms with them.  Tiles of
-// 32 x 32 (16 sums a thread) were slower: 6.4 ms on the wide sectors, too few warps for
-// their registers.
+// at m = 1000 472 -> 277 us, 16 sectors 16..512 wide 4.96 -> 4.23 ms, the 2 x 32
+// ladder at m = 1000 (16 members) 3.15 -> 2.90 ms, with the per-term dots 4.21
+// -> 3.62 ms; a real m = 1000 superblock (blocks up to 424 wide, 16 members) 37.9
+// -> 37.0 ms (24 x 24 tiles; 40.2 with 16 x 16), with the dots 41.3 -> 40.5 ms (16 x
+// 16: the dots need a third set of sums).  Tiles of 32 x 32 (16 sums a thread)
+// were slower: 6.4 ms on the 16 sectors, too few warps for their registers.
 
 #include <algorithm>
 
@@ -92,19 +92,19 @@ struct ArDF {
   }
 };
 
-#define SEG_SHAPES(CASE) CASE(1, 1) CASE(1, 2) CASE(2, 1) CASE(2, 2)
 
-template <bool DOTS>
+// BMAX: the widest tile edge of the list
+template <bool DOTS, int BMAX>
 __global__ void __launch_bounds__(SEG_THREADS, 8)
 seg_gemm_df_kernel(const TileF64* __restrict__ tiles, const SegF64* __restrict__ segs, Bufs bufs,
                    const double* __restrict__ coef, int n_terms, int batch, int accumulate,
                    double* __restrict__ dot_out) {
-  __shared__ SegSmem<16> sm;
+  __shared__ SegSmem<BMAX> sm;
   const TileF64 t = tiles[blockIdx.x / batch];
   const int member = blockIdx.x % batch;
 #define DF_CASE(I, J)                                                                                       \
   case (I) | ((J) << 8):                                                                                    \
-    seg_tile<ArDF, I, J, DOTS>(t, member, batch, segs, bufs, coef, n_terms, accumulate, dot_out, sm); \
+    if constexpr (8 * I <= BMAX && 8 * J <= BMAX) seg_tile<ArDF, I, J, DOTS>(t, member, batch, segs, bufs, coef, n_terms, accumulate, dot_out, sm); \
     break;
   switch (t.shape) {
     SEG_SHAPES(DF_CASE)
@@ -116,14 +116,15 @@ seg_gemm_df_kernel(const TileF64* __restrict__ tiles, const SegF64* __restrict__
 void launch_seg_gemm_df(const TaskListF64& tl, const Bufs& bufs, const double* coef, int n_terms, int batch,
                         int accumulate, cudaStream_t st) {
   if (tl.n_tiles_df == 0) return;
-  seg_gemm_df_kernel<false><<<(unsigned)(tl.n_tiles_df * batch), SEG_THREADS, 0, st>>>(
-      tl.d_tiles_df, tl.d_segs, bufs, coef, n_terms, batch, accumulate, nullptr);
+  (tl.wide_df ? seg_gemm_df_kernel<false, SEG_BWIDE> : seg_gemm_df_kernel<false, 16>)
+      <<<(unsigned)(tl.n_tiles_df * batch), SEG_THREADS, 0, st>>>(tl.d_tiles_df, tl.d_segs, bufs, coef, n_terms, batch,
+                                                                 accumulate, nullptr);
 }
 
 void launch_seg_gemm_df_dots(const TaskListF64& tl, const Bufs& bufs, const double* coef, int n_terms, int batch,
                              int accumulate, double* dot_out, cudaStream_t st) {
   if (tl.n_tiles_df == 0) return;
-  seg_gemm_df_kernel<true><<<(unsigned)(tl.n_tiles_df * batch), SEG_THREADS, 0, st>>>(
+  seg_gemm_df_kernel<true, 16><<<(unsigned)(tl.n_tiles_df * batch), SEG_THREADS, 0, st>>>(
       tl.d_tiles_df, tl.d_segs, bufs, coef, n_terms, batch, accumulate, dot_out);
 }
 

@@ -13,9 +13,10 @@
 // Measured against 64 x 64 tiles of 256 threads with one chunk in flight and
 // the two output groups in launches of their own: one product of the 12-site
 // ladder at m = 60 (2 members) 145 -> 26 us, of the 32-site chain at m = 200
-// 108 -> 27 us, at m = 1000 1429 -> 743 us, of the 2 x 32 ladder at m = 400 (4
-// members) 707 -> 212 us, of 16 sectors 16..512 wide 17.3 -> 14.1 ms (1.14
-// TFLOP/s; the float64 unit is 95-97 % busy).
+// 107 -> 27 us, at m = 1000 1428 -> 742 us, of the 2 x 32 ladder at m = 400 (4
+// members) 708 -> 212 us, at m = 1000 (16 members) 7.80 -> 7.43 ms, of 16 sectors
+// 16..512 wide 17.3 -> 14.0 ms (1.15 TFLOP/s; the float64 unit is 95-97 % busy), of
+// a real m = 1000 superblock (16 members) 135.0 -> 131.6 ms.
 
 #include "internal.h"
 #include "seg_tile.cuh"
@@ -55,20 +56,20 @@ struct ArF64 {
   }
 };
 
-#define SEG_SHAPES(CASE) CASE(1, 1) CASE(1, 2) CASE(2, 1) CASE(2, 2)
 
-template <bool DOTS>
+// BMAX: the widest tile edge of the list
+template <bool DOTS, int BMAX>
 __global__ void __launch_bounds__(SEG_THREADS, 8)
 seg_gemm_f64_kernel(const TileF64* __restrict__ tiles, const SegF64* __restrict__ segs, Bufs bufs,
                     const double* __restrict__ coef, int n_terms, int batch, int accumulate,
                     double* __restrict__ dot_out, const int32_t* __restrict__ skip) {
-  __shared__ SegSmem<16> sm;
+  __shared__ SegSmem<BMAX> sm;
   if (skip && *skip) return;
   const TileF64 t = tiles[blockIdx.x / batch];
   const int member = blockIdx.x % batch;
 #define F64_CASE(I, J)                                                                                       \
   case (I) | ((J) << 8):                                                                                     \
-    seg_tile<ArF64, I, J, DOTS>(t, member, batch, segs, bufs, coef, n_terms, accumulate, dot_out, sm); \
+    if constexpr (8 * I <= BMAX && 8 * J <= BMAX) seg_tile<ArF64, I, J, DOTS>(t, member, batch, segs, bufs, coef, n_terms, accumulate, dot_out, sm); \
     break;
   switch (t.shape) {
     SEG_SHAPES(F64_CASE)
@@ -80,15 +81,16 @@ seg_gemm_f64_kernel(const TileF64* __restrict__ tiles, const SegF64* __restrict_
 void launch_seg_gemm_f64_dots(const TaskListF64& tl, const Bufs& bufs, const double* coef, int n_terms, int batch,
                               int accumulate, double* dot_out, const int32_t* skip, cudaStream_t st) {
   if (tl.n_tiles == 0) return;
-  seg_gemm_f64_kernel<true><<<(unsigned)(tl.n_tiles * batch), SEG_THREADS, 0, st>>>(
+  seg_gemm_f64_kernel<true, 16><<<(unsigned)(tl.n_tiles * batch), SEG_THREADS, 0, st>>>(
       tl.d_tiles, tl.d_segs, bufs, coef, n_terms, batch, accumulate, dot_out, skip);
 }
 
 void launch_seg_gemm_f64(const TaskListF64& tl, const Bufs& bufs, const double* coef, int n_terms, int batch,
                          int accumulate, double* dot_out, const int32_t* skip, cudaStream_t st) {
   if (tl.n_tiles == 0) return;
-  seg_gemm_f64_kernel<false><<<(unsigned)(tl.n_tiles * batch), SEG_THREADS, 0, st>>>(
-      tl.d_tiles, tl.d_segs, bufs, coef, n_terms, batch, accumulate, dot_out, skip);
+  (tl.wide ? seg_gemm_f64_kernel<false, SEG_BWIDE> : seg_gemm_f64_kernel<false, 16>)
+      <<<(unsigned)(tl.n_tiles * batch), SEG_THREADS, 0, st>>>(tl.d_tiles, tl.d_segs, bufs, coef, n_terms, batch,
+                                                              accumulate, dot_out, skip);
 }
 
 }  // namespace dmrg

@@ -6,13 +6,13 @@
 // (one unit shared by the SM's four schedulers: a warp's instruction takes 16
 // cycles of it), so the product is bound by that unit as soon as a few warps
 // per SM have work, and by the length of one output element's chain of
-// multiply-adds when an SM has too little of it.  Hence small tiles: 16 x 16
-// or 8 x 8 outputs, 64 threads, at most four chains per thread.  Operand
-// traffic does not matter at this rate (a 16 x 16 tile reads 1 byte per
-// multiply-add from L2), padding and idle SMs do: sector blocks are 1..80 wide
-// in a DMRG superblock, 16..512 in the widest, and a tile is padded to
-// multiples of 8 only.  Every SM holds many such blocks, which hides the
-// latency of each one's loads and barriers.
+// multiply-adds when an SM has too little of it.  Hence small tiles: 8, 16 or,
+// in lists that fill the chip several times over, 24 outputs a side, 64 threads,
+// at most nine chains per thread.  Operand traffic does not matter at this rate
+// (a 16 x 16 tile reads 1 byte per multiply-add from L2), padding and idle SMs
+// do: sector blocks are 1..80 wide in a DMRG superblock, up to 512 in the
+// widest, and a tile is padded to multiples of 8 only.  Every SM holds many
+// such blocks, which hides the latency of each one's loads and barriers.
 //
 // The segments of a tile are one flat sequence of K chunks of 16, copied by
 // cp.async (8 bytes per element, zero outside the operands) into a ring of
@@ -32,6 +32,11 @@
 #include "internal.h"
 
 namespace dmrg {
+
+// tile shapes 8 I x 8 J (a kernel for lists up to BMAX wide compiles those that fit)
+#define SEG_SHAPES(CASE) \
+  CASE(1, 1) CASE(1, 2) CASE(2, 1) CASE(2, 2) CASE(1, 3) CASE(2, 3) CASE(3, 1) CASE(3, 2) CASE(3, 3)
+constexpr int SEG_BWIDE = 24;  // widest tile edge of a wide list
 
 constexpr int SEG_THREADS = 64;
 constexpr int SEG_BK = 16;      // K chunk
@@ -108,12 +113,34 @@ struct SegCopier {
     const int l = i - t.seg_begin;
     return l < SEG_SMEM_SEGS ? sm.segs[l] : seg_view(segs[i], t, member, sm.base, coef, n_terms);
   }
-  // element slots of this thread: index tid + 64 e runs along the operand's contiguous direction
-  static __device__ __forceinline__ void l_slot(int idx, int trans, int& m, int& k) {
-    if (trans) { k = idx / BM; m = idx % BM; } else { m = idx / SEG_BK; k = idx % SEG_BK; }
+  // Element slot e of thread tid in an operand with an outer index o of width B
+  // (rows of L, columns of R) and the K index: consecutive threads run along
+  // the contiguous direction, K (k_fast) or o.  `step` is the slot's distance
+  // from the thread's slot 0 as o and k.
+  template <int B>
+  static __device__ __forceinline__ void slot(int tid, int e, bool k_fast, int& o, int& k) {
+    if (k_fast) {
+      o = (tid + e * SEG_THREADS) / SEG_BK;
+      k = (tid + e * SEG_THREADS) % SEG_BK;
+    } else if (SEG_THREADS % B == 0) {
+      k = (tid + e * SEG_THREADS) / B;
+      o = (tid + e * SEG_THREADS) % B;
+    } else {  // runs of 8 along o
+      k = tid / 8 + 8 * (e / (B / 8));
+      o = tid % 8 + 8 * (e % (B / 8));
+    }
   }
-  static __device__ __forceinline__ void r_slot(int idx, int trans, int& n, int& k) {
-    if (trans) { n = idx / SEG_BK; k = idx % SEG_BK; } else { k = idx / BN; n = idx % BN; }
+  template <int B>
+  static __device__ __forceinline__ int64_t step(int e, bool k_fast, int32_t ld) {
+    if (k_fast) return (int64_t)ld * (e * SEG_THREADS / SEG_BK);
+    if (SEG_THREADS % B == 0) return (int64_t)ld * (e * SEG_THREADS / B);
+    return (int64_t)ld * (8 * (e / (B / 8))) + 8 * (e % (B / 8));
+  }
+  static __device__ __forceinline__ void l_slot(int tid, int e, int trans, int& m, int& k) {
+    slot<BM>(tid, e, !trans, m, k);
+  }
+  static __device__ __forceinline__ void r_slot(int tid, int e, int trans, int& n, int& k) {
+    slot<BN>(tid, e, trans, n, k);
   }
   __device__ __forceinline__ void open() {
     if (q >= t.seg_end) return;
@@ -125,8 +152,8 @@ struct SegCopier {
     ldl = s.ldl;
     ldr = s.ldr;
     int m, n, kl, kr;
-    l_slot(tid, l_trans, m, kl);
-    r_slot(tid, r_trans, n, kr);
+    l_slot(tid, 0, l_trans, m, kl);
+    r_slot(tid, 0, r_trans, n, kr);
     lp = s.L + (l_trans ? (int64_t)kl * ldl + m : (int64_t)m * ldl + kl);
     rp = s.R + (r_trans ? (int64_t)n * ldr + kr : (int64_t)kr * ldr + n);
   }
@@ -137,16 +164,16 @@ struct SegCopier {
 #pragma unroll
       for (int e = 0; e < SL; ++e) {
         int m, k;
-        l_slot(tid + e * SEG_THREADS, l_trans, m, k);
+        l_slot(tid, e, l_trans, m, k);
         const bool in = t.m0 + m < t.M && k0 + k < K;
-        cp_async8(&sm.L[stage][k][m], in ? lp + (int64_t)ldl * (e * SEG_THREADS / (l_trans ? BM : SEG_BK)) : none, in);
+        cp_async8(&sm.L[stage][k][m], in ? lp + step<BM>(e, !l_trans, ldl) : none, in);
       }
 #pragma unroll
       for (int e = 0; e < SR; ++e) {
         int n, k;
-        r_slot(tid + e * SEG_THREADS, r_trans, n, k);
+        r_slot(tid, e, r_trans, n, k);
         const bool in = t.n0 + n < t.N && k0 + k < K;
-        cp_async8(&sm.R[stage][k][n], in ? rp + (int64_t)ldr * (e * SEG_THREADS / (r_trans ? SEG_BK : BN)) : none, in);
+        cp_async8(&sm.R[stage][k][n], in ? rp + step<BN>(e, r_trans, ldr) : none, in);
       }
       lp += l_trans ? (int64_t)SEG_BK * ldl : SEG_BK;
       rp += r_trans ? SEG_BK : (int64_t)SEG_BK * ldr;
@@ -230,14 +257,14 @@ __device__ __forceinline__ void seg_tile(const TileF64& t, int member, int batch
 #pragma unroll
         for (int e = 0; e < cp.SL; ++e) {
           int m, k;
-          cp.l_slot(tid + e * SEG_THREADS, lt, m, k);
+          cp.l_slot(tid, e, lt, m, k);
           sm.L[stage][k][m] = AR::scaled(sm.L[stage][k][m], f);
         }
       } else if (scale == 2) {
 #pragma unroll
         for (int e = 0; e < cp.SR; ++e) {
           int n, k;
-          cp.r_slot(tid + e * SEG_THREADS, rt, n, k);
+          cp.r_slot(tid, e, rt, n, k);
           sm.R[stage][k][n] = AR::scaled(sm.R[stage][k][n], f);
         }
       }
@@ -259,8 +286,17 @@ __device__ __forceinline__ void seg_tile(const TileF64& t, int member, int batch
       // its bits, unrolled, so that the shared-memory loads run ahead of the
       // chains (the double-float loop would outgrow the instruction cache)
       if (kmax == SEG_BK) {
+        if (!AR::unrolled_tail && NI * NJ > 4) {
+          // two steps at a time: unrolled, the 24-wide double-float chunk is 30 KB
+          // of instructions, and the blocks of an SM, each at another place, fetch
+          // them from L2 (real m = 1000 superblock, unrolled by 2 / 4 / 8 / 16: 37.0 /
+          // 37.1 / 40.6 / 40.8 ms; 64 sectors 16..512 wide 14.1 / 15.1 / 19.5 / 19.6 ms)
+#pragma unroll 2
+          for (int k = 0; k < SEG_BK; ++k) step(k);
+        } else {
 #pragma unroll
-        for (int k = 0; k < SEG_BK; ++k) step(k);
+          for (int k = 0; k < SEG_BK; ++k) step(k);
+        }
       } else if (!AR::unrolled_tail) {
         for (int k = 0; k < kmax; ++k) step(k);
       } else {
