@@ -726,6 +726,16 @@ __device__ __forceinline__ void warp_product_scan(float* r, int n, bool backward
     for (int i = b; i < e; ++i) at(i) *= before;
 }
 
+// How far above the value that stops a member the float32 estimate may be for
+// the deciding solve to be due.  An estimate that is too high by more than this
+// delays a stop, one that is too low costs a float64 solve of 0.2 ms.  Against
+// the exact last component (Lanczos matrices of up to 140 steps, |T| 1 to 200) it
+// is good to 5e-4 when the lowest gap is above 0.1, to 10 % at gaps of 1e-5 |T|,
+// to 1.5 at 1e-6 |T|; at 1e-7 |T|, where float32 does not tell the two lowest
+// eigenvalues apart, it was 100 times too high at worst, and one solve in six
+// stopped 2 to 5 steps later than by a float64 test at every step (of 60).
+constexpr double LZ_DUE = 2.0;
+
 // The end of a Lanczos step, one block per member:
 //  - alpha_j = the sum of the v_j coefficients of the passes that ran, beta_j
 //    = |w| after the last pass (not in the final pass);
@@ -746,8 +756,8 @@ __device__ __forceinline__ void warp_product_scan(float* r, int n, bool backward
 //  in absolute terms only: tolerances below 1e-5 had needed the float64
 //  eigenpair at every check from 1e-2 |T| on.)
 //  Decision, by one warp:
-//  - tol >= 1e-5, once the estimate is within a factor 2 of the value that
-//    stops the member (half the tolerance): float32 multisection and inverse
+//  - tol >= 1e-5, once the estimate is within LZ_DUE of the value that stops
+//    the member (half the tolerance): float32 multisection and inverse
 //    iteration; when they pass, the member stops as LZ_PENDING; after the
 //    iteration loop one launch (final_pass) computes the eigenpair of every
 //    pending member at its own length in float64 (multisection from the
@@ -758,7 +768,7 @@ __device__ __forceinline__ void warp_product_scan(float* r, int n, bool backward
 //    Ritz vector: the members' float64 solves run side by side in one launch
 //    instead of each in the launch where its member converged;
 //  - tol < 1e-5: that float64 eigenpair and test as soon as the estimate is
-//    within a factor 8 of the tolerance;
+//    within LZ_DUE of the tolerance;
 //  - a pivot that was not positive leaves no estimate: the warp decides;
 //  - at breakdown or the cap the float64 eigenpair is computed at once.
 // GB300 issues float64 at 1/64 of the float32 rate: a warp's instruction holds
@@ -951,9 +961,9 @@ k_tridiag(const double* __restrict__ h, const double* __restrict__ npart_b, cons
       nz = tri_block_sum(nz, red);
       const double est = beta * (double)(fabsf(n - 1 >= kt ? dmi[n - 1] : dpl[n - 1]) * rsqrtf(nz));
       const double bound = tol * fmax(1.0, fabs((double)th32));
-      // a decision is due when the estimate is within a factor 2 of the value
-      // that stops the member, or says nothing
-      const bool far = !unsure && isfinite(est) && est > (tol < 1e-5 ? 2.0 : 1.0) * bound;
+      // a decision is due when the estimate comes near the value that stops the
+      // member (the tolerance or half of it), or says nothing
+      const bool far = !unsure && isfinite(est) && est > LZ_DUE * (tol < 1e-5 ? 1.0 : 0.5) * bound;
       if (far && !force) {
         if (tid == 0) {
           out[b * 4 + 0] = th32;

@@ -10,7 +10,6 @@ namespace dmrg {
 constexpr int LZ_THREADS = 256;   // threads of the vector kernels
 constexpr int LZ_EPT = 4;         // elements per thread
 constexpr int LZ_CHUNK = LZ_THREADS * LZ_EPT;
-constexpr int LZ_ROWS = 4;        // Krylov rows reduced together in k_multidot
 constexpr int LZ_TRI = 256;       // threads of the tridiagonal eigenproblem
 constexpr int LZ_DOT_EPT = 16;    // elements per thread in the reorthogonalisation dots
 constexpr int LZ_DOT_CHUNK = LZ_THREADS * LZ_DOT_EPT;
