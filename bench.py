@@ -189,13 +189,14 @@ GROWN_MIXED_TOL = 2e-4  # mixed Lanczos tolerance of the isometry-grown stand-in
 
 def recorded_traffic(name):
     """DRAM bytes per product from profiles/traffic.json, or None if the
-    kernel's sources changed since the capture."""
+    kernel's sources changed since the capture (or are others now)."""
+    from paper_0902_3185_gb300.prof import TRAFFIC_KERNELS, traffic_sources
     p = os.path.join(ROOT, "profiles", "traffic.json")
     if not os.path.exists(p):
         return None
     with open(p) as f:
         rec = json.load(f).get(name)
-    if not rec or source_sha(rec["sources"]) != rec["source_sha"]:
+    if not rec or name not in TRAFFIC_KERNELS or source_sha(traffic_sources(name)) != rec["source_sha"]:
         return None
     return rec["dram_bytes_per_product"]
 

@@ -34,19 +34,36 @@ if ROOT not in sys.path:
     sys.path.insert(0, ROOT)
 
 
-# kernel sources whose hash keys each traffic record (a change voids the record)
-TRAFFIC_SOURCES = {
-    "tensor_product_bf16x3": ["paper_0902_3185_gb300/csrc/matvec_tc.cu", "paper_0902_3185_gb300/csrc/tc_kernel.cuh"],
-    "tensor_product_tf32": ["paper_0902_3185_gb300/csrc/matvec_tc.cu", "paper_0902_3185_gb300/csrc/tc_kernel.cuh"],
-    "tensor_product_bf16x3_real": ["paper_0902_3185_gb300/csrc/matvec_tc.cu",
-                                   "paper_0902_3185_gb300/csrc/tc_kernel.cuh"],
-    "df64_product_real": ["paper_0902_3185_gb300/csrc/matvec_df.cu", "paper_0902_3185_gb300/csrc/df.cuh",
-                          "paper_0902_3185_gb300/csrc/tc_kernel.cuh"],
-    "fp64_product": ["paper_0902_3185_gb300/csrc/matvec_f64.cu"],
-    "gram_schmidt_pass_bf16x3_real": ["paper_0902_3185_gb300/csrc/lanczos.cu", "paper_0902_3185_gb300/csrc/lanczos.h",
-                                      "paper_0902_3185_gb300/csrc/df.cuh"],
-    "df64_product": ["paper_0902_3185_gb300/csrc/matvec_df.cu", "paper_0902_3185_gb300/csrc/tc_kernel.cuh"],
+# the source file of each traffic record's kernels
+CSRC = "paper_0902_3185_gb300/csrc/"
+TRAFFIC_KERNELS = {
+    "tensor_product_bf16x3": "matvec_tc.cu",
+    "tensor_product_tf32": "matvec_tc.cu",
+    "tensor_product_bf16x3_real": "matvec_tc.cu",
+    "df64_product": "matvec_df.cu",
+    "df64_product_real": "matvec_df.cu",
+    "fp64_product": "matvec_f64.cu",
+    "fp64_product_real": "matvec_f64.cu",
+    "gram_schmidt_pass_bf16x3_real": "lanczos.cu",
 }
+
+
+def traffic_sources(name):
+    """The sources whose hash keys a traffic record (a change voids it): the
+    kernels' file, its own header and every .cuh that they include, directly or
+    through another; the other headers hold host state and declarations."""
+    import re
+    out, todo = [], [TRAFFIC_KERNELS[name]]
+    while todo:
+        f = todo.pop(0)
+        if CSRC + f in out:
+            continue
+        out.append(CSRC + f)
+        with open(os.path.join(ROOT, CSRC, f)) as fh:
+            for inc in re.findall(r'^#include "([^"]+)"', fh.read(), re.M):
+                if inc.endswith(".cuh") or inc == TRAFFIC_KERNELS[name].replace(".cu", ".h"):
+                    todo.append(inc)
+    return sorted(out)
 
 
 def record_traffic(name, csv_path, note=""):
@@ -73,11 +90,12 @@ def record_traffic(name, csv_path, note=""):
                 total += float(d[k]) * scales[units[hdr.index(k)].lower()]
             launches += 1
     h = hashlib.sha256()
-    for f in TRAFFIC_SOURCES[name]:
+    sources = traffic_sources(name)
+    for f in sources:
         h.update(open(os.path.join(ROOT, f), "rb").read())
     out_path = os.path.join(ROOT, "profiles", "traffic.json")
     data = json.load(open(out_path)) if os.path.exists(out_path) else {}
-    data[name] = {"dram_bytes_per_product": total, "launches": launches, "sources": TRAFFIC_SOURCES[name],
+    data[name] = {"dram_bytes_per_product": total, "launches": launches, "sources": sources,
                   "source_sha": h.hexdigest()[:16], "capture": note}
     with open(out_path, "w") as f:
         json.dump(data, f, indent=1, sort_keys=True)
