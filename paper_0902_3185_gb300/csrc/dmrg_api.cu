@@ -739,7 +739,7 @@ void lz_enqueue_iteration(dmrg_sb* sb, int prec, cudaStream_t st) {
   const int ndot = lz_dot_nchunk(D);
   const bool pair = lz_pair(prec);  // the Krylov basis as double-float pairs (mixed-precision solves)
   lz_launch_dots_local(sb->lz_V, sb->lz_w, sb->lz_partial, ctl, D, B, cap, st, pair);
-  if (lz_short(D, B)) {
+  if (lz_short(D, B, pair)) {
     lz_launch_update_local(sb->lz_V, sb->lz_w, sb->lz_partial, hA, nA, ctl, D, B, cap, st, pair);
     lz_launch_multidot(sb->lz_V, sb->lz_w, sb->lz_partial, ctl, D, B, cap, 0, nullptr, st, nullptr, nullptr, pair);
     lz_launch_reduce_rows(sb->lz_partial, hB, ctl, lz_dot_nparts(D), cap, B, 0, nullptr, st);
@@ -1619,7 +1619,7 @@ dmrg_status dmrg_time_reorth(dmrg_sb* sb, int32_t prec, int32_t j, int32_t reps,
       lz_launch_multidot(sb->lz_V, sb->lz_w, sb->lz_partial, sb->lz_ctl, D, B, cap, 0, nullptr, st, nullptr, nullptr,
                          pair);
       lz_launch_reduce_rows(sb->lz_partial, hB, sb->lz_ctl, lz_dot_nparts(D), cap, B, 0, nullptr, st);
-      lz_launch_multiaxpy(sb->lz_V, sb->lz_w, hB, lz_short(D, B) ? nullptr : nB, sb->lz_ctl, D, B, cap, nch, 0, nullptr,
+      lz_launch_multiaxpy(sb->lz_V, sb->lz_w, hB, lz_short(D, B, pair) ? nullptr : nB, sb->lz_ctl, D, B, cap, nch, 0, nullptr,
                           st, pair);
     };
     pass();

@@ -1234,9 +1234,9 @@ void lz_launch_cfrac(const double* norm2, const double* alpha, const double* bet
 // blocks of a dot pass: LZ_DOT_WARPS warps each (one row of blocks), or for a
 // short vector single warps with the row groups (rg rows) over z, up to about
 // 16 warps per SM
-static void dot_grid(int64_t D, int batch, int cap, int rg, dim3& g, int& threads) {
+static void dot_grid(int64_t D, int batch, int cap, int rg, bool pair, dim3& g, int& threads) {
   const int nch = lz_dot_nchunk(D);
-  if (!lz_short(D, batch)) {
+  if (!lz_short(D, batch, pair)) {
     g = dim3(nch, batch);
     threads = LZ_THREADS;
     return;
@@ -1254,7 +1254,7 @@ void lz_launch_multidot(const double* V, double* w, double* partial, const int32
   const bool fine = !h_pre && !pair && (int64_t)nch * LZ_DOT_WARPS * batch * 32 <= 152 * 16;
   dim3 g(nch, batch);
   int threads = LZ_THREADS;
-  if (!h_pre) dot_grid(D, batch, cap, fine ? 2 : 8, g, threads);
+  if (!h_pre) dot_grid(D, batch, cap, fine ? 2 : 8, pair, g, threads);
   if (pair)
     k_multidot<true, 8><<<g, threads, 0, st>>>(V, w, partial, ctl, D, batch, cap, nch, win, gate, h_pre, npart_pre);
   else if (fine)
@@ -1266,7 +1266,7 @@ void lz_launch_dots_local(const double* V, const double* w, double* partial, con
                           int batch, int cap, cudaStream_t st, bool pair) {
   dim3 g;
   int threads;
-  dot_grid(D, batch, 1, 8, g, threads);
+  dot_grid(D, batch, 1, 8, pair, g, threads);
   if (pair)
     k_dots_local<true><<<g, threads, 0, st>>>(V, w, partial, ctl, D, batch, cap, lz_dot_nchunk(D));
   else

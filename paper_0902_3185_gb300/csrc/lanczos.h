@@ -42,9 +42,14 @@ inline int lz_dot_nparts(int64_t D) { return lz_dot_nchunk(D) * LZ_DOT_WARPS; }
 // use blocks of one or two warps, and pass A's update and pass B's norms
 // kernels of their own.  All of a step's passes, before -> after: 32-site
 // chain at m = 200 (4 chunks) 80 -> 31 us, ladder at m = 400 (28 chunks, 4
-// members) 134 -> 53 us, chain at m = 1000 in pairs (77 chunks) 64 -> 61 us; the
-// m = 1000 ladder (656 chunks) keeps the update inside the sweep.
-inline bool lz_short(int64_t D, int batch) { return (int64_t)lz_dot_nchunk(D) * batch < 2 * 152; }
+// members) 134 -> 53 us.  The pair basis, whose passes are bound by instructions
+// where float64's wait for their unit, gives it up sooner: 60 mixed Lanczos
+// steps, usual / short blocks, with 69 chunks 11.2 / 9.9 ms, 77 10.4 / 9.7, 82 12.1 /
+// 11.7, 127 15.5 / 15.8, 162 14.5 / 16.2, 217 17.0 / 18.8, 246 20.1 / 22.5 (float64 up to 246
+// the same or 5 % in favour of short ones).
+inline bool lz_short(int64_t D, int batch, bool pair) {
+  return (int64_t)lz_dot_nchunk(D) * batch < (pair ? 100 : 2 * 152);
+}
 
 // Gram-Schmidt passes over the Krylov rows first_row(j, win)..j (win = 0: all
 // rows); members with gate != NULL and gate[b] == 0 are skipped.
