@@ -37,8 +37,9 @@
 // the mean work of an SM.  The tiles are dealt to the blocks by their modelled
 // length, and the longest ones split along N first.  Measured against a
 // round-robin deal of the sorted, unsplit tiles: 64 sectors 16..512 wide
-// 363 -> 328 us, 16 such sectors 173 -> 161 us, the m = 1000 chain 57 -> 52 us, the
-// m = 1000 ladder (16 members) 191 -> 186 us, the m = 400 ladder 61 -> 56 us.
+// 362 -> 320 us, 16 such sectors 160 -> 152 us, the m = 1000 chain 58 -> 52 us, the
+// m = 1000 ladder (16 members) 190 -> 187 us, the m = 400 ladder 60 -> 56 us, a real
+// m = 1000 superblock with one member 107 -> 103 us, with 16 647 -> 643 us.
 //
 // Eight draining warps rather than twelve: the block then gets 168 registers
 // a thread without spills (at 448 threads the cap of 128 spilled inside the
@@ -1250,17 +1251,21 @@ static int64_t build_set(const dmrg_sb* sb, int prec, const std::vector<EPair>& 
     std::vector<TcTile> t;
     t.reserve(B.tiles.size());
     std::vector<int32_t> begin;
-    // A launch lasts at least as long as its longest tile: tiles above 1.3
+    // A launch lasts at least as long as its longest tile: tiles above 1.6
     // times the mean work of an SM are split along N, down to 32 columns.  Each
-    // part repeats the L copies: splits down to the mean, or to 0.7 of it, cost
-    // wide sectors more than the balance gave (16 sectors 16..512 wide: 163 us,
-    // against 175 and 192).  An element's sum keeps its order in any width.
+    // part repeats the L copies.  Products with unsplit tiles / split above 2.0 /
+    // 1.6 / 1.3 times the mean, in us, split BF16: real m = 1000 superblock with 1, 2
+    // members 106 / 103 / 102 / 108, 134 / 134 / 135 / 145, 32-site chain at m = 1000 60 / 55 /
+    // 53 / 53, 16 sectors 16..512 wide 156 / 152 / 152 / 153, with 4 members 250 / 250 / 250 /
+    // 256, 64 sectors 319 / 319 / 319 / 318; TF32, the same: 127 / 118 / 112 / 114, 160 / 148 /
+    // 149 / 170, 68 / 58 / 55 / 55, 179 / 162 / 159 / 159, 241 / 236 / 235 / 225, 310 / 307 / 304 /
+    // 297.  An element's sum keeps its order in any width.
     std::vector<TcTile> all;
     std::vector<int64_t> weight;
     if (tune.heavy_first) {
       int64_t sum = 0;
       for (int64_t w : B.weight) sum += w;
-      const int64_t most = std::max<int64_t>(sum / n_sms * 13 / 10, 1);
+      const int64_t most = std::max<int64_t>(sum / n_sms * 16 / 10, 1);
       for (size_t i = 0; i < B.tiles.size(); ++i) {
         const TcTile& u = B.tiles[i];
         const int parts = (int)std::min<int64_t>(cdiv(B.weight[i], most), u.ntile / 32);
@@ -1304,7 +1309,7 @@ static int64_t build_set(const dmrg_sb* sb, int prec, const std::vector<EPair>& 
         for (size_t i : l) t.push_back(all[i]);
       }
       begin.push_back((int32_t)t.size());
-      L.cta_begin = up(begin);
+      if (t.size() > G) L.cta_begin = up(begin);  // else one tile per block: no table to read first
     } else {
       t = B.tiles;
     }
