@@ -610,7 +610,9 @@ bool launch_eig_cluster(std::vector<EigJob> jobs, cudaStream_t st) {
   if (jobs.empty()) return true;
   if (g_cluster_ok == 0) return false;
   std::stable_sort(jobs.begin(), jobs.end(), [](const EigJob& x, const EigJob& y) { return x.n > y.n; });
-  const int C = eig_cluster_blocks(jobs[0].n);
+  std::vector<int> sizes;
+  for (const EigJob& j : jobs) sizes.push_back(j.n);
+  const int C = eig_cluster_blocks(sizes);
   size_t smem = 0;
   for (const EigJob& j : jobs) smem = std::max(smem, eig_cluster_smem(j.n, C));
   smem = (smem + 15) & ~(size_t)15;

@@ -49,9 +49,22 @@ struct EigJob {
 };
 constexpr int EIG_SMEM_MAX_N = 110;  // A and V in shared memory up to this size
 constexpr int EIG_CLUSTER = 16;      // blocks of a cluster, at most
-// Blocks per cluster for matrices up to n: the float64 work of a round, 3 n^2
-// cycles of one SM, against the cluster's barriers.
-inline int eig_cluster_blocks(int n) { return n > 64 ? EIG_CLUSTER : 8; }
+// Blocks per cluster for a list of matrices: the float64 work of a round, 3 n^2
+// cycles of one SM, against the cluster's barriers; and half as many where the
+// list is long enough (twenty of the widest's work) that clusters take turns
+// and two of 8 fit where one of 16 does.  16 / 8 blocks, ms: 24 matrices of n =
+// 130 16.9 / 15.2, of 200 52 / 42; 50 of 111 27 / 12, of 160 39 / 30, of 200 88 / 83; 100 of
+// 130 51 / 40, of 200 160 / 125; but 10 of 130 11.2 / 11.9, of 200 26 / 29, and 50 of 250 148 /
+// 180 (one block of 8's shared memory fills an SM from about 210 on).
+inline int eig_cluster_blocks(const std::vector<int>& sizes) {
+  int n = 0;
+  for (int s : sizes) n = s > n ? s : n;
+  if (n <= 64) return 8;
+  if (n <= EIG_SMEM_MAX_N || n > 208) return EIG_CLUSTER;
+  double work = 0.0;
+  for (int s : sizes) work += (double)s * s * s;
+  return work >= 20.0 * n * n * n ? 8 : EIG_CLUSTER;
+}
 // Whether matrices of these sizes (up to EIG_SMEM_MAX_N) are faster one per
 // cluster, or one per block.  One block takes longer for a wide matrix, but
 // hundreds of them run side by side; clusters take turns.  Modelled times (ms)
@@ -68,7 +81,7 @@ inline bool eig_clusters_pay(const std::vector<int>& sizes) {
   int n = 0;
   for (int s : sizes) n = s > n ? s : n;
   if (n <= 32) return false;
-  const bool wide = eig_cluster_blocks(n) == EIG_CLUSTER;
+  const bool wide = eig_cluster_blocks(sizes) == EIG_CLUSTER;
   const double block = 0.026 * n + 1.56e-5 * n * n * n;                       // the widest, alone in its block
   const double cluster = wide ? 0.0346 * n + 1.7e-4 * n * n : 0.0415 * n;     // alone in its cluster
   double share = 0.0;  // the clusters' time when they keep the device busy

@@ -18,6 +18,14 @@ MEASURED = [(33, 24, 1.60, 1.70), (33, 150, 2.16, 4.93), (33, 600, 5.31, 15.4), 
             (80, 1, 9.33, 3.75), (80, 24, 10.1, 5.95), (80, 60, 10.2, 11.4), (80, 150, 10.6, 26.9), (80, 600, 35.7, 101.3),
             (110, 1, 23.6, 5.86), (110, 24, 24.2, 10.1), (110, 150, 24.8, 45.5)]
 
+# (size, count, measured with clusters of 16 blocks, of 8)
+CLUSTERS = [(111, 10, 7.33, 7.62), (111, 50, 27.3, 12.3), (111, 100, 33.0, 23.3), (130, 1, 8.74, 11.7),
+            (130, 10, 11.2, 11.9), (130, 24, 16.9, 15.2), (130, 50, 28.3, 21.2), (130, 100, 51.0, 40.4),
+            (160, 10, 14.9, 16.2), (160, 24, 21.8, 21.5), (160, 50, 38.6, 30.1), (160, 150, 102.6, 89.1),
+            (200, 1, 19.6, 28.9), (200, 10, 25.8, 29.5), (200, 24, 52.3, 42.1), (200, 50, 88.4, 83.3),
+            (200, 100, 159.6, 125.1), (250, 1, 28.6, 45.6), (250, 24, 75.1, 91.0), (250, 50, 148.4, 179.8),
+            (300, 24, 128.4, 151.1)]
+
 
 def test_the_faster_side_is_taken(tmp_path):
     cxx = shutil.which("g++")
@@ -32,10 +40,13 @@ def test_the_faster_side_is_taken(tmp_path):
         '  for (auto& x : c) printf("%d ", (int)dmrg::eig_clusters_pay(std::vector<int>(x[1], x[0])));\n'
         "  std::vector<int> v(400, 9);  // many small ones beside a wide one\n"
         '  v.push_back(36); printf("%d ", (int)dmrg::eig_clusters_pay(v));\n'
-        '  printf("%d\\n", (int)dmrg::eig_clusters_pay({}));\n'
+        '  printf("%d ", (int)dmrg::eig_clusters_pay({}));\n'
+        "  const int w[][2] = {" + ", ".join("{%d, %d}" % m[:2] for m in CLUSTERS) + "};\n"
+        '  for (auto& x : w) printf("%d ", dmrg::eig_cluster_blocks(std::vector<int>(x[1], x[0])));\n'
         "}\n")
     exe = str(tmp_path / "route")
     subprocess.run([cxx, "-std=c++17", "-I" + build.CSRC, "-I" + include, str(tmp_path / "route.cpp"), "-o", exe],
                    check=True)
     got = subprocess.run([exe], capture_output=True, text=True, timeout=60).stdout.split()
-    assert got == [str(int(c < b)) for _, _, b, c in MEASURED] + ["0", "0"]
+    assert got[:len(MEASURED) + 2] == [str(int(c < b)) for _, _, b, c in MEASURED] + ["0", "0"]
+    assert got[len(MEASURED) + 2:] == ["8" if e < s else "16" for _, _, s, e in CLUSTERS]
