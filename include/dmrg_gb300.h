@@ -141,6 +141,10 @@ dmrg_status dmrg_query(const dmrg_sb* sb, dmrg_sb_info* info);
  * succeeds.  Work on other streams that reads this superblock must be
  * ordered before the call by the caller. */
 dmrg_status dmrg_set_coeffs(dmrg_sb* sb, const double* coeffs, void* stream);
+/* 1 if `coeffs` (host, [batch][n_terms]) is, bit for bit, the table that the
+ * superblock was created with or that the last dmrg_set_coeffs set and waited
+ * for; 0 otherwise (also after a call that failed).  Touches no stream. */
+int32_t dmrg_has_coeffs(const dmrg_sb* sb, const double* coeffs);
 
 /* Sec. 3.3 x += H y: y = H psi (accumulate = 0) or y += H psi (accumulate =
  * 1) for every batch member.  psi, y: device [batch][D], must not overlap. */

@@ -30,7 +30,7 @@ SYMBOLS = ["dmrg_create_superblock", "dmrg_destroy_superblock", "dmrg_last_error
            "dmrg_test_inject", "dmrg_lanczos_ground_grad", "dmrg_apply_H_term_dots", "dmrg_lanczos_coeffs",
            "dmrg_continued_fraction", "dmrg_sys_create", "dmrg_sys_destroy", "dmrg_sys_last_error",
            "dmrg_sys_infinite", "dmrg_sys_sweeps", "dmrg_sys_last_superblock", "dmrg_sym_eig_batched",
-           "dmrg_time_reorth"]
+           "dmrg_time_reorth", "dmrg_has_coeffs"]
 
 
 class DmrgError(RuntimeError):
@@ -135,6 +135,8 @@ def load(build_if_missing: bool = True):
     lib.dmrg_query.argtypes = [vp, C.POINTER(_Info)]
     lib.dmrg_set_coeffs.argtypes = [vp, dp, vp]
     lib.dmrg_apply_H.argtypes = [vp, dp, dp, i32, i32, vp]
+    lib.dmrg_has_coeffs.argtypes = [vp, dp]
+    lib.dmrg_has_coeffs.restype = i32
     lib.dmrg_apply_H_backward.argtypes = [vp, dp, dp, dp, dp, i32, vp]
     lib.dmrg_lanczos_ground.argtypes = [vp, dp, dp, dp, C.POINTER(LanczosOpts), C.POINTER(LanczosInfo), vp]
     lib.dmrg_energy_grad.argtypes = [vp, dp, dp, i32, vp]
@@ -242,6 +244,11 @@ class GpuSuperblock:
         c = np.ascontiguousarray(np.broadcast_to(np.asarray(coeffs, dtype=np.float64),
                                                  (self.batch, self.n_terms)))
         self._check(self.lib.dmrg_set_coeffs(self.h, c.ctypes.data, _stream(stream)))
+
+    def has_coeffs(self, coeffs):
+        """Whether this table ([batch, n_terms] numpy float64) is the one that is set."""
+        c = np.ascontiguousarray(coeffs, dtype=np.float64)
+        return c.shape == (self.batch, self.n_terms) and bool(self.lib.dmrg_has_coeffs(self.h, c.ctypes.data))
 
     def apply_H(self, psi, y=None, accumulate=False, prec="fp64", stream=None):
         if y is None:
@@ -368,7 +375,8 @@ class ApplyH(torch.autograd.Function):
     @staticmethod
     def forward(ctx, psi, coeffs, gsb: GpuSuperblock, prec="fp64"):
         c = coeffs.detach().cpu().numpy().copy()
-        gsb.set_coeffs(c)
+        if not gsb.has_coeffs(c):  # setting a table waits for the stream
+            gsb.set_coeffs(c)
         ctx.gsb = gsb
         ctx.prec = prec
         ctx.coeffs = c  # the library holds one coefficient table: restore it for backward
@@ -379,7 +387,8 @@ class ApplyH(torch.autograd.Function):
     def backward(ctx, g):
         (psi,) = ctx.saved_tensors
         need_psi, need_c = ctx.needs_input_grad[0], ctx.needs_input_grad[1]
-        ctx.gsb.set_coeffs(ctx.coeffs)
+        if not ctx.gsb.has_coeffs(ctx.coeffs):
+            ctx.gsb.set_coeffs(ctx.coeffs)
         dpsi, dc = ctx.gsb.apply_H_backward(psi, g.contiguous(), want_dpsi=need_psi, want_dc=need_c,
                                             prec=ctx.prec)
         return dpsi, dc, None, None

@@ -1310,13 +1310,18 @@ dmrg_status dmrg_query(const dmrg_sb* sb, dmrg_sb_info* info) {
   return DMRG_OK;
 }
 
+int32_t dmrg_has_coeffs(const dmrg_sb* sb, const double* coeffs) {
+  return sb && coeffs && sb->coeffs_set &&
+         memcmp(sb->coeffs.data(), coeffs, sb->coeffs.size() * sizeof(double)) == 0;
+}
+
 dmrg_status dmrg_set_coeffs(dmrg_sb* sb, const double* coeffs, void* stream) {
   if (!sb || !coeffs) return DMRG_EINVAL;
   return guard(sb, [&] {
     cudaStream_t st = (cudaStream_t)stream;
     const size_t n = (size_t)sb->batch * sb->n_terms;
     // the table that is set already, by a call that went through: nothing to write
-    if (sb->coeffs_set && memcmp(sb->coeffs.data(), coeffs, n * sizeof(double)) == 0) {
+    if (dmrg_has_coeffs(sb, coeffs)) {
       CK(cudaStreamSynchronize(st));
       return DMRG_OK;
     }
