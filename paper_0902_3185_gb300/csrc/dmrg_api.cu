@@ -244,7 +244,7 @@ TileF64 out_tile(int32_t buf, int64_t off, int64_t bs, int32_t ldc, int32_t M, i
 // output list, more in the intermediates': 279 / 285 us; 355 wide ones 413 /
 // 423 us), double-float 5 to 9 % in favour of 16.
 constexpr int64_t SEG_FEW_TILES = 152 * 6;
-// From this many 24 x 24 tiles (all members; three rounds of eight blocks per
+// From this many 24 x 24 tiles (all members; three waves of eight blocks per
 // SM) a list may use tiles up to 24 wide, if that saves at least a third of the
 // tiles (outputs wide enough to fill them).  An operand element is copied and
 // scaled once for 24 outputs instead of 16 or 8.  Both lists of a product 16
